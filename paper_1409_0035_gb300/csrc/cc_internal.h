@@ -54,10 +54,15 @@ enum : uint32_t {
 
 // Per-level statistics, indexed by level mod 4 (written during level l,
 // read during l+1 and l+2, cleared during l+3).
-struct LevelCtl {
+struct alignas(8) LevelCtl {
+    // Pairs that a CTA adds to with one 64-bit atomic each (every total is
+    // below 2^31, so nothing carries into the upper half).
     unsigned int qlen;          // nodes with new bits this level (queue length)
-    unsigned int tlen;          // touched nodes (top-down)
     unsigned int ninc_dec;      // nodes that became complete this level
+    unsigned int ef;            // sum of degrees of the frontier nodes
+    unsigned int eu_dec;        // sum of degrees of nodes completed
+    unsigned int hinc;          // heavy nodes left incomplete (bottom-up)
+    unsigned int tlen;          // touched nodes (top-down)
     unsigned int alen;          // rebuilt light list length (bottom-up)
     unsigned int qcnt;          // frontier queue built from the stamps (top-down)
     unsigned int mlen;          // rebuilt medium list length (bottom-up)
@@ -65,8 +70,6 @@ struct LevelCtl {
     unsigned int hclen;         // rebuilt heavy chunk list length (bottom-up)
     unsigned int tlen2;         // rebuilt tiny list length (bottom-up)
     unsigned int hnext;         // next heavy chunk task to take (bottom-up)
-    unsigned long long ef;      // sum of degrees of the frontier nodes
-    unsigned long long eu_dec;  // sum of degrees of nodes completed
 };
 
 constexpr int kTraceLevels = 64;

@@ -289,16 +289,15 @@ __device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, bool valid,
     }
 }
 
-// The words gathered on level l (the pass total and the level's trace).
-__device__ __forceinline__ void flush_words(Ctl *ctl, int l, unsigned words)
+// Number of W-lane groups with a bit set in the ballot b.
+template <int W>
+__device__ __forceinline__ unsigned groups_of(unsigned b)
 {
-    unsigned long long x = words;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-    if ((threadIdx.x & 31) == 0 && x) {
-        atomicAdd(&ctl->words, x);
-        if (l < kTraceLevels) atomicAdd(&ctl->lvl_words[l], x);
-    }
+    for (int o = 1; o < W; o <<= 1) b |= b >> o;
+    constexpr unsigned M = W == 1 ? 0xFFFFFFFFu : W == 2 ? 0x55555555u : W == 4 ? 0x11111111u
+                         : W == 8 ? 0x01010101u : W == 16 ? 0x00010001u : 1u;
+    return __popc(b & M);
 }
 
 // OR of `x` over the lanes holding the same word slot (lane % W).
@@ -400,13 +399,19 @@ __device__ __forceinline__ uint64_t gather_scan(const int32_t *__restrict__ col,
     return acc;
 }
 
-// Flush per-lane counters of one level phase to the level control block and
-// (when asked) the CTA histogram to the global histogram of level l.
-__device__ void flush_level(const BfsJob &J, int l, LevelCtl *C, LaneAcc &A,
+// Flush per-lane counters of one level to the level control block and
+// (when asked) the CTA histogram to the global histogram of level l.  hinc:
+// the lane's heavy nodes left incomplete.  What bounds a short level is the
+// same-address atomics ahead of the barrier (608 CTAs on one line), so the
+// counters go out as packed pairs, one atomic per CTA each, and the gathered
+// words (the pass total and the level's trace) are reduced with them, where
+// every warp had added its own.
+__device__ void flush_level(const BfsJob &J, int l, LevelCtl *C, LaneAcc &A, unsigned hinc,
                             unsigned *s_hist, bool flush_hist)
 {
     __shared__ unsigned long long s_red[4][kBlock / 32];
-    unsigned long long x[4] = {A.ef, A.eu_dec, A.ninc_dec, A.nfront};
+    unsigned long long x[4] = {A.nfront | ((unsigned long long)A.ninc_dec << 32),
+                               A.ef | ((unsigned long long)A.eu_dec << 32), A.words, hinc};
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -419,12 +424,16 @@ __device__ void flush_level(const BfsJob &J, int l, LevelCtl *C, LaneAcc &A,
         unsigned long long t = 0;
         for (int i = 0; i < kBlock / 32; ++i) t += s_red[threadIdx.x][i];
         if (t) {
-            if (threadIdx.x == 0) atomicAdd(&C->ef, t);
-            if (threadIdx.x == 1) atomicAdd(&C->eu_dec, t);
-            if (threadIdx.x == 2) atomicAdd(&C->ninc_dec, (unsigned)t);
-            if (threadIdx.x == 3) atomicAdd(&C->qlen, (unsigned)t);
+            if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long *>(&C->qlen), t);
+            if (threadIdx.x == 1) atomicAdd(reinterpret_cast<unsigned long long *>(&C->ef), t);
+            if (threadIdx.x == 2) {
+                atomicAdd(&J.ctl->words, t);
+                if (l < kTraceLevels) atomicAdd(&J.ctl->lvl_words[l], t);
+            }
+            if (threadIdx.x == 3) atomicAdd(&C->hinc, (unsigned)t);
         }
     }
+    A.words = 0;
     A.ef = A.eu_dec = 0;
     A.ninc_dec = A.nfront = 0;
     if (!flush_hist) return;
@@ -714,7 +723,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
         if (J.red & RED_LEVELS) J.dist_out[(int64_t)v * J.dist_ld + i] = 0u;
         if (J.red & RED_PIVOT) { J.pivot[v] = (int)i; J.delta[v] = 0; }
         if (J.red & RED_DCC) J.dcc[i * J.dcc_k + J.sidx[v]] = 0;
-        const unsigned long long d = (unsigned long long)(rp[v + 1] - rp[v]);
+        const unsigned d = (unsigned)(rp[v + 1] - rp[v]);
         atomicAdd(&ctl->lev[0].ef, d);
         if (J.k == 1) {
             atomicAdd(&ctl->lev[0].eu_dec, d);
@@ -776,7 +785,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
         }
         if (gtid == 0) {
             LevelCtl *Z = &ctl->lev[(l + 1) & 3];
-            Z->qlen = 0; Z->tlen = 0; Z->ninc_dec = 0; Z->ef = 0; Z->eu_dec = 0;
+            Z->qlen = 0; Z->tlen = 0; Z->ninc_dec = 0; Z->ef = 0; Z->eu_dec = 0; Z->hinc = 0;
             Z->alen = 0; Z->qcnt = 0; Z->mlen = 0; Z->hlen = 0; Z->hclen = 0; Z->tlen2 = 0;
             Z->hnext = 0;
         }
@@ -898,26 +907,30 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                 }
                 tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, deg, Fout, A, s_hist, true);
             }
-            flush_words(ctl, l, A.words);
-            A.words = 0;
-            flush_level(J, l, C, A, s_hist, doHist);
+            flush_level(J, l, C, A, 0u, s_hist, doHist);
             if (!sync_after(CC_PH_TD_FINAL)) return;
             if (gtid == 0) ctl->td_levels += 1;
             prev_td = true;
             prevT = Tout;
         } else {
-            // Rebuild the light list when fewer than half of it can still be
-            // incomplete (ninc bounds the incomplete light nodes).
-            // ninc bounds the incomplete nodes of every class; the medium and
-            // heavy lists are rebuilt with the light list (heavy nodes complete
-            // early) or on their own bound.
-            // The tiny and light lists are rebuilt together, once fewer than
-            // half of their entries can still be incomplete.
-            const bool rb_tl = 2 * ninc < s_al.nL + s_al.nT;
+            // Lists are compacted to the incomplete nodes (ninc bounds them in
+            // every class) once fewer than half of their entries can still be
+            // incomplete, the tiny and light lists together -- but only while
+            // a list is longer than two steps of every warp: below that a
+            // rebuild (its dependent loads, a waited atomic and a barrier)
+            // costs more than the entries it drops.
+            const int64_t short_tl = 2 * nwarps * NPW, short_m = 2 * nwarps;
+            const bool rb_tl = s_al.nL + s_al.nT > short_tl && 2 * ninc < s_al.nL + s_al.nT;
             const bool rb_t = rb_tl && s_al.nT > 0;
             const bool rb_l = rb_tl && s_al.nL > 0;
-            const bool rb_m = s_al.nM > 0 && (rb_l || 2 * ninc < s_al.nM);
-            const bool rb_h = s_al.nH > 0 && (rb_l || 2 * ninc < s_al.nH);
+            const bool rb_m = s_al.nM > short_m && 2 * ninc < s_al.nM;
+            // Heavy nodes complete early: the last bottom-up level counted
+            // those it left incomplete, and once none is, their phases and
+            // the barrier between them are skipped.
+            const int64_t hleft = prev_td ? s_al.nH : (int64_t)P->hinc;
+            const bool heavy = s_al.nH > 0 && hleft > 0;
+            const bool rb_h = heavy && s_al.nHC > short_m &&
+                              2 * (hleft < ninc ? hleft : ninc) < s_al.nH;
             if (rb_t || rb_l || rb_m || rb_h) {
                 auto incomplete = [&](int64_t v) {
                     bool inc = false;
@@ -1086,72 +1099,75 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
             // prefetches its lines to the L2 (wider variants), so that a
             // step waits only for its frontier gathers (headline traversal:
             // prefetch 0.831 -> 0.803 ms, staging instead 0.779 -> 0.763).
-            const int32_t *const HCcur = s_al.HC;
-            const int64_t hc_len = s_al.nHC;
-            auto heavy_task = [&](int64_t t) {
-                const int32_t ti = HCcur ? HCcur[t] : (int32_t)t;
-                const int v = J.Hch_node[ti];
-                const int64_t vw = (int64_t)v * W + w;
-                const int64_t b = J.Hch_begin[ti];
-                const int64_t e = min(b + (int64_t)kChunk, prp[v + 1]);
-                const uint64_t visw = J.vis[vw];
-                const uint64_t cur = J.nxt[vw];
-                if (__all_sync(FULL, (visw | cur) == ~0ull)) return;
-                auto done = [&](uint64_t a) {
-                    return __all_sync(FULL, (or_same_word<W>(a) | visw | cur) == ~0ull);
+            unsigned hinc = 0;
+            if (heavy) {
+                const int32_t *const HCcur = s_al.HC;
+                const int64_t hc_len = s_al.nHC;
+                auto heavy_task = [&](int64_t t) {
+                    const int32_t ti = HCcur ? HCcur[t] : (int32_t)t;
+                    const int v = J.Hch_node[ti];
+                    const int64_t vw = (int64_t)v * W + w;
+                    const int64_t b = J.Hch_begin[ti];
+                    const int64_t e = min(b + (int64_t)kChunk, prp[v + 1]);
+                    const uint64_t visw = J.vis[vw];
+                    const uint64_t cur = J.nxt[vw];
+                    if (__all_sync(FULL, (visw | cur) == ~0ull)) return;
+                    auto done = [&](uint64_t a) {
+                        return __all_sync(FULL, (or_same_word<W>(a) | visw | cur) == ~0ull);
+                    };
+                    uint64_t acc;
+                    if constexpr (kStageHub) {
+                        const int32_t *srow = stage_cols(s_buf + (threadIdx.x >> 5) * kHubSlots,
+                                                         pcol, J.arcs, b, e, lane);
+                        acc = gather_scan<W, kUnrollH, true>(srow, Fin, 0, grp, e - b, NPW, w,
+                                                             A.words, chk, done);
+                    } else {
+                        if (lane <= kChunk / 32) prefetch_l2(pcol + min(b + 32 * lane, e - 1));
+                        acc = gather_scan<W, kUnrollH>(pcol, Fin, b, grp, e, NPW, w, A.words, chk,
+                                                       done);
+                    }
+                    const uint64_t nbits = or_same_word<W>(acc) & ~visw & ~cur;
+                    if (lane < W && nbits) atomicOr((unsigned long long *)&J.nxt[vw], nbits);
                 };
-                uint64_t acc;
-                if constexpr (kStageHub) {
-                    const int32_t *srow = stage_cols(s_buf + (threadIdx.x >> 5) * kHubSlots,
-                                                     pcol, J.arcs, b, e, lane);
-                    acc = gather_scan<W, kUnrollH, true>(srow, Fin, 0, grp, e - b, NPW, w,
-                                                         A.words, chk, done);
+                if (hc_len > 2 * nwarps) {
+                    // Many tasks: the warps take them from a counter, kGrab at a
+                    // time, so that warps done early with the other classes take
+                    // more of them (dealt in turn, the level waits for the warp
+                    // with the most work; 0.803 -> 0.789 ms).
+                    for (;;) {
+                        unsigned tb = 0;
+                        if (lane == 0) tb = atomicAdd(&C->hnext, (unsigned)kGrab);
+                        tb = __shfl_sync(FULL, tb, 0);
+                        if ((int64_t)tb >= hc_len) break;
+                        const int64_t tend = min((int64_t)tb + kGrab, hc_len);
+                        for (int64_t t = tb; t < tend; ++t) heavy_task(t);
+                    }
                 } else {
-                    if (lane <= kChunk / 32) prefetch_l2(pcol + min(b + 32 * lane, e - 1));
-                    acc = gather_scan<W, kUnrollH>(pcol, Fin, b, grp, e, NPW, w, A.words, chk,
-                                                   done);
+                    for (int64_t t = gwarp; t < hc_len; t += nwarps) heavy_task(t);
                 }
-                const uint64_t nbits = or_same_word<W>(acc) & ~visw & ~cur;
-                if (lane < W && nbits) atomicOr((unsigned long long *)&J.nxt[vw], nbits);
-            };
-            if (hc_len > 2 * nwarps) {
-                // Many tasks: the warps take them from a counter, kGrab at a
-                // time, so that warps done early with the other classes take
-                // more of them (dealt in turn, the level waits for the warp
-                // with the most work; 0.803 -> 0.789 ms).
-                for (;;) {
-                    unsigned tb = 0;
-                    if (lane == 0) tb = atomicAdd(&C->hnext, (unsigned)kGrab);
-                    tb = __shfl_sync(FULL, tb, 0);
-                    if ((int64_t)tb >= hc_len) break;
-                    const int64_t tend = min((int64_t)tb + kGrab, hc_len);
-                    for (int64_t t = tb; t < tend; ++t) heavy_task(t);
+                if (!sync_after(CC_PH_BU_HEAVY)) return;
+                // B: finalise the heavy nodes.
+                const int32_t *const HLcur = s_al.H;
+                const int64_t hl_len = s_al.nH;
+                for (int64_t t = gwarp; t * NPW < hl_len; t += nwarps) {
+                    const int64_t li = t * NPW + grp;
+                    const bool valid = li < hl_len;
+                    const int v = valid ? HLcur[li] : 0;
+                    const int64_t vw = (int64_t)v * W + w;
+                    uint64_t vis = ~0ull, acc = 0;
+                    int64_t deg = 0;
+                    if (valid) {
+                        vis = J.vis[vw];
+                        acc = J.nxt[vw];
+                        if (acc) J.nxt[vw] = 0;
+                        deg = prp[v + 1] - prp[v];
+                    }
+                    tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, deg, Fout, A, s_hist, false);
+                    const unsigned left = __ballot_sync(FULL, (vis | acc) != ~0ull);
+                    if (lane == 0) hinc += groups_of<W>(left);
                 }
-            } else {
-                for (int64_t t = gwarp; t < hc_len; t += nwarps) heavy_task(t);
             }
-            if (!sync_after(CC_PH_BU_HEAVY)) return;
-            // B: finalise the heavy nodes.
-            const int32_t *const HLcur = s_al.H;
-            const int64_t hl_len = s_al.nH;
-            for (int64_t t = gwarp; t * NPW < hl_len; t += nwarps) {
-                const int64_t li = t * NPW + grp;
-                const bool valid = li < hl_len;
-                const int v = valid ? HLcur[li] : 0;
-                const int64_t vw = (int64_t)v * W + w;
-                uint64_t vis = ~0ull, acc = 0;
-                int64_t deg = 0;
-                if (valid) {
-                    vis = J.vis[vw];
-                    acc = J.nxt[vw];
-                    if (acc) J.nxt[vw] = 0;
-                    deg = prp[v + 1] - prp[v];
-                }
-                tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, deg, Fout, A, s_hist, false);
-            }
-            flush_words(ctl, l, A.words);
-            A.words = 0;
-            flush_level(J, l, C, A, s_hist, doHist);
+            flush_level(J, l, C, A, hinc, s_hist, doHist);
             if (!sync_after(CC_PH_BU_FINAL)) return;
             if (gtid == 0) ctl->bu_levels += 1;
             prev_td = false;
