@@ -92,145 +92,162 @@ struct LaneAcc {
 };
 
 // Update, reduce and enqueue one warp tile.  Lanes form groups of W; group
-// g = lane / W is one node (valid or not), lane % W its word.  Must be
-// called by all 32 lanes together.
+// g = lane / W is one node (valid or not: an invalid lane passes nw = 0),
+// lane % W its word.  Must be called by all 32 lanes together.
+//
+// Bound by instructions issued on dense levels and by its chain of dependent
+// accesses on sparse ones, so: a tile in which nothing arrived leaves at
+// once; flags over a node's words come from ballots, not shuffle trees; the
+// per-node loads (sample index, Delta, band flag) are issued together up
+// front; and the sums leave as reductions without a return value, which no
+// later instruction waits for.
 template <int W>
-__device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, bool valid,
-                                            int v, uint64_t vis, uint64_t nw,
-                                            int64_t deg, uint64_t *Fout,
-                                            LaneAcc &A, unsigned *s_hist,
-                                            bool clear_tflag)
+__device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, int v, uint64_t vis,
+                                            uint64_t nw, int64_t deg, uint64_t *Fout,
+                                            LaneAcc &A, unsigned *s_hist)
 {
+    const unsigned bn = __ballot_sync(FULL, nw != 0ull);
+    if (bn == 0u) return;
     const int lane = threadIdx.x & 31;
     const int w = lane & (W - 1);
+    const int g0 = lane & ~(W - 1);  // first lane of the node's group
+    constexpr unsigned GM = W == 32 ? FULL : (1u << (W & 31)) - 1u;
+    const unsigned gb = (bn >> g0) & GM;  // the node's words with new bits
+    const bool fresh = gb != 0u;
+    const bool leader = fresh && w == 0;
     const int64_t vw = (int64_t)v * W + w;
+    // A level with (l + 1) eps_a <= eps_b puts every bit in L(v) whatever
+    // Delta(v) >= 1: nothing to record (all levels of a small-diameter
+    // graph).
+    const bool band = (J.red & RED_BAND) && ((uint64_t)l + 1u) * J.eps_a > J.eps_b;
+    int sx = -1;
+    uint32_t dl = 0;
+    uint8_t bf = 0;
+    if (fresh && (J.red & (RED_DCC | RED_HIST | RED_LC | RED_BAND))) sx = J.sidx[v];
+    if (fresh && band) {
+        dl = J.delta[v];
+        bf = J.bflag[v];  // bit 0: the band row is cleared; bit 1: lc2 holds sums
+    }
     // Frontier and visited words are written only when new bits arrive.  A
     // frontier word left unwritten keeps bits of an older level of the same
     // parity; each such source reached every neighbour one level after this
     // node, so those bits are already in the neighbours' visited words and
     // are masked off wherever the word is read.
-    if (valid && nw) {
+    if (nw) {
         Fout[vw] = nw;
         J.vis[vw] = vis | nw;
     }
-    int sx = -1;
-    if (valid && (J.red & (RED_DCC | RED_HIST | RED_LC | RED_BAND))) sx = J.sidx[v];
-    int c = __popcll(nw);
-    int cL = 0;
-    unsigned long long xs = 0;
-    if ((J.red & RED_LC) && valid && sx < 0 && nw) {
-        const uint64_t lm = J.Lmask[vw];
-        cL = __popcll(nw & lm);
-        if (J.red & RED_SQ) {
-            const uint8_t f = J.sqflag[v];
-            if (f) {
-                const int p = J.pivot[v];
-                if (f & 1) {
-                    // Sources beyond the threshold reaching v now, at level l.
-                    uint64_t bh = nw & ~lm;
-                    while (bh) {
-                        const int i = w * 64 + __ffsll((long long)bh) - 1;
-                        bh &= bh - 1;
-                        const long long e = (long long)l - J.dcc[(int64_t)p * J.dcc_k + i];
-                        xs += (unsigned long long)(e * e);
-                    }
-                }
-                if (f & 2) {
-                    const int is = J.istar[p];
-                    if ((is >> 6) == w && ((nw >> (is & 63)) & 1ull)) J.fdist[v] = (uint32_t)l;
-                }
-            }
-        }
-    }
-    int had = (vis & ~pad_mask(J.k, w)) != 0;
-    int done_before = vis == ~0ull;
-    int done_after = (vis | nw) == ~0ull;
-    int pv = nw ? (w * 64 + __ffsll((long long)nw) - 1) : 0x7FFFFFFF;
+    const bool had =
+        ((__ballot_sync(FULL, (vis & ~pad_mask(J.k, w)) != 0ull) >> g0) & GM) != 0u;
+    // A node that gained bits was not complete before.
+    const bool done = ((__ballot_sync(FULL, (vis | nw) == ~0ull) >> g0) & GM) == GM;
+    const int pc = __popcll(nw);
+    int c = pc;
 #pragma unroll
-    for (int o = 1; o < W; o <<= 1) {
-        c += __shfl_xor_sync(FULL, c, o);
-        cL += __shfl_xor_sync(FULL, cL, o);
-        xs += __shfl_xor_sync(FULL, xs, o);
-        had |= __shfl_xor_sync(FULL, had, o);
-        done_before &= __shfl_xor_sync(FULL, done_before, o);
-        done_after &= __shfl_xor_sync(FULL, done_after, o);
-        pv = min(pv, __shfl_xor_sync(FULL, pv, o));
-    }
-    const bool leader = valid && w == 0;
-    // (l + 1) eps_a <= eps_b puts every bit of level l in L(v) whatever
-    // Delta(v) >= 1: nothing to record (all levels of a small-diameter
-    // graph).
-    if ((J.red & RED_BAND) && valid && sx < 0 && c > 0 &&
-        ((uint64_t)l + 1u) * J.eps_a > J.eps_b) {
-        // The hybrid's classification on arrival (section 3's use of the
-        // triangle inequality): d(c(v), c_i) lies within l -+ Delta(v).  The
-        // class is the same for the W lanes of v (same l and Delta).
-        // lc2 collects the complement of L(v) (the sums over HC(v)), so a
-        // node whose bits all land in L(v) -- every node of a graph of
-        // small diameter -- writes nothing here.
-        const uint64_t Dv = had ? (uint64_t)J.delta[v] : (uint64_t)l;
-        const uint64_t ul = (uint64_t)l;
-        if ((ul - Dv) * J.eps_a > Dv * J.eps_b) {
-            if (leader) {  // in HC(v); bflag bit 2: lc2[v] holds sums
-                const uint8_t f = J.bflag[v];
-                const uint64_t s1 = ul * (uint64_t)c, s2 = ul * ul * (uint64_t)c;
-                if (f & 2) {
-                    J.lc2[2 * (int64_t)v] += s1;
-                    J.lc2[2 * (int64_t)v + 1] += s2;
-                } else {
-                    J.lc2[2 * (int64_t)v] = s1;
-                    J.lc2[2 * (int64_t)v + 1] = s2;
-                    J.bflag[v] = f | 2;
-                }
-            }
-        } else if ((ul + Dv) * J.eps_a > Dv * J.eps_b) {
-            // Deferred: a byte per source, the first such level clearing
-            // the row (each lane its own word's 64 bytes).
-            const uint64_t o = ul + Dv - Dv * J.eps_b / J.eps_a;  // 1 .. 2 Delta
-            uint8_t *row = J.band + (int64_t)v * (64 * W) + 64 * w;
-            const unsigned gmask =
-                W == 32 ? FULL : (((1u << (W & 31)) - 1u) << ((lane / W) * W));
-            const uint8_t f = J.bflag[v];  // bit 1: v's band row is cleared
-            __syncwarp(gmask);               // every lane of v has read it
-            if (!(f & 1)) {
-                uint4 *r4 = reinterpret_cast<uint4 *>(row);
-                const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-                r4[0] = z; r4[1] = z; r4[2] = z; r4[3] = z;
-                if (leader) J.bflag[v] = f | 1;
-            }
-            if (o > 255u) {
-                if (leader) J.ctl->band_ovf = 1;
-            } else {
-                uint64_t bb = nw;
-                while (bb) {
-                    row[__ffsll((long long)bb) - 1] = (uint8_t)o;
-                    bb &= bb - 1;
-                }
-            }
-        }
-    }
-    if (leader && c > 0) {
-        const uint64_t ul = (uint64_t)l;
-        if (J.red & RED_SUM) {
-            J.sum2[2 * (int64_t)v] += ul * (uint64_t)c;
-            J.sum2[2 * (int64_t)v + 1] += ul * ul * (uint64_t)c;
-        }
-        if (cL > 0) {
-            J.lc2[2 * (int64_t)v] += ul * (uint64_t)cL;
-            J.lc2[2 * (int64_t)v + 1] += ul * ul * (uint64_t)cL;
-        }
-        if (xs) {
-            const uint64_t lo = J.hcse[2 * (int64_t)v] + xs;
-            J.hcse[2 * (int64_t)v + 1] += lo < xs ? 1u : 0u;
-            J.hcse[2 * (int64_t)v] = lo;
-        }
-        if ((J.red & RED_PIVOT) && !had) {
+    for (int o = 1; o < W; o <<= 1) c += __shfl_xor_sync(FULL, c, o);
+    const uint64_t ul = (uint64_t)l;
+    if ((J.red & RED_PIVOT) && __any_sync(FULL, fresh && !had)) {
+        // lowest new bit of the node: in its first word with new bits
+        const int f = w * 64 + __ffsll((long long)nw) - 1;
+        const int pv = __shfl_sync(FULL, f, g0 + __ffs(gb | (1u << (W - 1))) - 1);
+        if (leader && !had) {
             J.pivot[v] = pv;
             J.delta[v] = (uint32_t)l;
         }
     }
-    if (leader && clear_tflag) J.tflag[v] = 0u;
-    if ((J.red & RED_LEVELS) && valid && nw) {
+    if ((J.red & RED_SUM) && leader) {
+        atomicAdd((unsigned long long *)&J.sum2[2 * (int64_t)v], ul * (uint64_t)c);
+        atomicAdd((unsigned long long *)&J.sum2[2 * (int64_t)v + 1], ul * ul * (uint64_t)c);
+    }
+    if (J.red & RED_LC) {
+        int cL = 0;
+        unsigned long long xs = 0;
+        if (sx < 0 && nw) {
+            const uint64_t lm = J.Lmask[vw];
+            cL = __popcll(nw & lm);
+            if (J.red & RED_SQ) {
+                const uint8_t f = J.sqflag[v];
+                if (f) {
+                    const int p = J.pivot[v];
+                    if (f & 1) {
+                        // Sources beyond the threshold reaching v now, at level l.
+                        uint64_t bh = nw & ~lm;
+                        while (bh) {
+                            const int i = w * 64 + __ffsll((long long)bh) - 1;
+                            bh &= bh - 1;
+                            const long long e =
+                                (long long)l - J.dcc[(int64_t)p * J.dcc_k + i];
+                            xs += (unsigned long long)(e * e);
+                        }
+                    }
+                    if (f & 2) {
+                        const int is = J.istar[p];
+                        if ((is >> 6) == w && ((nw >> (is & 63)) & 1ull))
+                            J.fdist[v] = (uint32_t)l;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < W; o <<= 1) {
+            cL += __shfl_xor_sync(FULL, cL, o);
+            xs += __shfl_xor_sync(FULL, xs, o);
+        }
+        if (leader && cL > 0) {
+            J.lc2[2 * (int64_t)v] += ul * (uint64_t)cL;
+            J.lc2[2 * (int64_t)v + 1] += ul * ul * (uint64_t)cL;
+        }
+        if (leader && xs) {
+            const uint64_t lo = J.hcse[2 * (int64_t)v] + xs;
+            J.hcse[2 * (int64_t)v + 1] += lo < xs ? 1u : 0u;
+            J.hcse[2 * (int64_t)v] = lo;
+        }
+    }
+    if (band) {
+        __syncwarp();  // every lane of v has read its flag
+        if (fresh && sx < 0) {
+            // The hybrid's classification on arrival (section 3's use of the
+            // triangle inequality): d(c(v), c_i) lies within l -+ Delta(v).
+            // The class is the same for the W lanes of v (same l and Delta).
+            // lc2 collects the complement of L(v) (the sums over HC(v)), so
+            // a node whose bits all land in L(v) writes nothing here.
+            const uint64_t Dv = had ? (uint64_t)dl : ul;
+            if ((ul - Dv) * J.eps_a > Dv * J.eps_b) {
+                if (leader) {  // in HC(v)
+                    const uint64_t s1 = ul * (uint64_t)c, s2 = ul * ul * (uint64_t)c;
+                    if (bf & 2) {
+                        atomicAdd((unsigned long long *)&J.lc2[2 * (int64_t)v], s1);
+                        atomicAdd((unsigned long long *)&J.lc2[2 * (int64_t)v + 1], s2);
+                    } else {
+                        J.lc2[2 * (int64_t)v] = s1;
+                        J.lc2[2 * (int64_t)v + 1] = s2;
+                        J.bflag[v] = bf | 2;
+                    }
+                }
+            } else if ((ul + Dv) * J.eps_a > Dv * J.eps_b) {
+                // Deferred: a byte per source, the first such level clearing
+                // the row (each lane its own word's 64 bytes).
+                const uint64_t o = ul + Dv - Dv * J.eps_b / J.eps_a;  // 1 .. 2 Delta
+                uint8_t *row = J.band + (int64_t)v * (64 * W) + 64 * w;
+                if (!(bf & 1)) {
+                    uint4 *r4 = reinterpret_cast<uint4 *>(row);
+                    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+                    r4[0] = z; r4[1] = z; r4[2] = z; r4[3] = z;
+                    if (leader) J.bflag[v] = bf | 1;
+                }
+                if (o > 255u) {
+                    if (leader) J.ctl->band_ovf = 1;
+                } else {
+                    uint64_t bb = nw;
+                    while (bb) {
+                        row[__ffsll((long long)bb) - 1] = (uint8_t)o;
+                        bb &= bb - 1;
+                    }
+                }
+            }
+        }
+    }
+    if ((J.red & RED_LEVELS) && nw) {
         uint64_t b = nw;
         while (b) {
             const int i = w * 64 + __ffsll((long long)b) - 1;
@@ -247,24 +264,31 @@ __device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, bool valid,
         }
     }
     if (J.red & RED_HIST) {
-        const uint64_t x = (valid && sx < 0) ? nw : 0ull;
-        if constexpr (W <= 8) {
-            if (__ballot_sync(FULL, x != 0ull)) {
-                const uint32_t lo = warp_transpose32((uint32_t)x, lane);
-                const uint32_t hi = warp_transpose32((uint32_t)(x >> 32), lane);
-                constexpr uint32_t M0 = W == 1 ? 0xFFFFFFFFu
-                                      : W == 2 ? 0x55555555u
-                                      : W == 4 ? 0x11111111u
-                                               : 0x01010101u;
+        // Lanes with one or two bits each add them one by one; a warp with a
+        // fuller word transposes its words, so that a lane holds the counts
+        // of sources s*64 + lane and s*64 + 32 + lane (distinct banks: no
+        // conflicts).  More turns of the loop are dearer than their count:
+        // early on many lanes hold the bits of the same few far-reaching
+        // sources and their adds serialise (R-MAT 20, k = 256, level 2: 276
+        // us at up to 6 turns, 219 at 1 or 2).  Sixteen words: bit by bit
+        // alone took R-MAT 18, k = 1000 1.80 ms a traversal, this 0.66.
+        constexpr int kBitLoop = W <= 8 ? 2 : 8;
+        const uint64_t x = sx < 0 ? nw : 0ull;
+        if (__any_sync(FULL, sx < 0 && pc > kBitLoop)) {
+            const uint32_t lo = warp_transpose32((uint32_t)x, lane);
+            const uint32_t hi = warp_transpose32((uint32_t)(x >> 32), lane);
+            constexpr uint32_t M0 = W == 1 ? 0xFFFFFFFFu
+                                  : W == 2 ? 0x55555555u
+                                  : W == 4 ? 0x11111111u
+                                  : W == 8 ? 0x01010101u
+                                  : W == 16 ? 0x00010001u
+                                            : 1u;
 #pragma unroll
-                for (int s = 0; s < W; ++s) {
-                    // lane holds the counts of sources s*64 + lane and
-                    // s*64 + 32 + lane (distinct banks: no conflicts)
-                    const unsigned c0 = __popc(lo & (M0 << s));
-                    const unsigned c1 = __popc(hi & (M0 << s));
-                    if (c0) atomicAdd(&s_hist[s * 64 + lane], c0);
-                    if (c1) atomicAdd(&s_hist[s * 64 + 32 + lane], c1);
-                }
+            for (int s = 0; s < W; ++s) {
+                const unsigned c0 = __popc(lo & (M0 << s));
+                const unsigned c1 = __popc(hi & (M0 << s));
+                if (c0) atomicAdd(&s_hist[s * 64 + lane], c0);
+                if (c1) atomicAdd(&s_hist[s * 64 + 32 + lane], c1);
             }
         } else {
             uint64_t b = x;
@@ -277,15 +301,14 @@ __device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, bool valid,
     }
     // Stamp frontier nodes with the level (a later top-down level builds its
     // queue from the stamps) and count level statistics.
-    const bool fr = leader && c > 0;
-    if (fr) {
+    if (leader) {
         J.fstamp[v] = (uint32_t)l;
         A.ef += (unsigned)deg;
         A.nfront += 1;
-    }
-    if (leader && done_after && !done_before) {
-        A.eu_dec += (unsigned)deg;
-        A.ninc_dec += 1;
+        if (done) {
+            A.eu_dec += (unsigned)deg;
+            A.ninc_dec += 1;
+        }
     }
 }
 
@@ -520,7 +543,7 @@ __device__ void block_compact(int64_t N, Keep keep, Get get, int32_t *out, unsig
 template <int W>
 __device__ __forceinline__ void td_push(const BfsJob &J, const int32_t *__restrict__ col,
                                         uint64_t f, int64_t b, int64_t e, LevelCtl *C,
-                                        int32_t *Tout, LaneAcc &A, const Stage &stage)
+                                        int32_t *Tout, LaneAcc &A, const Stage &stage, unsigned lv)
 {
     constexpr int NPW = 32 / W;
     const int lane = threadIdx.x & 31;
@@ -556,7 +579,7 @@ __device__ __forceinline__ void td_push(const BfsJob &J, const int32_t *__restri
                     if (!nbits) continue;
                     const uint64_t old =
                         atomicOr((unsigned long long *)&J.nxt[(int64_t)v * W + ww], nbits);
-                    if (old == 0ull && atomicCAS(&J.tflag[v], 0u, 1u) == 0u)
+                    if (old == 0ull && atomicExch(&J.tflag[v], lv) != lv)
                         stage_push(stage, v, Tout, &C->tlen);
                 }
             }
@@ -586,7 +609,7 @@ __device__ __forceinline__ void td_push(const BfsJob &J, const int32_t *__restri
             if (!nbits) continue;
             const uint64_t old =
                 atomicOr((unsigned long long *)&J.nxt[(int64_t)v * W + w], nbits);
-            if (old == 0ull && atomicCAS(&J.tflag[v], 0u, 1u) == 0u)
+            if (old == 0ull && atomicExch(&J.tflag[v], lv) != lv)
                 stage_push(stage, v, Tout, &C->tlen);
         }
     }
@@ -600,7 +623,7 @@ __device__ __forceinline__ void td_push(const BfsJob &J, const int32_t *__restri
 template <int W>
 __device__ __forceinline__ void td_push_lane(const BfsJob &J, const int32_t *__restrict__ row,
                                              int len, uint64_t f, int w, LevelCtl *C,
-                                             int32_t *Tout, LaneAcc &A, const Stage &stage)
+                                             int32_t *Tout, LaneAcc &A, const Stage &stage, unsigned lv)
 {
     unsigned wl = 0;
     for (int x = 0; x < len; x += kUnroll) {
@@ -619,7 +642,7 @@ __device__ __forceinline__ void td_push_lane(const BfsJob &J, const int32_t *__r
             if (!nbits) continue;
             const uint64_t old =
                 atomicOr((unsigned long long *)&J.nxt[(int64_t)v * W + w], nbits);
-            if (old == 0ull && atomicCAS(&J.tflag[v], 0u, 1u) == 0u)
+            if (old == 0ull && atomicExch(&J.tflag[v], lv) != lv)
                 stage_push(stage, v, Tout, &C->tlen);
         }
     }
@@ -670,15 +693,16 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
     if (threadIdx.x == 0) s_cnt = 0;
 
     // Warp time per phase (tracing): lane 0 of each warp adds the clock
-    // cycles since its previous lap to the CTA's counter of the phase that
+    // cycles since its previous lap to the warp's counter of the phase that
     // just ended; waits in the grid barrier count as CC_PH_BARRIER.
-    __shared__ unsigned long long s_ph[CC_NUM_PHASES];
-    if (threadIdx.x < CC_NUM_PHASES) s_ph[threadIdx.x] = 0;
+    __shared__ unsigned long long s_ph[CC_NUM_PHASES][kBlock / 32];
+    for (int i = tid; i < CC_NUM_PHASES * (kBlock / 32); i += kBlock)
+        s_ph[i / (kBlock / 32)][i % (kBlock / 32)] = 0;
     __syncthreads();
     long long ph_t = clock64();
     auto lap = [&](int p) {
         const long long t = clock64();
-        if (lane == 0) atomicAdd(&s_ph[p], (unsigned long long)(t - ph_t));
+        if (lane == 0) s_ph[p][tid >> 5] += (unsigned long long)(t - ph_t);
         ph_t = t;
     };
     auto sync_after = [&](int p) {
@@ -822,7 +846,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                 const int64_t bb = b + part * per, ee = min(e, bb + per);
                 if (bb >= ee) continue;
                 const uint64_t f = Fin[(int64_t)u * W + w];
-                td_push<W>(J, col, f, bb, ee, C, Tout, A, stage);
+                td_push<W>(J, col, f, bb, ee, C, Tout, A, stage, (unsigned)l);
             }
             // Otherwise nodes of at most kLightMaxDeg entries: a lane group
             // each, NPW per warp (a grid's frontier node has 4 entries: a
@@ -835,7 +859,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                     const int64_t b = rp[u], e = rp[u + 1];
                     if (e - b <= kLightMaxDeg) {
                         const uint64_t f = Fin[(int64_t)u * W + w];
-                        if (f) td_push_lane<W>(J, col + b, (int)(e - b), f, w, C, Tout, A, stage);
+                        if (f) td_push_lane<W>(J, col + b, (int)(e - b), f, w, C, Tout, A, stage, (unsigned)l);
                     }
                 }
             }
@@ -862,7 +886,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                     const int64_t bb = __shfl_sync(FULL, b, src);
                     const int64_t ee = __shfl_sync(FULL, e, src);
                     const uint64_t f = Fin[(int64_t)uu * W + w];
-                    td_push<W>(J, col, f, bb, ee, C, Tout, A, stage);
+                    td_push<W>(J, col, f, bb, ee, C, Tout, A, stage, (unsigned)l);
                 }
             }
             // Heavy frontier nodes: the warp's chunk tasks (every nwarps-th)
@@ -885,7 +909,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                     if (__all_sync(FULL, f == 0ull)) continue;
                     const int64_t b = J.tHb[gwarp + (j0 + src) * nwarps];
                     td_push<W>(J, col, f, b, min(b + (int64_t)kChunk, rp[uu + 1]), C, Tout,
-                               A, stage);
+                               A, stage, (unsigned)l);
                 }
             }
             stage_flush(stage, Tout, &C->tlen);
@@ -905,7 +929,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                     if (acc) J.nxt[vw] = 0;
                     deg = prp[v + 1] - prp[v];
                 }
-                tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, deg, Fout, A, s_hist, true);
+                tile_reduce<W>(J, l, v, vis, acc & ~vis, deg, Fout, A, s_hist);
             }
             flush_level(J, l, C, A, 0u, s_hist, doHist);
             if (!sync_after(CC_PH_TD_FINAL)) return;
@@ -997,13 +1021,26 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                 }
                 __syncthreads();
             }
+            // With fewer tasks than warps the classes are dealt to the warps
+            // one after another, so that none works through a light tile, a
+            // medium node and a chunk in turn while others idle.
+            const int64_t tl_len = s_al.nT, ml_len = s_al.nM;
+            // With fewer light and medium nodes than warps, light nodes take a
+            // warp each too (one step over at most 32 entries in place of
+            // up to eight dependent ones).
+            const bool lw = s_al.nL + ml_len <= nwarps;
+            const int64_t al_len = lw ? 0 : s_al.nL, lw_len = lw ? s_al.nL : 0;
+            int64_t dealt = (tl_len + NPW - 1) / NPW;
+            auto my_turn = [&]() {
+                const int64_t x = gwarp - (dealt < nwarps ? dealt : 0);
+                return x < 0 ? x + nwarps : x;
+            };
             // A0: tiny nodes, one thread per (node, word); the neighbours come
             // with the list entry, so every frontier word is gathered at once.
             // The next tile's entries load while this tile's words are in
             // flight.
             const int32_t *const TLcur = s_al.T;
             const int4 *const TAcur = s_al.TA;
-            const int64_t tl_len = s_al.nT;
             int vnext = 0;
             int4 nbnext = make_int4(-1, -1, -1, -1);
             if (gwarp * NPW + grp < tl_len) {
@@ -1031,13 +1068,13 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                     A.words += wl;
                 }
                 __syncwarp();
-                tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, deg, Fout, A, s_hist, false);
+                tile_reduce<W>(J, l, v, vis, acc & ~vis, deg, Fout, A, s_hist);
             }
             // A1: light nodes of the active list, one thread per (node, word).
             const int32_t *const ALcur = s_al.L;
-            const int64_t al_len = s_al.nL;
-            int anext = gwarp * NPW + grp < al_len ? ALcur[gwarp * NPW + grp] : 0;
-            for (int64_t t = gwarp; t * NPW < al_len; t += nwarps) {
+            const int64_t t0L = my_turn();
+            int anext = t0L * NPW + grp < al_len ? ALcur[t0L * NPW + grp] : 0;
+            for (int64_t t = t0L; t * NPW < al_len; t += nwarps) {
                 const int64_t li = t * NPW + grp;
                 const bool valid = li < al_len;
                 const int v = valid ? anext : 0;
@@ -1051,24 +1088,23 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                     acc = gather_scan<W, kUnroll>(pcol, Fin, b, 0, e, 1, w, A.words, 1,
                                                   [&](uint64_t a) { return (a | vis) == ~0ull; });
                 __syncwarp();
-                tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, e - b, Fout, A, s_hist,
-                               false);
+                tile_reduce<W>(J, l, v, vis, acc & ~vis, e - b, Fout, A, s_hist);
             }
             lap(CC_PH_BU_LIGHT);
-            // A2: medium nodes, a warp per node.  The warp scans NPW of its
+            // A2: medium nodes (and few light ones), a warp per node.  It scans NPW of its
             // nodes one after another, lane group g keeping node g's words,
             // then one fused reduction covers all NPW.
             const int32_t *const MLcur = s_al.M;
-            const int64_t ml_len = s_al.nM;
-            for (int64_t t0 = gwarp; t0 < ml_len; t0 += (int64_t)NPW * nwarps) {
+            dealt += (al_len + NPW - 1) / NPW;
+            const int64_t wl_len = lw_len + ml_len;
+            for (int64_t t0 = my_turn(); t0 < wl_len; t0 += (int64_t)NPW * nwarps) {
                 int myv = 0;
                 uint64_t myvis = ~0ull, myres = 0;
                 int64_t mydeg = 0;
-                bool myvalid = false;
                 for (int g = 0; g < NPW; ++g) {
                     const int64_t t = t0 + (int64_t)g * nwarps;
-                    if (t >= ml_len) break;
-                    const int v = MLcur[t];
+                    if (t >= wl_len) break;
+                    const int v = t < lw_len ? ALcur[t] : MLcur[t - lw_len];
                     const uint64_t visw = J.vis[(int64_t)v * W + w];
                     const int64_t b = prp[v], e = prp[v + 1];
                     uint64_t r = 0;
@@ -1084,11 +1120,9 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                         myvis = visw;
                         myres = r;
                         mydeg = e - b;
-                        myvalid = true;
                     }
                 }
-                tile_reduce<W>(J, l, myvalid, myv, myvis, myres & ~myvis, mydeg, Fout, A,
-                               s_hist, false);
+                tile_reduce<W>(J, l, myv, myvis, myres & ~myvis, mydeg, Fout, A, s_hist);
             }
             lap(CC_PH_BU_MEDIUM);
             // A3: heavy nodes, 256-entry warp tasks OR-ing into nxt.  Read in
@@ -1143,7 +1177,8 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                         for (int64_t t = tb; t < tend; ++t) heavy_task(t);
                     }
                 } else {
-                    for (int64_t t = gwarp; t < hc_len; t += nwarps) heavy_task(t);
+                    dealt += wl_len;
+                    for (int64_t t = my_turn(); t < hc_len; t += nwarps) heavy_task(t);
                 }
                 if (!sync_after(CC_PH_BU_HEAVY)) return;
                 // B: finalise the heavy nodes.
@@ -1162,7 +1197,7 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
                         if (acc) J.nxt[vw] = 0;
                         deg = prp[v + 1] - prp[v];
                     }
-                    tile_reduce<W>(J, l, valid, v, vis, acc & ~vis, deg, Fout, A, s_hist, false);
+                    tile_reduce<W>(J, l, v, vis, acc & ~vis, deg, Fout, A, s_hist);
                     const unsigned left = __ballot_sync(FULL, (vis | acc) != ~0ull);
                     if (lane == 0) hinc += groups_of<W>(left);
                 }
@@ -1174,7 +1209,12 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
         }
     }
     // Pass statistics.
-    if (tid < CC_NUM_PHASES) atomicAdd(&ctl->ph_cycles[tid], s_ph[tid]);
+    __syncthreads();
+    if (tid < CC_NUM_PHASES) {
+        unsigned long long t = 0;
+        for (int i = 0; i < kBlock / 32; ++i) t += s_ph[tid][i];
+        atomicAdd(&ctl->ph_cycles[tid], t);
+    }
     if (gtid == 0) {
         ctl->levels = last;
         ctl->ninc_final = ninc;
