@@ -180,8 +180,8 @@ struct cc_graph {
     uint64_t beta_total = 0;
     bool has_beta = false;
     // outbound / inbound reachability samples: order, per-node state, queues
-    DevBuf rc_order, rc_rank, rc_cnt, rc_extra, rc_dsum, rc_T, rc_qstamp, rc_vis, rc_F, rc_nxt,
-        rc_lev, rc_Q0, rc_Q1, rc_TL, rc_out;
+    DevBuf rc_order, rc_rank, rc_cnt, rc_sat, rc_dsum, rc_T, rc_qstamp, rc_vis, rc_F, rc_nxt,
+        rc_lev, rc_Q0, rc_Q1, rc_QB0, rc_QB1, rc_TL, rc_out;
     bool sq = false;       // the current cc_estimate call wants SqErrEst
     int64_t D1 = 0;        // levels (largest distance) of the last first pass
     int cw = 32;           // sources per chunk of the last chunked first pass
@@ -583,9 +583,9 @@ void free_graph(cc_graph *g)
                      &g->beta, &g->nw_keys, &g->nw_tk, &g->nw_vals, &g->nw_tv, &g->nw_pre,
                      &g->nw_flags, &g->nw_tau, &g->nw_pick, &g->nw_mu, &g->nw_bsrc,
                      &g->nw_msum, &g->nw_wsum, &g->nw_S, &g->nw_hist, &g->nw_TS, &g->nw_lc,
-                     &g->nw_out, &g->rc_order, &g->rc_rank, &g->rc_cnt, &g->rc_extra,
+                     &g->nw_out, &g->rc_order, &g->rc_rank, &g->rc_cnt, &g->rc_sat,
                      &g->rc_dsum, &g->rc_T, &g->rc_qstamp, &g->rc_vis, &g->rc_F, &g->rc_nxt,
-                     &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_TL, &g->rc_out};
+                     &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
     for (DevBuf *b : all) b->release();
     if (g->ev0) cudaEventDestroy(g->ev0);
     if (g->ev1) cudaEventDestroy(g->ev1);
@@ -1407,9 +1407,9 @@ size_t ccg::graph_workspace_bytes(cc_graph_t g)
                      &g->beta, &g->nw_keys, &g->nw_tk, &g->nw_vals, &g->nw_tv, &g->nw_pre,
                      &g->nw_flags, &g->nw_tau, &g->nw_pick, &g->nw_mu, &g->nw_bsrc,
                      &g->nw_msum, &g->nw_wsum, &g->nw_S, &g->nw_hist, &g->nw_TS, &g->nw_lc,
-                     &g->nw_out, &g->rc_order, &g->rc_rank, &g->rc_cnt, &g->rc_extra,
+                     &g->nw_out, &g->rc_order, &g->rc_rank, &g->rc_cnt, &g->rc_sat,
                      &g->rc_dsum, &g->rc_T, &g->rc_qstamp, &g->rc_vis, &g->rc_F, &g->rc_nxt,
-                     &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_TL, &g->rc_out};
+                     &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
     size_t t = 0;
     for (const DevBuf *b : ws) t += b->cap;
     return t;
@@ -2110,7 +2110,7 @@ int cc_reach_estimate(cc_graph_t g, int32_t k, uint64_t seed, int32_t inbound, v
     RC(g->rc_order.ensure(n * 4));
     RC(g->rc_rank.ensure(n * 4));
     RC(g->rc_cnt.ensure(n * 4));
-    RC(g->rc_extra.ensure(n));
+    RC(g->rc_sat.ensure(n * 4));
     RC(g->rc_dsum.ensure(n * 8));
     RC(g->rc_T.ensure(n * 8));
     RC(g->rc_qstamp.ensure(n * 4));
@@ -2121,10 +2121,13 @@ int cc_reach_estimate(cc_graph_t g, int32_t k, uint64_t seed, int32_t inbound, v
     RC(g->rc_Q0.ensure(n * 4));
     RC(g->rc_Q1.ensure(n * 4));
     RC(g->rc_TL.ensure(n * 4));
+    const size_t nbig = (size_t)g->arcs / kReachBigDeg + 1;
+    RC(g->rc_QB0.ensure(nbig * 4));
+    RC(g->rc_QB1.ensure(nbig * 4));
     RC(g->rc_out.ensure(n * 16));
     RC(g->ctl.ensure(sizeof(Ctl)));
     CK(cudaMemsetAsync(g->rc_cnt.p, 0, n * 4, st));
-    CK(cudaMemsetAsync(g->rc_extra.p, 0, n, st));
+    CK(cudaMemsetAsync(g->rc_sat.p, 0xFF, n * 4, st));
     CK(cudaMemsetAsync(g->rc_dsum.p, 0, n * 8, st));
     CK(cudaMemsetAsync(g->rc_T.p, 0, n * 8, st));
     CK(cudaMemsetAsync(g->rc_qstamp.p, 0, n * 4, st));
@@ -2146,7 +2149,7 @@ int cc_reach_estimate(cc_graph_t g, int32_t k, uint64_t seed, int32_t inbound, v
     j.order = g->rc_order.as<int32_t>();
     j.rank = g->rc_rank.as<int32_t>();
     j.cnt = g->rc_cnt.as<int32_t>();
-    j.extra = g->rc_extra.as<uint8_t>();
+    j.satpos = g->rc_sat.as<uint32_t>();
     j.dsum = g->rc_dsum.as<uint64_t>();
     j.T = g->rc_T.as<int64_t>();
     j.qstamp = g->rc_qstamp.as<uint32_t>();
@@ -2157,6 +2160,8 @@ int cc_reach_estimate(cc_graph_t g, int32_t k, uint64_t seed, int32_t inbound, v
     j.Q[0] = g->rc_Q0.as<int32_t>();
     j.Q[1] = g->rc_Q1.as<int32_t>();
     j.TL = g->rc_TL.as<int32_t>();
+    j.QB[0] = g->rc_QB0.as<int32_t>();
+    j.QB[1] = g->rc_QB1.as<int32_t>();
     j.ctl = g->ctl.as<Ctl>();
     j.timeout_ns = kTimeoutNs;
     if (!g->ev0) {

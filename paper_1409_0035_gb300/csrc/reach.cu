@@ -4,7 +4,7 @@
 // their distances, and the rank position of the k-th.
 //
 // One persistent cooperative launch walks the order in groups of 64 W
-// sources.  Each group is a bit-packed multi-source BFS on the search graph
+// sources whose search can still reach a node that takes samples.  Each group is a bit-packed multi-source BFS on the search graph
 // (G^T for outbound, G for inbound: bit i leaves the group's i-th source),
 // recording the level at which each bit first reaches each node; then every
 // node it touched accepts its lowest-rank bits (its own excluded) until it
@@ -12,7 +12,7 @@
 // next samples in rank order.
 //
 // Pruning: a node x saturated at the start of a group -- k + 1 sources
-// other than x have reached it, or k have and x's own search has run --
+// other than x have reached it, or k have and x's own position is past --
 // holds k + 1 nodes of smaller rank than every source still to come among
 // x and its reachability set; every node that reaches x through x holds k
 // of them other than itself, so x is neither entered nor expanded.  Nodes
@@ -48,171 +48,332 @@ namespace ccg {
 namespace {
 
 constexpr int kRT = 256;
+// Positions of the order tested for useful sources at once.
+constexpr int kMaxWin = 32768;
+// Arcs beyond which a source is taken without a proof that it is useful.
+constexpr int kTestArcs = 4096;
 
 struct RState {
-    unsigned qlen[2];
+    unsigned qlen[2], blen[2];  // frontier queue: small nodes, big ones
     unsigned tlen[2];
-    unsigned long long levels, groups, pushes;
+    unsigned long long levels, groups;
+    uint8_t flags[2][kMaxWin / 8];  // useful positions of a window, by parity
 };
 
-__device__ __forceinline__ bool saturated(const ReachJob &J, int32_t x, int64_t base)
+// x is saturated for the sources from position base on (see above): k others
+// have reached it and either another one has or its own position is past.
+__device__ __forceinline__ bool saturated(const ReachJob &J, int32_t x, uint32_t base)
 {
-    const int c = J.cnt[x];
-    return c >= J.k && (J.extra[x] || (int64_t)J.rank[x] < base);
+    return base >= J.satpos[x];
 }
 
+// Mark the useful sources among positions [pos, hi): unsaturated nodes with
+// an unsaturated neighbour on the search graph.  The search of any other
+// source touches no node but its own, whose own bit does not count, so it is
+// dropped (saturation only grows: it stays useless).  Eight positions per
+// warp, four lanes each over the first 64 arcs, the whole warp over a longer
+// row of saturated neighbours.
+__device__ void mark_useful(const ReachJob &J, int64_t pos, int64_t hi, uint8_t *flags,
+                            int64_t gw, int64_t nwarps, int lane)
+{
+    const uint32_t base = (uint32_t)pos;
+    const int64_t nbytes = (hi - pos + 31) / 32 * 4;
+    const int sub = lane >> 2, t = lane & 3;
+    for (int64_t wi = gw; wi < nbytes; wi += nwarps) {
+        const int64_t p = pos + wi * 8 + sub;
+        int64_t b = 0, e = 0;
+        if (p < hi) {
+            const int32_t s = J.order[p];
+            if (!saturated(J, s, base)) {
+                b = J.rp[s];
+                e = J.rp[s + 1];
+            }
+        }
+        bool found = false;
+        int64_t x = b + t;
+        for (int step = 0; step < 4; ++step, x += 16) {
+            int32_t c[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[q] = !found && x + 4 * q < e ? J.col[x + 4 * q] : -1;
+            bool f = false;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) f |= c[q] >= 0 && !saturated(J, c[q], base);
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, f);
+            found = found || ((m >> (4 * sub)) & 15u) != 0u;
+            if (__all_sync(0xFFFFFFFFu, found || x - t + 16 >= e)) break;
+        }
+        unsigned rest = __ballot_sync(0xFFFFFFFFu, t == 0 && !found && e > b + 64);
+        unsigned got = 0;
+        while (rest) {
+            const int l0 = __ffs(rest) - 1;
+            rest &= rest - 1;
+            const int64_t bb = __shfl_sync(0xFFFFFFFFu, b, l0) + 64;
+            const int64_t ee = __shfl_sync(0xFFFFFFFFu, e, l0);
+            bool any = ee - bb > kTestArcs;
+            for (int64_t y = bb; y < ee && !any; y += 128) {
+                int32_t c[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    c[q] = y + lane + 32 * q < ee ? J.col[y + lane + 32 * q] : -1;
+                bool f = false;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) f |= c[q] >= 0 && !saturated(J, c[q], base);
+                any = __any_sync(0xFFFFFFFFu, f);
+            }
+            if (any) got |= 1u << l0;
+        }
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, t == 0 && found) | got;  // bits 0, 4, ..
+        if (lane == 0) {
+            unsigned byte = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) byte |= ((m >> (4 * q)) & 1u) << q;
+            flags[wi] = (uint8_t)byte;
+        }
+    }
+}
+
+// The first G marked positions (offsets from the window's start, ascending)
+// into s_src, by every CTA alike; returns how many the window marks.
+__device__ int pick_sources(const uint8_t *flags, int64_t len, int G, int *s_src)
+{
+    __shared__ int s_w[kRT / 32];
+    const int nwords = (int)((len + 31) / 32);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int kPer = kMaxWin / 32 / kRT;  // words per thread
+    uint32_t m[kPer];
+    int c = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int i = (int)threadIdx.x * kPer + j;
+        m[j] = i < nwords ? __ldcg(reinterpret_cast<const uint32_t *>(flags) + i) : 0u;
+        c += __popc(m[j]);
+    }
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    __syncthreads();  // s_w and s_src of the group before are no longer read
+    if (lane == 31) s_w[wid] = incl;
+    __syncthreads();
+    int at = incl - c, total = 0;
+    for (int w = 0; w < kRT / 32; ++w) {
+        if (w < wid) at += s_w[w];
+        total += s_w[w];
+    }
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+        for (uint32_t b = m[j]; b && at < G; b &= b - 1, ++at)
+            s_src[at] = ((int)threadIdx.x * kPer + j) * 32 + __ffs(b) - 1;
+    __syncthreads();
+    return total;
+}
+
+// What bounds a pass: the grid barriers of its groups (five or more each)
+// and, after the first few groups, nothing else -- most nodes are saturated,
+// and of 512 consecutive sources almost all are useless.  So a group takes
+// the next 64 W *useful* sources of the order, however far apart (directed
+// R-MAT 18 kept whole, k = 64, 262,144 nodes: 21.5 -> 8.0 ms).
 __global__ void __launch_bounds__(kRT, 4) k_reach(ReachJob J, RState *rs)
 {
+    constexpr unsigned FULL = 0xFFFFFFFFu;
     const unsigned nb = gridDim.x;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     const int64_t gw = tid >> 5, nwarps = nthr >> 5;
     const int W = J.W, G = 64 * W;
-    volatile unsigned *qlen = rs->qlen, *tlen = rs->tlen;
+    // lane groups of W lanes: one node's words
+    const int gq = lane & (W - 1), g0 = lane & ~(W - 1), NPW = 32 / W;
+    const unsigned gm = W == 32 ? FULL : ((1u << W) - 1u) << g0;
+    volatile unsigned *qlen = rs->qlen, *blen = rs->blen, *tlen = rs->tlen;
+    __shared__ int s_src[64 * kReachMaxW];
     unsigned epoch = 0;
-    int par = 0;
-    for (int64_t base = 0; base < J.n; base += G, par ^= 1) {
-        const int gs = (int)(J.n - base < G ? J.n - base : G);
+    int wpar = 0, par = 0;
+    int64_t win = 2 * G, next = 0;
+    auto queue = [&](int which, int32_t v) {
+        if (J.rp[v + 1] - J.rp[v] > kReachBigDeg)
+            J.QB[which][atomicAdd((unsigned *)&blen[which], 1u)] = v;
+        else
+            J.Q[which][atomicAdd((unsigned *)&qlen[which], 1u)] = v;
+    };
+    for (int64_t pos = 0; pos < J.n; pos = next, wpar ^= 1) {
+        const int64_t hi = pos + win < J.n ? pos + win : J.n;
+        const uint32_t base = (uint32_t)pos;
+        mark_useful(J, pos, hi, rs->flags[wpar], gw, nwarps, lane);
+        if (!grid_sync(J.ctl, blockIdx.x, nb, J.timeout_ns)) return;
+        const int found = pick_sources(rs->flags[wpar], hi - pos, G, s_src);
+        const int gs = found < G ? found : G;
+        next = found > G ? pos + s_src[G - 1] + 1 : hi;
+        // the next window: twice what this group consumed, in whole words
+        win = ((2 * (next - pos) + 31) & ~31ll);
+        win = win < 2 * G ? 2 * G : win > kMaxWin ? kMaxWin : win;
+        if (gs == 0) continue;
         int cur = 0;
         // sources of the group (distinct nodes: one thread each)
         for (int64_t i = tid; i < gs; i += nthr) {
-            const int32_t s = J.order[base + i];
-            if (saturated(J, s, base)) continue;
+            const int32_t s = J.order[pos + s_src[i]];
             const uint64_t bit = 1ull << (i & 63);
             J.vis[(int64_t)s * W + (i >> 6)] = bit;
             J.F[(int64_t)s * W + (i >> 6)] = bit;
             J.lev[(int64_t)s * G + i] = 0;
-            J.Q[0][atomicAdd((unsigned *)&qlen[0], 1u)] = s;
-            J.TL[atomicAdd((unsigned *)&tlen[par], 1u)] = s;
+            queue(0, s);
+            J.TL[i] = s;
         }
+        if (tid == 0) tlen[par] = (unsigned)gs;
         if (!grid_sync(J.ctl, blockIdx.x, nb, J.timeout_ns)) return;
         uint32_t level = 0;
         for (;;) {
-            const unsigned qn = qlen[cur];
-            if (qn == 0) break;
+            const unsigned qn = qlen[cur], bn = blen[cur];
+            if (qn + bn == 0) break;
             ++level;
             ++epoch;
             const int nxq = cur ^ 1;
-            // expand: a warp per frontier node, a lane per arc
-            for (int64_t idx = gw; idx < qn; idx += nwarps) {
-                const int32_t u = J.Q[cur][idx];
-                uint64_t Fu[kReachMaxW];
-#pragma unroll
-                for (int q = 0; q < kReachMaxW; ++q)
-                    Fu[q] = q < W ? J.F[(int64_t)u * W + q] : 0;
-                for (int64_t e = J.rp[u] + lane; e < J.rp[u + 1]; e += 32) {
-                    const int32_t w = J.col[e];
-                    if (saturated(J, w, base)) continue;
+            // Expand arcs x0, x0 + step, ... of node u, a lane per arc (all
+            // lanes of the warp together).
+            auto expand = [&](int32_t u, int64_t x0, int64_t step) {
+                const uint64_t Fw = lane < W ? J.F[(int64_t)u * W + lane] : 0;
+                const unsigned words = __ballot_sync(FULL, Fw != 0);
+                const int64_t end = J.rp[u + 1];
+                for (int64_t e0 = J.rp[u] + x0; e0 < end; e0 += step) {
+                    const int64_t e = e0 + lane;
+                    int32_t w = 0;
+                    bool ok = e < end;
+                    if (ok) {
+                        w = J.col[e];
+                        ok = !saturated(J, w, base);
+                    }
+                    if (!__any_sync(FULL, ok)) continue;
                     bool any = false;
-                    if (J.w) {
-                        // arc lengths: relax every changed source of u into w
-                        const uint64_t len = J.w[e];
-#pragma unroll
-                        for (int q = 0; q < kReachMaxW; ++q) {
-                            if (q >= W) break;
-                            uint64_t imp = 0;
-                            for (uint64_t x = Fu[q]; x; x &= x - 1) {
+                    const uint64_t len = J.w && ok ? J.w[e] : 0;
+                    for (unsigned m = words; m; m &= m - 1) {
+                        const int q = __ffs(m) - 1;
+                        const uint64_t fq = __shfl_sync(FULL, Fw, q);
+                        if (!ok) continue;
+                        uint64_t nbits = 0;
+                        if (J.w) {
+                            // arc lengths: relax every changed source of u into w
+                            for (uint64_t x = fq; x; x &= x - 1) {
                                 const int i = q * 64 + (__ffsll((long long)x) - 1);
                                 const uint64_t cand =
                                     (uint64_t)__ldcg(&J.lev[(int64_t)u * G + i]) + len;
                                 if (cand >= (uint64_t)kInf) continue;
                                 const uint32_t old =
                                     atomicMin(&J.lev[(int64_t)w * G + i], (uint32_t)cand);
-                                if (cand < old) imp |= 1ull << (i & 63);
+                                if (cand < old) nbits |= 1ull << (i & 63);
                             }
-                            if (imp) {
-                                atomicOr((unsigned long long *)&J.nxt[(int64_t)w * W + q],
-                                         (unsigned long long)imp);
-                                any = true;
-                            }
+                        } else {
+                            nbits = fq & ~J.vis[(int64_t)w * W + q];
                         }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < kReachMaxW; ++q) {
-                            if (q >= W) break;
-                            const uint64_t nbits = Fu[q] & ~J.vis[(int64_t)w * W + q];
-                            if (nbits) {
-                                atomicOr((unsigned long long *)&J.nxt[(int64_t)w * W + q],
-                                         (unsigned long long)nbits);
-                                any = true;
-                            }
+                        if (nbits) {
+                            atomicOr((unsigned long long *)&J.nxt[(int64_t)w * W + q],
+                                     (unsigned long long)nbits);
+                            any = true;
                         }
                     }
-                    if (any && atomicExch(&J.qstamp[w], epoch) != epoch)
-                        J.Q[nxq][atomicAdd((unsigned *)&qlen[nxq], 1u)] = w;
+                    if (any && atomicExch(&J.qstamp[w], epoch) != epoch) queue(nxq, w);
                 }
-            }
+            };
+            // Small nodes: a warp each, or several warps each while there
+            // are fewer nodes than warps.
+            const int64_t S = qn > 0 && qn < nwarps ? nwarps / qn : 1;
+            for (int64_t i = gw; i < (int64_t)qn * S; i += nwarps)
+                expand(J.Q[cur][i % qn], i / qn * 32, S * 32);
+            for (unsigned i = 0; i < bn; ++i) expand(J.QB[cur][i], gw * 32, nwarps * 32);
             if (!grid_sync(J.ctl, blockIdx.x, nb, J.timeout_ns)) return;
             // the next frontier: new bits (with arc lengths: the sources whose
-            // distance dropped), their levels, first touches
-            const unsigned qn2 = qlen[nxq];
-            for (int64_t idx = tid; idx < qn2; idx += nthr) {
-                const int32_t w = J.Q[nxq][idx];
-                bool fresh = true;
-                for (int q = 0; q < W; ++q) {
-                    const int64_t at = (int64_t)w * W + q;
-                    const uint64_t old = J.vis[at];
-                    const uint64_t nbits = J.w ? J.nxt[at] : J.nxt[at] & ~old;
-                    if (old) fresh = false;
-                    J.nxt[at] = 0;
-                    J.vis[at] = old | nbits;
-                    J.F[at] = nbits;
-                    if (!J.w)
-                        for (uint64_t x = nbits; x; x &= x - 1)
-                            J.lev[(int64_t)w * G + q * 64 + (__ffsll((long long)x) - 1)] = level;
-                }
-                if (fresh) J.TL[atomicAdd((unsigned *)&tlen[par], 1u)] = w;
+            // distance dropped), their levels, first touches; W lanes a node
+            const int64_t qn2 = qlen[nxq], all2 = qn2 + blen[nxq];
+            for (int64_t i0 = gw * NPW; i0 < all2; i0 += nwarps * NPW) {
+                const int64_t i = i0 + lane / W;
+                const bool ok = i < all2;
+                const int32_t w = ok ? (i < qn2 ? J.Q[nxq][i] : J.QB[nxq][i - qn2]) : 0;
+                const int64_t at = (int64_t)w * W + gq;
+                const uint64_t old = ok ? J.vis[at] : 0, nx = ok ? J.nxt[at] : 0;
+                const uint64_t nbits = J.w ? nx : nx & ~old;
+                const bool fresh = (__ballot_sync(FULL, old != 0) & gm) == 0;
+                if (!ok) continue;
+                if (nx) J.nxt[at] = 0;
+                if (nbits & ~old) J.vis[at] = old | nbits;
+                J.F[at] = nbits;
+                if (!J.w)
+                    for (uint64_t x = nbits; x; x &= x - 1)
+                        J.lev[(int64_t)w * G + gq * 64 + (__ffsll((long long)x) - 1)] = level;
+                if (fresh && gq == 0) J.TL[atomicAdd((unsigned *)&tlen[par], 1u)] = w;
             }
             if (tid == 0) {
                 qlen[cur] = 0;
-                atomicAdd(&rs->levels, 1ull);
+                blen[cur] = 0;
+                rs->levels += 1;
             }
             cur = nxq;
             if (!grid_sync(J.ctl, blockIdx.x, nb, J.timeout_ns)) return;
         }
-        // acceptance: each touched node takes its lowest-rank bits
+        // acceptance: each touched node takes its lowest-rank bits, W lanes a
+        // node, a lane a word
         const unsigned tn = tlen[par];
-        for (int64_t idx = tid; idx < tn; idx += nthr) {
-            const int32_t v = J.TL[idx];
+        for (int64_t i0 = gw * NPW; i0 < tn; i0 += nwarps * NPW) {
+            const int64_t i = i0 + lane / W;
+            const bool ok = i < tn;
+            const int32_t v = ok ? J.TL[i] : 0;
+            const int64_t at = (int64_t)v * W + gq;
             const int64_t rv = J.rank[v];
-            int c = J.cnt[v];
-            uint64_t ds = J.dsum[v];
-            bool done = false;
-            for (int q = 0; q < W; ++q) {
-                const int64_t at = (int64_t)v * W + q;
-                const uint64_t reached = J.vis[at];
-                uint64_t bits = reached;
-                J.vis[at] = 0;
-                J.F[at] = 0;
-                if (rv >= base && rv < base + gs && (rv - base) >> 6 == q)
-                    bits &= ~(1ull << ((rv - base) & 63));  // its own search
-                for (; bits && !done; bits &= bits - 1) {
-                    const int i = q * 64 + (__ffsll((long long)bits) - 1);
-                    if (c < J.k) {
-                        ds += J.lev[(int64_t)v * G + i];
-                        if (++c == J.k) {
-                            const int64_t t = base + i + 1;  // 1-based rank position
-                            J.T[v] = rv < base + i ? t - 1 : t;
-                        }
-                    } else {
-                        J.extra[v] = 1;  // a (k+1)-th source reached v
-                        done = true;
-                    }
+            const int c0 = J.cnt[v];
+            const uint64_t reached = ok ? J.vis[at] : 0;
+            uint64_t bits = reached;
+            if (ok && rv >= pos && rv < next) {  // its own search, if it ran
+                int lo = 0, up = gs;
+                while (lo < up) {
+                    const int mid = (lo + up) >> 1;
+                    if (s_src[mid] < (int)(rv - pos)) lo = mid + 1;
+                    else up = mid;
                 }
-                if (J.w)  // tentative distances start at infinity in every group
-                    for (uint64_t x = reached; x; x &= x - 1)
-                        J.lev[(int64_t)v * G + q * 64 + (__ffsll((long long)x) - 1)] = kInf;
+                if (lo < gs && s_src[lo] == (int)(rv - pos) && (lo >> 6) == gq)
+                    bits &= ~(1ull << (lo & 63));
             }
-            J.cnt[v] = c;
-            J.dsum[v] = ds;
+            const int pc = __popcll(bits);
+            int incl = pc;
+            for (int o = 1; o < W; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, incl, o, W);
+                if (gq >= o) incl += y;
+            }
+            const int first = c0 + incl - pc;  // samples before this word's
+            const int total = c0 + __shfl_sync(FULL, incl, g0 + W - 1);
+            int take = J.k - first;
+            take = take < 0 ? 0 : take > pc ? pc : take;
+            unsigned long long ds = 0;
+            uint64_t x = bits;
+            for (int a = 0; a < take; ++a, x &= x - 1) {
+                const int bit = gq * 64 + (__ffsll((long long)x) - 1);
+                ds += __ldcg(&J.lev[(int64_t)v * G + bit]);
+                if (first + a + 1 == J.k) {
+                    const int64_t p = pos + s_src[bit];
+                    J.T[v] = rv < p ? p : p + 1;  // 1-based, v not counted
+                }
+            }
+            for (int o = 1; o < W; o <<= 1) ds += __shfl_xor_sync(FULL, ds, o);
+            if (!ok) continue;
+            if (reached) J.vis[at] = 0;
+            J.F[at] = 0;
+            if (J.w)  // tentative distances start at infinity in every group
+                for (uint64_t y = reached; y; y &= y - 1)
+                    J.lev[(int64_t)v * G + gq * 64 + (__ffsll((long long)y) - 1)] = kInf;
+            if (gq == 0) {
+                const int c = total < J.k ? total : J.k;
+                J.cnt[v] = c;
+                J.dsum[v] += ds;
+                // a (k+1)-th source reached it: saturated from now on; k: once
+                // its own position is past
+                if (c == J.k) J.satpos[v] = total > J.k ? 0u : (uint32_t)rv + 1u;
+            }
         }
         if (tid == 0) {
             tlen[par ^ 1] = 0;  // the next group's touched list
             rs->groups += 1;
         }
         if (!grid_sync(J.ctl, blockIdx.x, nb, J.timeout_ns)) return;
-        if (tid == 0) tlen[par] = 0;  // read by every CTA before the barrier
+        par ^= 1;
     }
 }
 

@@ -9,6 +9,9 @@
 namespace ccg {
 
 constexpr int kReachMaxW = 16;  // words per node: groups of up to 1024 sources
+// Frontier nodes with more arcs are expanded by every warp of the grid (a
+// hub's row would take one warp milliseconds while the others wait).
+constexpr int kReachBigDeg = 2048;
 
 struct ReachJob {
     int64_t n;
@@ -19,7 +22,8 @@ struct ReachJob {
     const int32_t *order, *rank;  // the random order and its inverse
     // per node
     int32_t *cnt;                 // samples taken (<= k)
-    uint8_t *extra;               // a (k+1)-th source other than the node reached it
+    uint32_t *satpos;             // first order position from which the node is
+                                  // saturated (kInf: not yet known)
     uint64_t *dsum;               // sum of the samples' distances
     int64_t *T;                   // rank position of the k-th sample, mark rule
     uint32_t *qstamp;             // level stamp of the last push to the queue
@@ -28,6 +32,7 @@ struct ReachJob {
                                   // (arc lengths: tentative distance, kInf
                                   // outside a group's search)
     int32_t *Q[2], *TL;           // frontier queues, touched list (n each)
+    int32_t *QB[2];               // frontier nodes of more than kReachBigDeg arcs
     Ctl *ctl;                     // barrier counter and error code
     uint64_t timeout_ns;
 };
@@ -43,7 +48,7 @@ int reach_order(int64_t n, uint64_t seed, uint64_t *keys, uint32_t *vals, uint64
                 uint32_t *tv, int32_t *order, int32_t *rank, cudaStream_t st);
 
 // The cooperative launch over every group; the per-node state must start
-// zeroed.  Synchronises the stream; returns CC_ERR_TIMEOUT if a barrier wait
+// zeroed, satpos at kInf.  Synchronises the stream; returns CC_ERR_TIMEOUT if a barrier wait
 // ran out.
 int reach_run(const ReachJob &job, cudaStream_t st, ReachStats *stats);
 

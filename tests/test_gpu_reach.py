@@ -128,3 +128,35 @@ def test_reach_group_width_does_not_change_samples(cc, inbound):
                 assert (r[key] == ref[key]).all(), (words, key)
     finally:
         cc.cc_graph_free(g)
+
+
+def hub_edges(leaves, seed):
+    # a hub that most nodes point to and that points to some, among a sparse
+    # random directed graph: rows longer than the cooperative expansion's and
+    # the usefulness test's limits
+    rng = np.random.default_rng(seed)
+    n = leaves + 1
+    s = np.concatenate([np.arange(1, n), np.zeros(leaves // 3), rng.integers(0, n, 2 * n)])
+    d = np.concatenate([np.zeros(leaves), rng.integers(1, n, leaves // 3),
+                        rng.integers(0, n, 2 * n)])
+    return n, s.astype(np.uint32), d.astype(np.uint32)
+
+
+@pytest.mark.parametrize("words", [1, 8, 16])
+@pytest.mark.parametrize("leaves,k,inbound", [(2500, 3, False), (2500, 40, True),
+                                              (5000, 2, False), (5000, 9, True)])
+def test_reach_hubs_and_dropped_sources(cc, leaves, k, inbound, words):
+    """Most sources are dropped as useless once their neighbours are
+    saturated; the samples stay the oracle's at every group width."""
+    n, s, d = hub_edges(leaves, leaves + k)
+    g, _ = cc.cc_graph_from_edges(n, s, d, directed=True, keep_component=False)
+    try:
+        cc.cc_set_param(g, cc.CC_PARAM_REACH_WORDS, words)
+        r = cc.cc_reach_estimate(g, k, 7, inbound)
+    finally:
+        cc.cc_graph_free(g)
+    og = orc.csr_from_edges(n, s, d, directed=True, keep_component=False)
+    ref = orc.reach_from_table(orc.all_pairs(og), orc.sample_order(og.n, 7), k, inbound=inbound)
+    for key in ("count", "distsum", "T"):
+        assert np.array_equal(r[key], ref[key]), key
+    assert close(r["avg"], ref["avg"]).all() and close(r["R_hat"], ref["R_hat"]).all()
