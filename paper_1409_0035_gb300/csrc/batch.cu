@@ -550,6 +550,8 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
         j.Tlist = v.T; j.Tadj = v.Tadj; j.nT = v.nT;
         j.Hch_node = v.Hn; j.Hch_begin = v.Hb; j.nHch = v.nHch;
         j.tHn = v.Hn; j.tHb = v.Hb; j.ntH = v.nHch;
+        j.push_big = v.nM + v.nH > 0;
+        j.nadj = v.nadj;
         j.prp = v.rp; j.pcol = v.col;
         void *p[20];
         p[0] = take(n * W * 8); p[1] = take(n * W * 8); p[2] = take(n * W * 8);

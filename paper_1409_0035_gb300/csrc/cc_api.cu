@@ -71,7 +71,7 @@ struct DevBuf {
 
 // Degree classes of one CSR for the bottom-up scan.
 struct Classes {
-    DevBuf L, M, H, Hn, Hb, T, Tadj;
+    DevBuf L, M, H, Hn, Hb, T, Tadj, Nadj;
     int64_t nL = 0, nM = 0, nH = 0, nHch = 0, nT = 0;
 };
 
@@ -90,6 +90,24 @@ __global__ void k_tiny_adj(const int32_t *T, int64_t nT, const int64_t *rp, cons
         if (d > 2) a.z = col[b + 2];
         if (d > 3) a.w = col[b + 3];
         adj[t] = a;
+    }
+}
+
+// The same by node id, for the pushes of graphs whose rows are mostly that
+// short (grids, road networks); x = -2 marks a longer row.
+__global__ void k_node_adj(int64_t n, const int64_t *rp, const int32_t *col, int4 *adj)
+{
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = rp[v], d = rp[v + 1] - b;
+        int4 a = make_int4(d > kTinyMaxDeg ? -2 : -1, -1, -1, -1);
+        if (d <= kTinyMaxDeg) {
+            if (d > 0) a.x = col[b];
+            if (d > 1) a.y = col[b + 1];
+            if (d > 2) a.z = col[b + 2];
+            if (d > 3) a.w = col[b + 3];
+        }
+        adj[v] = a;
     }
 }
 
@@ -294,6 +312,12 @@ int build_classes(const std::vector<int64_t> &rp, int64_t n, Classes &c, const i
         const int64_t g = std::min<int64_t>((c.nT + 255) / 256, 152 * 32);
         k_tiny_adj<<<(int)g, 256>>>(c.T.as<int32_t>(), c.nT, drp, dcol, c.Tadj.as<int4>());
         CK(cudaGetLastError());
+        if (2 * c.nT >= n) {
+            RC(c.Nadj.ensure((size_t)n * 16));
+            k_node_adj<<<(int)std::min<int64_t>((n + 255) / 256, 152 * 32), 256>>>(
+                n, drp, dcol, c.Nadj.as<int4>());
+            CK(cudaGetLastError());
+        }
         CK(cudaDeviceSynchronize());  // estimates may run on other streams
     }
     RC(upload(c.L, L.data(), L.size() * 4));
@@ -356,6 +380,8 @@ BfsJob base_job(cc_graph *g, int W, const DevCSR &push, const DevCSR &pull)
     j.tHn = push.cls.Hn.as<int32_t>();
     j.tHb = push.cls.Hb.as<int64_t>();
     j.ntH = push.cls.nHch;
+    j.push_big = push.cls.nM + push.cls.nH > 0;
+    j.nadj = push.cls.Nadj.as<int4>();
     j.prp = pull.rp.as<int64_t>();
     j.pcol = pull.col.as<int32_t>();
     j.Llist = csr.cls.L.as<int32_t>();
@@ -559,18 +585,18 @@ void free_graph(cc_graph *g)
     if (g->borrowed) {  // drop the borrowed CSR pointers unfreed
         DevBuf *csr[] = {&g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
                          &g->lw_perm, &g->lw_iperm, &g->fw.cls.L, &g->fw.cls.M,
-                         &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj,
+                         &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
                      &g->rv.rp, &g->rv.col,
                          &g->rv.w, &g->rv.cls.L, &g->rv.cls.M, &g->rv.cls.H, &g->rv.cls.Hn,
-                         &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj};
+                         &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj, &g->rv.cls.Nadj};
         for (DevBuf *b : csr) { b->p = nullptr; b->cap = 0; }
     }
     DevBuf *all[] = {&g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
                      &g->lw_perm, &g->lw_iperm, &g->lw_src, &g->fw.cls.L, &g->fw.cls.M,
-                     &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj,
+                     &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
                      &g->rv.rp, &g->rv.col,
                      &g->rv.w, &g->rv.cls.L, &g->rv.cls.M, &g->rv.cls.H, &g->rv.cls.Hn,
-                     &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1,
+                     &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj, &g->rv.cls.Nadj, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1,
                      &g->T, &g->tflag, &g->sidx, &g->sum2, &g->pivot, &g->delta, &g->lc2,
                      &g->Lmask, &g->hp, &g->dcc, &g->hist, &g->TN, &g->TS, &g->Ssamp,
                      &g->maxd, &g->sources, &g->npartial, &g->ctl, &g->shat, &g->clo,
@@ -1378,7 +1404,7 @@ int ccg::graph_borrow(cc_graph_t dst, cc_graph_t src)
         Classes &c = d ? dst->rv.cls : dst->fw.cls;
         const Classes &s = d ? src->rv.cls : src->fw.cls;
         cp(c.L, s.L); cp(c.M, s.M); cp(c.H, s.H); cp(c.Hn, s.Hn); cp(c.Hb, s.Hb);
-        cp(c.T, s.T); cp(c.Tadj, s.Tadj);
+        cp(c.T, s.T); cp(c.Tadj, s.Tadj); cp(c.Nadj, s.Nadj);
         c.nL = s.nL; c.nM = s.nM; c.nH = s.nH; c.nHch = s.nHch; c.nT = s.nT;
     }
     dst->alpha = src->alpha;
@@ -1461,6 +1487,7 @@ int ccg::graph_view(cc_graph_t g, GraphView *v)
     v->L = g->fw.cls.L.as<int32_t>();
     v->T = g->fw.cls.T.as<int32_t>();
     v->Tadj = g->fw.cls.Tadj.as<int4>();
+    v->nadj = g->fw.cls.Nadj.as<int4>();
     v->nT = g->fw.cls.nT;
     v->M = g->fw.cls.M.as<int32_t>();
     v->H = g->fw.cls.H.as<int32_t>();

@@ -108,6 +108,10 @@ struct BfsJob {
     const int32_t *tHn;
     const int64_t *tHb;
     int64_t ntH;
+    int push_big;           // the push CSR may hold rows longer than kLightMaxDeg
+    // Inline entries of the push CSR by node id (null: none kept): the row
+    // padded with -1, or x = -2 for a row of more than four entries.
+    const int4 *nadj;
     const int64_t *prp;
     const int32_t *pcol;
     int k;                  // sources in this pass
@@ -182,7 +186,7 @@ struct GraphView {
     const int64_t *rp;
     const int32_t *col;
     const int32_t *L, *M, *H, *Hn, *T;
-    const int4 *Tadj;
+    const int4 *Tadj, *nadj;
     const int64_t *Hb;
     int64_t nL, nM, nH, nHch, nT;
     int alpha;

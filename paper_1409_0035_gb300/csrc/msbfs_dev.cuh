@@ -128,15 +128,15 @@ __device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, int v, uint6
         dl = J.delta[v];
         bf = J.bflag[v];  // bit 0: the band row is cleared; bit 1: lc2 holds sums
     }
-    // Frontier and visited words are written only when new bits arrive.  A
-    // frontier word left unwritten keeps bits of an older level of the same
-    // parity; each such source reached every neighbour one level after this
-    // node, so those bits are already in the neighbours' visited words and
-    // are masked off wherever the word is read.
-    if (nw) {
-        Fout[vw] = nw;
-        J.vis[vw] = vis | nw;
-    }
+    // A node that gained bits gets its whole frontier row written, empty
+    // words too: a top-down level pushes every set bit of its queued nodes,
+    // and words left over from an older level made it push 3.5 times the
+    // bits on a grid.  Rows of other nodes keep bits of an older level of the
+    // same parity; each such source reached every neighbour one level after
+    // the node, so bottom-up scans, which do read them, mask them off by the
+    // neighbours' visited words.
+    if (fresh) Fout[vw] = nw;
+    if (nw) J.vis[vw] = vis | nw;
     const bool had =
         ((__ballot_sync(FULL, (vis & ~pad_mask(J.k, w)) != 0ull) >> g0) & GM) != 0u;
     // A node that gained bits was not complete before.
@@ -616,35 +616,83 @@ __device__ __forceinline__ void td_push(const BfsJob &J, const int32_t *__restri
     A.words += wl;
 }
 
-// Top-down push of one low-degree frontier node by its lane group: lane w
-// pushes word f (its word w) to the `len` entries of `row`, kUnroll entries
-// per step (the column indices are the same for the group's lanes and load
-// as one broadcast).  Same effect as td_push.
+// Lanes that push one frontier node of at most kLightMaxDeg entries.
 template <int W>
-__device__ __forceinline__ void td_push_lane(const BfsJob &J, const int32_t *__restrict__ row,
-                                             int len, uint64_t f, int w, LevelCtl *C,
-                                             int32_t *Tout, LaneAcc &A, const Stage &stage, unsigned lv)
+constexpr int kPushLanes = W < 4 ? 4 : W;
+
+// Top-down push of low-degree frontier nodes, kPushLanes<W> lanes each (u:
+// the group's node, or -1): lane j takes the node's entries j, j + lanes, ...
+// and pushes the words with bits, two at a time, so that a grid node's four
+// entries take one chain of dependent accesses (its row or inline entries
+// and frontier words, the neighbour's visited word, the OR into its scratch
+// word, its touched stamp) with every access of a step in flight together.
+// Same effect as td_push; called by the whole warp.
+template <int W>
+__device__ __forceinline__ void td_push_group(const BfsJob &J, const uint64_t *Fin, int u,
+                                              LevelCtl *C, int32_t *Tout, LaneAcc &A,
+                                              const Stage &stage, unsigned lv)
 {
-    unsigned wl = 0;
-    for (int x = 0; x < len; x += kUnroll) {
-        int vv[kUnroll];
-        load_row<kUnroll>(row, x, len, 1, vv);
-        uint64_t vs[kUnroll];
-#pragma unroll
-        for (int q = 0; q < kUnroll; ++q)
-            vs[q] = vv[q] >= 0 ? J.vis[(int64_t)vv[q] * W + w] : ~0ull;
-#pragma unroll
-        for (int q = 0; q < kUnroll; ++q) {
-            if (vv[q] < 0) continue;
-            const int v = vv[q];
-            wl += 1;
-            const uint64_t nbits = f & ~vs[q];
-            if (!nbits) continue;
-            const uint64_t old =
-                atomicOr((unsigned long long *)&J.nxt[(int64_t)v * W + w], nbits);
-            if (old == 0ull && atomicExch(&J.tflag[v], lv) != lv)
-                stage_push(stage, v, Tout, &C->tlen);
+    constexpr int GL = kPushLanes<W>;
+    constexpr unsigned WM = W == 32 ? FULL : (1u << (W & 31)) - 1u;
+    const int lane = threadIdx.x & 31;
+    const int j = lane & (GL - 1), g0 = lane & ~(GL - 1);
+    uint64_t f = 0;
+    int len = 0, v = -1;
+    const int32_t *row = nullptr;
+    if (u >= 0) {
+        if (j < W) f = Fin[(int64_t)u * W + j];
+        int4 a = make_int4(-2, -1, -1, -1);
+        if (J.nadj) a = J.nadj[u];
+        if (a.x != -2) {
+            v = j == 0 ? a.x : j == 1 ? a.y : j == 2 ? a.z : j == 3 ? a.w : -1;
+            len = 1;
+        } else {
+            const int64_t b = J.rp[u], e = J.rp[u + 1];
+            if (e - b <= kLightMaxDeg) {
+                len = (int)(e - b);
+                row = J.col + b;
+                if (j < len) v = __ldcs(row + j);
+            }
         }
+    }
+    const unsigned words = (__ballot_sync(FULL, f != 0ull) >> g0) & WM;
+    const int steps = __reduce_max_sync(FULL, (unsigned)((len + GL - 1) / GL));
+    const int turns = __reduce_max_sync(FULL, (unsigned)(__popc(words) + 1) / 2);
+    unsigned wl = 0;
+    for (int x = 0; x < steps; ++x) {
+        const int nx = j + (x + 1) * GL;
+        const int vnext = row && nx < len ? __ldcs(row + nx) : -1;
+        unsigned m = words;
+        for (int t = 0; t < turns; ++t) {
+            uint64_t nb[2], old[2];
+            int ww[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                ww[q] = m ? __ffs(m) - 1 : 0;
+                const uint64_t fw = __shfl_sync(FULL, f, g0 + ww[q]);
+                nb[q] = m && v >= 0 ? fw : 0ull;
+                m &= m - 1;
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (nb[q]) {
+                    wl += 1;
+                    nb[q] &= ~J.vis[(int64_t)v * W + ww[q]];
+                }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                old[q] = ~0ull;
+                if (nb[q])
+                    old[q] = atomicOr((unsigned long long *)&J.nxt[(int64_t)v * W + ww[q]],
+                                      (unsigned long long)nb[q]);
+            }
+            // first bits in a word: with one word per node that alone tells
+            // the node's first toucher
+            if (old[0] == 0ull || old[1] == 0ull)
+                if (W == 1 || atomicExch(&J.tflag[v], lv) != lv)
+                    stage_push(stage, v, Tout, &C->tlen);
+        }
+        v = vnext;
     }
     A.words += wl;
 }
@@ -836,38 +884,31 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
             // where a warp per node took several (heavy nodes pushed by
             // their chunk tasks below).
             const bool few = qn <= nwarps;
-            const int64_t S = few && qn > 0 ? nwarps / qn : 1;
-            for (int64_t t = gwarp; few && t < qn * S; t += nwarps) {
+            const int S = few && qn > 0 ? (int)nwarps / (int)qn : 1;
+            for (int t = (int)gwarp; few && J.push_big && t < (int)qn * S; t += (int)nwarps) {
                 const int u = Qin[t / S];
                 const int64_t part = t % S;
                 const int64_t b = rp[u], e = rp[u + 1];
-                if (J.ntH > 0 && e - b > kMediumMaxDeg) continue;
+                if (e - b <= kLightMaxDeg || (J.ntH > 0 && e - b > kMediumMaxDeg)) continue;
                 const int64_t per = (e - b + S - 1) / S;
                 const int64_t bb = b + part * per, ee = min(e, bb + per);
                 if (bb >= ee) continue;
                 const uint64_t f = Fin[(int64_t)u * W + w];
                 td_push<W>(J, col, f, bb, ee, C, Tout, A, stage, (unsigned)l);
             }
-            // Otherwise nodes of at most kLightMaxDeg entries: a lane group
-            // each, NPW per warp (a grid's frontier node has 4 entries: a
-            // warp each would leave most lanes idle and chain one node after
-            // another).
-            for (int64_t t0 = gwarp * NPW; !few && t0 < qn; t0 += nwarps * NPW) {
-                const int64_t t = t0 + grp;
-                if (t < qn) {
-                    const int u = Qin[t];
-                    const int64_t b = rp[u], e = rp[u + 1];
-                    if (e - b <= kLightMaxDeg) {
-                        const uint64_t f = Fin[(int64_t)u * W + w];
-                        if (f) td_push_lane<W>(J, col + b, (int)(e - b), f, w, C, Tout, A, stage, (unsigned)l);
-                    }
-                }
+            // Nodes of at most kLightMaxDeg entries: a lane group each (a
+            // grid's frontier node has 4 entries: a warp each would leave
+            // most lanes idle and chain one node after another).
+            constexpr int NPL = 32 / kPushLanes<W>;
+            for (int64_t t0 = gwarp * NPL; t0 < qn; t0 += nwarps * NPL) {
+                const int64_t t = t0 + lane / kPushLanes<W>;
+                td_push_group<W>(J, Fin, t < qn ? Qin[t] : -1, C, Tout, A, stage, (unsigned)l);
             }
             // Larger nodes: a warp tests its queue entries (every nwarps-th,
             // so that consecutive ones go to different warps) 32 at a time
             // by ballot and pushes each larger one whole; when the graph has
             // chunk tasks, a heavy node's list is pushed by them.
-            for (int64_t j0 = 0; !few && gwarp + j0 * nwarps < qn; j0 += 32) {
+            for (int64_t j0 = 0; !few && J.push_big && gwarp + j0 * nwarps < qn; j0 += 32) {
                 const int64_t t = gwarp + (j0 + lane) * nwarps;
                 int u = 0;
                 int64_t b = 0, e = 0;

@@ -237,6 +237,7 @@ extern "C" int cc_sampling_pivots_noalloc(int64_t n, const int64_t *d_row_ptr,
     j.sidx = sidx;
     j.Llist = Llist;
     j.nL = n;
+    j.push_big = 1;
     j.vis = vis; j.F0 = F0; j.F1 = F1; j.nxt = nxt;
     j.Q0 = Q0; j.Q1 = Q1; j.T = T; j.tflag = tflag;
     j.AL0 = AL0; j.AL1 = AL1;

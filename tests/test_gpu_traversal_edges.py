@@ -62,3 +62,36 @@ def test_estimate_at_the_edges(cc, name):
     for key in ("s_hat", "closeness"):
         rel = np.abs(r[key] - want[key]) / np.abs(want[key])
         assert rel.max() <= RTOL, key
+
+
+def ladder(n):
+    # rungs every third step, every twentieth node with a few extra leaves:
+    # rows of 2 to 7 entries around the four that are kept inline by node
+    a = np.arange(n - 1)
+    rung = np.arange(0, n, 3)
+    hub = np.repeat(np.arange(0, n, 20), 4)
+    leaf = 2 * n + np.arange(hub.size)
+    s = np.concatenate([a, n + a, rung, hub])
+    d = np.concatenate([a + 1, n + a + 1, n + rung, leaf])
+    return 2 * n + hub.size, s.astype(np.uint32), d.astype(np.uint32)
+
+
+@pytest.mark.parametrize("k", [1, 64, 65, 200, 500, 1000, 1500])
+@pytest.mark.parametrize("name", ["ladder", "grid"])
+def test_narrow_frontiers_at_every_width(cc, name, k):
+    """Top-down levels of few bits per word at 1 to 32 words per node, rows on
+    both sides of the inline limit."""
+    n, s, d = ladder(900) if name == "ladder" else synth.grid_edges(59, 41)
+    g, _ = cc.cc_graph_from_edges(n, s, d)
+    try:
+        og = orc.csr_from_edges(n, s, d)
+        C = cc.cc_sample_choose(g, k, 9)
+        o = cc.cc_opts_default(k)
+        r = cc.cc_estimate(g, C, o)
+        stats = cc.cc_last_pass_stats(g)
+    finally:
+        cc.cc_graph_free(g)
+    assert stats["td_levels"] > 0
+    want = orc.estimate(og, C, eps=(o.eps_num, o.eps_den))
+    for key in ("pivot", "delta", "sum", "S_samp", "delta_cc", "hyb"):
+        assert np.array_equal(r[key], want[key]), key
