@@ -87,6 +87,7 @@ def test_narrow_frontiers_at_every_width(cc, name, k):
         og = orc.csr_from_edges(n, s, d)
         C = cc.cc_sample_choose(g, k, 9)
         o = cc.cc_opts_default(k)
+        cc.cc_set_tuning(g, 1)  # top-down for as long as a frontier allows it
         r = cc.cc_estimate(g, C, o)
         stats = cc.cc_last_pass_stats(g)
     finally:
