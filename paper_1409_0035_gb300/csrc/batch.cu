@@ -57,6 +57,7 @@ struct BatchJob {
     Ctl *ctl1, *ctl2;
     double *shat, *clo;  // 4 x n each
     uint64_t *hyb;       // n x 6
+    uint64_t *ssum;      // n
     int *status;
 };
 
@@ -131,7 +132,7 @@ __device__ void run_job(const BatchJob &B, unsigned rank, unsigned size, Ctl *ba
         fa.clo[e] = B.clo + (int64_t)e * n;
     }
     fa.hyb_int = B.want_hybrid ? B.hyb : nullptr;
-    fa.sample_sum = nullptr;
+    fa.sample_sum = B.ssum;
     d_finalize(fa, gtid, gthreads);
     if (!grid_sync(bar, rank, size, to)) return;
     if (gtid == 0) *B.status = CC_OK;
@@ -607,8 +608,9 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
         J.shat = (double *)take((size_t)n * 8 * CC_NUM_EST);
         J.clo = (double *)take((size_t)n * 8 * CC_NUM_EST);
         J.hyb = (uint64_t *)take((size_t)n * 48);
+        J.ssum = (uint64_t *)take((size_t)n * 8);
         if (!J.hist || !J.TN || !J.TS || !J.Ssamp || !J.maxd || !J.hp || !J.Lmask ||
-            !J.lc2 || !J.npartial || !J.shat || !J.clo || !J.hyb)
+            !J.lc2 || !J.npartial || !J.shat || !J.clo || !J.hyb || !J.ssum)
             return CC_ERR_OOM;
         j.hist = J.hist;
         j.hist_cap = cap;
@@ -782,24 +784,23 @@ int cc_batch_result(cc_batch_t b, int32_t i, const cc_out *out, int32_t device_o
     const int64_t n = b->n[i];
     const int k = b->k[i];
     const cudaMemcpyKind kind = device_outputs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    // The copies are queued together and waited for once.
+    auto put = [&](void *dst, const void *src, size_t bytes) {
+        return !dst || cudaMemcpyAsync(dst, src, bytes, kind, 0) == cudaSuccess;
+    };
+    bool ok = true;
     for (int e = 0; e < CC_NUM_EST; ++e) {
-        if (out->s_hat[e]) B_CK(cudaMemcpy(out->s_hat[e], J.shat + (int64_t)e * n, n * 8, kind));
-        if (out->closeness[e])
-            B_CK(cudaMemcpy(out->closeness[e], J.clo + (int64_t)e * n, n * 8, kind));
+        ok = ok && put(out->s_hat[e], J.shat + (int64_t)e * n, n * 8);
+        ok = ok && put(out->closeness[e], J.clo + (int64_t)e * n, n * 8);
     }
-    if (out->pivot) B_CK(cudaMemcpy(out->pivot, J.j.pivot, n * 4, kind));
-    if (out->delta) B_CK(cudaMemcpy(out->delta, J.j.delta, n * 4, kind));
-    if (out->hyb_int) B_CK(cudaMemcpy(out->hyb_int, J.hyb, n * 48, kind));
-    if (out->S_sampled) B_CK(cudaMemcpy(out->S_sampled, J.Ssamp, (size_t)k * 8, kind));
-    if (out->delta_cc) B_CK(cudaMemcpy(out->delta_cc, J.j.dcc, (size_t)k * k * 4, kind));
-    if (out->sample_sum) {
-        std::vector<uint64_t> s2((size_t)n * 2);
-        B_CK(cudaMemcpy(s2.data(), J.j.sum2, n * 16, cudaMemcpyDeviceToHost));
-        std::vector<uint64_t> s(n);
-        for (int64_t v = 0; v < n; ++v) s[v] = s2[2 * v];
-        B_CK(cudaMemcpy(out->sample_sum, s.data(), n * 8,
-                        device_outputs ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost));
-    }
+    ok = ok && put(out->pivot, J.j.pivot, n * 4) && put(out->delta, J.j.delta, n * 4) &&
+         put(out->hyb_int, J.hyb, n * 48) && put(out->S_sampled, J.Ssamp, (size_t)k * 8) &&
+         put(out->delta_cc, J.j.dcc, (size_t)k * k * 4) &&
+         put(out->sample_sum, J.ssum, n * 8);
+    const cudaError_t e0 = cudaGetLastError();
+    if (!ok) note_cuda_error(e0, __FILE__, __LINE__);
+    B_CK(cudaStreamSynchronize(0));
+    if (!ok) return CC_ERR_CUDA;
     return CC_OK;
 }
 
