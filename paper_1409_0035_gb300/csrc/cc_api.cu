@@ -16,6 +16,7 @@
 #include "nodew.h"
 #include "reach.h"
 #include "sssp.h"
+#include "tiles.h"
 
 using namespace ccg;
 
@@ -36,6 +37,11 @@ constexpr int kReachDefaultW = 8;
 // node and source 2.65 at small widths, 3.3 at the largest; 8.7 without
 // buckets, 391 / 435 ms).
 constexpr double kDeltaMult = 96.0;
+// Tiles pay from about a thousand nodes and, on unit lengths, sixty-four
+// levels on (a level of the bit-packed search costs about 15 us, a round of
+// tiles, which goes on by twenty, about as much): MEASURE.
+constexpr int64_t kTileMinNodes = 1024;
+constexpr double kTileMinLevels = 64.0;
 constexpr double kMaxHistBytes = 4.0 * (1ull << 30);  // distance histogram cap
 
 // Bumped whenever a device buffer is (re)allocated or freed: a captured
@@ -180,6 +186,11 @@ struct cc_graph {
     DevCSR lw;
     DevBuf lw_perm, lw_iperm, lw_src;
     bool has_lw = false;
+    // Undirected graphs of short rows, cut into tiles (tiles.cu); their
+    // search's rows and queues.  on_tiles: the last first pass ran on them.
+    TileGraph tg;
+    bool has_tiles = false, on_tiles = false;
+    DevBuf t_dist, t_dirty0, t_dirty1, t_act0, t_act1, t_stamp, t_Q0, t_Q1;
     // workspace
     DevBuf vis, F0, F1, nxt, Q0, Q1, T, tflag, sidx, sum2, pivot, delta, lc2, Lmask, hp,
         dcc, hist, TN, TS, Ssamp, maxd, sources, npartial, ctl, shat, clo, hyb, ssum,
@@ -580,6 +591,28 @@ int build_locality(cc_graph *g, const std::vector<int64_t> &rp)
     return CC_OK;
 }
 
+// The same for a graph whose estimates run on tiles, when a call needs the
+// shortest-path rounds after all.
+int ensure_locality(cc_graph *g)
+{
+    if (!g->has_tiles || !g->weighted || g->has_lw || g->borrowed) return CC_OK;
+    std::vector<int64_t> rp((size_t)g->n + 1);
+    CK(cudaMemcpy(rp.data(), g->fw.rp.p, rp.size() * 8, cudaMemcpyDeviceToHost));
+    return build_locality(g, rp);
+}
+
+// Tiles of an undirected graph whose rows are short and mostly tiny
+// (tiles.cu decides whether they are local).
+int cut_tiles(cc_graph *g)
+{
+    const Classes &c = g->fw.cls;
+    if (g->directed || g->n < kTileMinNodes || c.nM + c.nH > 0 || 2 * c.nT < g->n) return CC_OK;
+    RC(tiles_build(g->n, g->arcs, g->fw.rp.as<int64_t>(), g->fw.col.as<int32_t>(),
+                   g->weighted ? g->fw.w.as<uint32_t>() : nullptr, g->tg, &g->has_tiles, 0));
+    CK(cudaDeviceSynchronize());  // estimates may run on other streams
+    return CC_OK;
+}
+
 void free_graph(cc_graph *g)
 {
     if (g->borrowed) {  // drop the borrowed CSR pointers unfreed
@@ -591,7 +624,9 @@ void free_graph(cc_graph *g)
                          &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj, &g->rv.cls.Nadj};
         for (DevBuf *b : csr) { b->p = nullptr; b->cap = 0; }
     }
-    DevBuf *all[] = {&g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
+    if (!g->borrowed) tiles_free(g->tg);
+    DevBuf *all[] = {&g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1, &g->t_stamp,
+                     &g->t_Q0, &g->t_Q1, &g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
                      &g->lw_perm, &g->lw_iperm, &g->lw_src, &g->fw.cls.L, &g->fw.cls.M,
                      &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
                      &g->rv.rp, &g->rv.col,
@@ -977,6 +1012,7 @@ int chunked_pass1(cc_graph *g, int k, cudaStream_t st, const NwJob *nw = nullptr
 {
     const int64_t n = g->n;
     const int W = pow2_words(k);
+    RC(ensure_locality(g));
     const int cw = chunk_width(g, k);
     g->cw = cw;
     // Keep every chunk's rows when they fit in a third of the free memory:
@@ -1115,12 +1151,200 @@ int chunked_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
     return CC_OK;
 }
 
+// Whether an estimate of k sources runs on the graph's tiles: not under a
+// setting of the search they replace (the direction switch or the two-pass
+// form on unit lengths, the bucket width with arc lengths), not in a server
+// slot (its launches are capped and its footprint is admitted for the other
+// path), and while the labels fit a third of the memory that is free or
+// already held by them.
+bool use_tiles(cc_graph *g, int64_t k)
+{
+    if (!g->has_tiles || g->borrowed || g->max_ctas > 0) return false;
+    if (g->weighted ? g->sssp_delta != 0
+                    : g->band_off || g->alpha != 0 || g->tg.levels < kTileMinLevels)
+        return false;
+    const double need = (double)k * (double)g->tg.slots * 4.25;
+    if ((double)g->t_dist.cap + (double)g->t_dirty0.cap * 2.0 >= need) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return need <= ((double)free_b + (double)g->t_dist.cap) / 3.0;
+}
+
+TileReduce tile_reduce_job(cc_graph *g, int k)
+{
+    TileReduce r;
+    std::memset((void *)&r, 0, sizeof(r));
+    r.g = g->tg;
+    r.k = k;
+    r.W = pow2_words(k);
+    r.dist = g->t_dist.as<uint32_t>();
+    r.sources = g->sources.as<int32_t>();
+    r.sidx = g->sidx.as<int32_t>();
+    r.sum2 = g->sum2.as<uint64_t>();
+    r.pivot = g->pivot.as<int32_t>();
+    r.delta = g->delta.as<uint32_t>();
+    r.dcc = g->dcc.as<uint32_t>();
+    r.S_samp = g->Ssamp.as<unsigned long long>();
+    r.dmax = g->dmax.as<unsigned long long>();
+    r.err = g->errflag.as<int>();
+    return r;
+}
+
+// First pass on tiles: the labels of all k sources, reduced into sums,
+// pivots, Delta, delta_cc and the exact S of the sampled nodes.  Returns 1
+// when a label came near 2^32: the shortest-path rounds then decide.
+int tiled_pass1(cc_graph *g, int k, cudaStream_t st)
+{
+    const int64_t n = g->n, slots = g->tg.slots;
+    const size_t units = (size_t)g->tg.tiles * ((k + 31) / 32);
+    RC(g->t_dist.ensure((size_t)k * slots * 4));
+    RC(g->t_dirty0.ensure((size_t)k * slots / 8));
+    RC(g->t_dirty1.ensure((size_t)k * slots / 8));
+    RC(g->t_act0.ensure(units * 4));
+    RC(g->t_act1.ensure(units * 4));
+    RC(g->t_stamp.ensure(units * 4));
+    RC(g->t_Q0.ensure(units * 4));
+    RC(g->t_Q1.ensure(units * 4));
+    RC(g->sum2.ensure(n * 16));
+    RC(g->dmax.ensure(8));
+    RC(g->errflag.ensure(4));
+    TileJob j;
+    std::memset((void *)&j, 0, sizeof(j));
+    j.g = g->tg;
+    j.k = k;
+    j.kw = (k + 31) / 32;
+    j.uw = tile_unit_words(g->tg, k);
+    j.ku = (j.kw + j.uw - 1) / j.uw;
+    j.stamp = g->t_stamp.as<uint32_t>();
+    j.sources = g->sources.as<int32_t>();
+    j.dist = g->t_dist.as<uint32_t>();
+    j.dirty[0] = g->t_dirty0.as<uint32_t>();
+    j.dirty[1] = g->t_dirty1.as<uint32_t>();
+    j.act[0] = g->t_act0.as<uint32_t>();
+    j.act[1] = g->t_act1.as<uint32_t>();
+    j.Q[0] = g->t_Q0.as<int32_t>();
+    j.Q[1] = g->t_Q1.as<int32_t>();
+    j.ctl = g->ctl.as<Ctl>();
+    j.timeout_ns = kTimeoutNs;
+    if (!g->ev0) {
+        CK(cudaEventCreate(&g->ev0));
+        CK(cudaEventCreate(&g->ev1));
+    }
+    CK(cudaMemsetAsync(g->ctl.p, 0, sizeof(Ctl), st));
+    CK(cudaMemsetAsync(g->Ssamp.p, 0, (size_t)k * 8, st));
+    CK(cudaMemsetAsync(g->dmax.p, 0, 8, st));
+    CK(cudaMemsetAsync(g->errflag.p, 0, 4, st));
+    CK(cudaEventRecord(g->ev0, st));
+    RC(launch_tiles(j, st));
+    CK(cudaEventRecord(g->ev1, st));
+    CK(cudaMemcpyAsync(&g->last, g->ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
+    run_tiles_reduce1(tile_reduce_job(g, k), st);
+    CK(cudaGetLastError());
+    unsigned long long dmax = 0;
+    int err = 0;
+    CK(cudaMemcpyAsync(&dmax, g->dmax.p, 8, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(&err, g->errflag.p, 4, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    float ms = 0.f;
+    CK(cudaEventElapsedTime(&ms, g->ev0, g->ev1));
+    g->call_launches += 1;
+    g->call_kernels += 4;
+    g->call_ms += ms;
+    // the labels written once, and per label carried on its word and its
+    // node's arcs (offsets, heads and lengths)
+    g->call_bytes += (double)n * k * 4.0 + (double)g->last.words * 12.0;
+    if (g->last.err < 0) return g->last.err;
+    if (g->last.band_ovf) return 1;
+    if (err) return err;
+    g->dist_max = (int64_t)dmax;
+    g->D1 = (int64_t)dmax;
+    return CC_OK;
+}
+
+// The hybrid part for eps = a/b after tiled_pass1.
+int tiled_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
+{
+    const int64_t n = g->n;
+    const int W = pow2_words(k);
+    const int64_t D = g->D1, hs = (D + 64) / 64 * 64;
+    if ((double)(D + 1) * k * 4.0 > (double)kMaxHistBytes) return CC_ERR_TOO_LARGE;
+    // Sums of squared distances (LCsumSq) stay in 64 bits.
+    if ((double)D * (double)D * (double)k >= 1.8e19) return CC_ERR_TOO_LARGE;
+    const size_t blocks = (size_t)k * (hs / 64 + 1) * 8;
+    RC(g->hist.ensure((size_t)hs * k * 4));
+    RC(g->TN.ensure(blocks));
+    RC(g->TS.ensure(blocks));
+    RC(g->maxd.ensure((size_t)k * 4));
+    RC(g->hp.ensure((size_t)n * sizeof(HybPrep)));
+    RC(g->npartial.ensure(8));
+    RC(g->Lmask.ensure((size_t)n * W * 8));
+    RC(g->lc2.ensure(n * 16));
+    CK(cudaMemsetAsync(g->npartial.p, 0, 8, st));
+    CK(cudaMemsetAsync(g->hist.p, 0, (size_t)hs * k * 4, st));
+    run_maxdelta(g->dcc.as<uint32_t>(), k, g->maxd.as<uint32_t>(), st);
+    SqPrep sq{nullptr};
+    if (g->sq) {
+        RC(prepare_sq(g, k, st));
+        sq.flag = g->sqflag.as<uint8_t>();
+    }
+    run_hyb_prep(1, n, k, DevCount{nullptr, D}, D + 1, a, b, g->sidx.as<int32_t>(),
+                 g->pivot.as<int32_t>(), g->delta.as<uint32_t>(), g->dcc.as<uint32_t>(),
+                 g->maxd.as<uint32_t>(), nullptr, nullptr, g->hp.as<HybPrep>(),
+                 g->npartial.as<unsigned>(), sq, st);
+    run_lmask(n, W, k, g->sidx.as<int32_t>(), g->pivot.as<int32_t>(), g->dcc.as<uint32_t>(),
+              g->hp.as<HybPrep>(), g->Lmask.as<uint64_t>(), nullptr, st);
+    TileReduce r = tile_reduce_job(g, k);
+    r.D = D;
+    r.hs = hs;
+    r.hist = g->hist.as<uint32_t>();
+    r.TN = g->TN.as<uint64_t>();
+    r.TS = g->TS.as<uint64_t>();
+    r.hp = g->hp.as<HybPrep>();
+    r.Lmask = g->Lmask.as<uint64_t>();
+    r.lc2 = g->lc2.as<uint64_t>();
+    if (g->sq) {
+        r.sqflag = g->sqflag.as<uint8_t>();
+        r.istar = g->istar.as<int32_t>();
+        r.hcse = g->hcse.as<uint64_t>();
+        r.fdist = g->fdist.as<uint32_t>();
+    }
+    run_tiles_reduce2(r, st);
+    CK(cudaGetLastError());
+    g->call_kernels += 9;
+    return CC_OK;
+}
+
+// First pass and hybrid part on distance rows: tiles where the graph has
+// them (g->on_tiles tells which ran last), else chunks.
+int rows_pass1(cc_graph *g, int k, cudaStream_t st)
+{
+    g->on_tiles = use_tiles(g, k);
+    if (g->on_tiles) {
+        const int rc = tiled_pass1(g, k, st);
+        if (rc != 1) return rc;
+        g->on_tiles = false;
+    }
+    return chunked_pass1(g, k, st);
+}
+
+int rows_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
+{
+    return g->on_tiles ? tiled_hybrid(g, k, a, b, st) : chunked_hybrid(g, k, a, b, st);
+}
+
 int estimate_chunked(cc_graph *g, int k, const cc_opts *opts, cudaStream_t st)
 {
-    RC(chunked_pass1(g, k, st));
+    RC(rows_pass1(g, k, st));
     if (!opts->want_hybrid) return CC_OK;
-    return chunked_hybrid(g, k, opts->eps_num, opts->eps_den, st);
+    return rows_hybrid(g, k, opts->eps_num, opts->eps_den, st);
 }
+
+// Whether an estimate's first pass leaves distance rows (arc lengths, round
+// trips, tiles) rather than the bit-packed pass's state.
+bool on_rows(cc_graph *g) { return g->weighted || g->directed || g->on_tiles; }
 
 // Finalise into device buffers (or straight into device outputs) and copy.
 // Arguments of the finalisation (host only: buffers sized, no stream work).
@@ -1172,7 +1396,7 @@ int prepare_finalize(cc_graph *g, int k, bool hyb, const cc_opts *opts, const cc
     // power-of-two k, and tables of the pivoting estimators over (c, Delta).
     if ((k & (k - 1)) == 0) fa.inv_k = 1.0 / (double)k;
     {
-        const bool chunked = g->weighted || g->directed;
+        const bool chunked = on_rows(g);
         const int64_t ts = std::min<int64_t>(chunked ? g->D1 + 1 : g->hist_cap, 256);
         RC(g->pt_clo1.ensure((size_t)k * 16));
         RC(g->pt_est2.ensure((size_t)k * ts * 8));
@@ -1211,7 +1435,7 @@ int prepare_finalize(cc_graph *g, int k, bool hyb, const cc_opts *opts, const cc
 // The estimator tables and the finalisation kernel (stream work only).
 void enqueue_finalize(cc_graph *g, int k, const FinalizeArgs &fa, cudaStream_t st)
 {
-    const bool chunked = g->weighted || g->directed;
+    const bool chunked = on_rows(g);
     const DevCount D = chunked ? DevCount{nullptr, g->D1} : DevCount{&g->ctl.as<Ctl>()->levels, 0};
     run_pivot_tables(g->n, k, g->Ssamp.as<uint64_t>(), D, fa.tstride, g->pt_clo1.as<double>(),
                      g->pt_est2.as<double>(), g->pt_clo2.as<double>(), fa.inv_k, fa.c0len,
@@ -1418,9 +1642,12 @@ int ccg::graph_borrow(cc_graph_t dst, cc_graph_t src)
 
 cc_graph_t ccg::graph_new_empty() { return new (std::nothrow) cc_graph(); }
 
+int ccg::graph_ready_to_borrow(cc_graph_t g) { return ensure_locality(g); }
+
 size_t ccg::graph_workspace_bytes(cc_graph_t g)
 {
-    const DevBuf *ws[] = {&g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1, &g->T, &g->tflag,
+    const DevBuf *ws[] = {&g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1,
+                          &g->t_stamp, &g->t_Q0, &g->t_Q1, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1, &g->T, &g->tflag,
                           &g->sidx, &g->sum2, &g->pivot, &g->delta, &g->lc2, &g->Lmask, &g->hp,
                           &g->dcc, &g->hist, &g->TN, &g->TS, &g->Ssamp, &g->maxd, &g->sources,
                           &g->npartial, &g->ctl, &g->shat, &g->clo, &g->hyb, &g->ssum,
@@ -1559,7 +1786,8 @@ int cc_graph_from_edges(int64_t n, int64_t m, const uint32_t *src, const uint32_
         DeviceCSR d;
         rc = build_csr_device(n, m, src, dst, w, keep_component != 0, d);
         if (rc == CC_OK) rc = adopt_device_csr(g, d);
-        if (rc == CC_OK && w) rc = build_locality(g, d.rp_host);
+        if (rc == CC_OK) rc = cut_tiles(g);
+        if (rc == CC_OK && w && !g->has_tiles) rc = build_locality(g, d.rp_host);
         if (d.rp) cudaFree(d.rp);
         if (d.col) cudaFree(d.col);
         if (d.w) cudaFree(d.w);
@@ -1769,7 +1997,9 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     CK(cudaMemcpyAsync(g->sources.p, sample, (size_t)k * 4, cudaMemcpyHostToDevice, st));
     const bool hyb = opts->want_hybrid != 0;
     g->sq = hyb && out->sq_err != nullptr;
-    const bool chunked = g->weighted || g->directed;
+    g->on_tiles = use_tiles(g, k);
+    const bool chunked = on_rows(g);
+    if (g->on_tiles) g->eg.replayed = 0;
     int rc = CC_OK;
     if (chunked) {
         run_fill_i32(g->sidx.as<int32_t>(), n, -1, st);
@@ -1834,9 +2064,10 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     run_fill_i32(g->sidx.as<int32_t>(), n, -1, st);
     run_scatter_sidx(g->sidx.as<int32_t>(), g->sources.as<int32_t>(), k, st);
     g->call_kernels += 2;
-    const bool chunked = g->weighted || g->directed;
+    g->on_tiles = use_tiles(g, k);
+    const bool chunked = on_rows(g);
     if (chunked) {
-        RC(chunked_pass1(g, k, st));
+        RC(rows_pass1(g, k, st));
     } else {
         for (;;) {
             RC(bfs_pass1(g, k, st));
@@ -1850,7 +2081,7 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     }
     g->sq = true;
     for (int e = 0; e < n_eps; ++e) {
-        RC(chunked ? chunked_hybrid(g, k, eps_num[e], eps_den[e], st)
+        RC(chunked ? rows_hybrid(g, k, eps_num[e], eps_den[e], st)
                    : bfs_hybrid(g, k, eps_num[e], eps_den[e], st));
         if (!chunked) {
             CK(cudaStreamSynchronize(st));
@@ -1998,6 +2229,7 @@ int cc_estimate_node_weighted(cc_graph_t g, const int32_t *sample, int32_t k,
               g->nw_bsrc.as<uint32_t>(), g->nw_mu.as<uint64_t>(),
               g->nw_msum.as<unsigned long long>(), st);
     g->call_kernels += 3;
+    RC(ensure_locality(g));
     NwJob j;
     std::memset(&j, 0, sizeof(j));
     j.n = n;
@@ -2233,6 +2465,7 @@ int cc_exact(cc_graph_t g, double *closeness, uint64_t *S)
         RC(g->sum2.ensure(n * 16));
         RC(g->ctl.ensure(sizeof(Ctl)));
         RC(g->sources.ensure((size_t)n * 4));
+        RC(ensure_locality(g));
         const int cw = chunk_width(g, n);
         RC(g->distF.ensure((size_t)n * cw * 4));
         if (g->directed) RC(g->distR.ensure((size_t)n * cw * 4));

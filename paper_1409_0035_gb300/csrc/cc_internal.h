@@ -220,6 +220,9 @@ __device__ __forceinline__ uint64_t splitmix64_out(uint64_t seed, uint64_t c)
 // resident CSR of another handle per request.
 cc_graph_t graph_new_empty();
 int graph_borrow(cc_graph_t dst, cc_graph_t src);
+// Called once per graph before its first borrow: lays out what a borrowing
+// handle uses and this one may not have needed yet.
+int graph_ready_to_borrow(cc_graph_t g);
 size_t graph_workspace_bytes(cc_graph_t g);
 // Estimates from the first pass resident in g's workspace (see cc_api.cu).
 int estimate_resident(cc_graph_t g, int32_t k, const cc_opts *opts, cc_out *out);

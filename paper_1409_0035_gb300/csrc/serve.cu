@@ -254,6 +254,8 @@ int cc_server_create(int32_t ngraphs, const cc_graph_t *graphs, int32_t slots,
         int64_t n = 0;
         if (!graphs[i] || cc_graph_info(graphs[i], &n, nullptr, nullptr, nullptr) != CC_OK)
             return CC_ERR_ARG;
+        const int rc = graph_ready_to_borrow(graphs[i]);
+        if (rc != CC_OK) return rc;
         srv->graphs.push_back(graphs[i]);
         srv->n.push_back(n);
     }

@@ -1,0 +1,94 @@
+// Shortest paths on graphs of narrow frontiers, tile by tile (tiles.cu).
+#pragma once
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+#include "cc_internal.h"
+#include "estimate.h"
+
+namespace ccg {
+
+constexpr int kTileCap = 512;      // nodes of a tile at most
+constexpr int kTileMean = 256;     // nodes per cluster centre
+constexpr int kTileArcs = 2560;    // arcs inside a tile at most
+constexpr int kUnitWords = 8;      // words of 32 sources a CTA takes at once
+
+// A graph cut into tiles of neighbouring nodes.  Slots are the nodes' numbers
+// tile by tile, each tile padded to whole 32-slot words (perm = -1 there).
+struct TileGraph {
+    int64_t n = 0, slots = 0;
+    int32_t tiles = 0;
+    double levels = 0.0;                         // estimated hops across the graph
+    int32_t *perm = nullptr, *iperm = nullptr;   // slot -> node, node -> slot
+    int32_t *tb = nullptr;                       // tiles + 1: first slot of each
+    int32_t *word_tile = nullptr;                // slots / 32: the word's tile
+    uint32_t *irp = nullptr, *erp = nullptr;     // slots + 1: arcs inside, leaving the tile
+    uint16_t *icol = nullptr;                    // head's slot within the tile
+    int32_t *ecol = nullptr;                     // head's slot
+    uint32_t *iw = nullptr, *ew = nullptr;       // their lengths (null: unit lengths)
+};
+
+// Cuts an undirected CSR (rows of at most kLightMaxDeg entries; w null: unit
+// lengths) into tiles.  *ok = false, and nothing kept, when the tiles would
+// not be local: see tiles.cu.
+int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
+                const uint32_t *w, TileGraph &out, bool *ok, cudaStream_t st);
+void tiles_free(TileGraph &g);
+
+struct TileJob {
+    TileGraph g;
+    int k;                      // sources
+    int kw;                     // words of 32 sources
+    int uw, ku;                 // words per unit of work (at most kUnitWords), units per tile
+    const int32_t *sources;     // k node ids
+    uint32_t *dist;             // k x slots, source-major
+    uint32_t *dirty[2];         // k x slots/32: slots lowered from outside, by round parity
+    uint32_t *act[2];           // tiles x kw: sources with dirty slots in the tile
+    uint32_t *stamp;            // tiles x ku: last round a unit was queued for
+    int32_t *Q[2];              // tiles x ku: units (tile, words) to process
+    Ctl *ctl;                   // band_ovf: some candidate label reached 2^32 - 1
+    uint64_t timeout_ns;
+};
+
+// Words per unit for k sources: as many as leave every CTA of the GPU two
+// units of a fully active round.
+int tile_unit_words(const TileGraph &g, int k);
+int launch_tiles(const TileJob &job, cudaStream_t st);
+
+// Reductions of the distances (source-major, dist[i * slots + slot]).
+struct TileReduce {
+    TileGraph g;
+    int k, W;
+    const uint32_t *dist;
+    const int32_t *sources, *sidx;
+    uint64_t *sum2;                 // n x 2
+    int32_t *pivot;
+    uint32_t *delta;
+    uint32_t *dcc;                  // k x k
+    unsigned long long *S_samp;     // k
+    unsigned long long *dmax;       // 1
+    int *err;                       // 1
+    // hybrid: distance histogram (source-major, hs = row stride >= D + 1 and a
+    // multiple of 64), suffix sums over its blocks of 64 distances
+    int64_t D, hs;
+    uint32_t *hist;
+    uint64_t *TN, *TS;              // k x (hs / 64 + 1)
+    HybPrep *hp;
+    const uint64_t *Lmask;          // n x W
+    uint64_t *lc2;                  // n x 2
+    // error estimate (null sqflag: not wanted; see ReduceJob)
+    const uint8_t *sqflag;
+    const int32_t *istar;
+    uint64_t *hcse;
+    uint32_t *fdist;
+};
+
+// Sums, pivots, Delta, delta_cc, exact S of the sampled nodes, the largest
+// distance and the reachability check.
+void run_tiles_reduce1(const TileReduce &r, cudaStream_t st);
+// After the thresholds and L(v) masks: histogram, tails, H statistics of
+// every node and the sums over L(v) n C.
+void run_tiles_reduce2(const TileReduce &r, cudaStream_t st);
+
+}  // namespace ccg
