@@ -42,6 +42,8 @@ constexpr double kDeltaMult = 96.0;
 // tiles, which goes on by twenty, about as much): MEASURE.
 constexpr int64_t kTileMinNodes = 1024;
 constexpr double kTileMinLevels = 64.0;
+// Mean arc lengths that a round's threshold moves on by: MEASURE2.
+constexpr double kTileDelta = 16.0;
 constexpr double kMaxHistBytes = 4.0 * (1ull << 30);  // distance histogram cap
 
 // Bumped whenever a device buffer is (re)allocated or freed: a captured
@@ -1219,6 +1221,7 @@ int tiled_pass1(cc_graph *g, int k, cudaStream_t st)
     j.uw = tile_unit_words(g->tg, k);
     j.ku = (j.kw + j.uw - 1) / j.uw;
     j.stamp = g->t_stamp.as<uint32_t>();
+    j.delta = (uint32_t)std::min(1e9, std::max(1.0, kTileDelta * g->w_mean));
     j.sources = g->sources.as<int32_t>();
     j.dist = g->t_dist.as<uint32_t>();
     j.dirty[0] = g->t_dirty0.as<uint32_t>();

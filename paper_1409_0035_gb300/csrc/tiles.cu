@@ -216,7 +216,7 @@ __global__ void k_tile_arcs(int64_t slots, const int32_t *perm, const int32_t *i
                             const int32_t *word_tile, const int32_t *tb, const int64_t *rp,
                             const int32_t *col, const uint32_t *w, const uint64_t *ioff,
                             const uint64_t *eoff, uint32_t *irp, uint32_t *erp, uint16_t *icol,
-                            int32_t *ecol, uint32_t *iw, uint32_t *ew)
+                            int32_t *ecol, uint16_t *etail, uint32_t *iw, uint32_t *ew)
 {
     for (STRIDED(s, slots + 1)) {
         uint32_t a = (uint32_t)ioff[s], b = (uint32_t)eoff[s];
@@ -233,6 +233,7 @@ __global__ void k_tile_arcs(int64_t slots, const int32_t *perm, const int32_t *i
                 ++a;
             } else {
                 ecol[b] = h;
+                etail[b] = (uint16_t)(s - tb[t]);
                 if (w) ew[b] = w[e];
                 ++b;
             }
@@ -307,114 +308,203 @@ k_tile_depth(const int32_t *tb, const int32_t *word_tile, const uint32_t *erp,
 // ---- the search -----------------------------------------------------------
 
 constexpr int kWarps = kT / 32;
+constexpr int kPair = 2;       // sources a warp takes together
+constexpr int kList = 256;     // labels to carry on that a list holds
+constexpr int kExt = 512;      // leaving arcs of a tile held in shared memory
 
 template <bool WT>
 struct TileShared {
-    uint32_t d[kWarps][kTileCap];
-    uint32_t off[kTileCap + 1];
-    uint32_t w[WT ? kTileArcs : 1];
+    uint32_t d[kWarps][kPair * kTileCap];
+    uint32_t chg[kWarps][kPair * kTileWords];
+    uint32_t w[WT ? kTileArcs : 1], ew[WT ? kExt : 1];
+    int32_t ecol[kExt];
+    uint16_t list[kWarps][2][kList];
+    uint16_t off[kTileCap + 2];
     uint16_t col[kTileArcs];
-    uint16_t list[kWarps][kTileCap];
-    uint32_t next[kWarps][kTileWords];
+    uint16_t etail[kExt];
 };
 
-// One (tile, source) pair on one warp; the tile's arcs are in S.
+// What a unit of work needs of its tile besides the arcs in shared memory.
+struct TileUnit {
+    int32_t s0;   // first slot
+    int nw;       // words
+    uint32_t e0;  // first leaving arc
+    int ext;      // leaving arcs
+};
+
+// A tile and up to two sources (src[1] = -1: one) on one warp, the labels of
+// both side by side: a front inside a tile is a dozen nodes wide, and two
+// fill a warp's lanes better than one.  Labels above T are lowered but not
+// carried on: they stay dirty for the next round (with arc lengths, whose
+// labels would otherwise run ahead of the shortest paths and be carried on
+// again and again).  pend: smallest label left dirty anywhere.
 template <bool WT>
-__device__ __forceinline__ void tile_source(const TileJob &J, TileShared<WT> &S, int src,
-                                            int32_t s0, int nw, int par, const Stage &stage,
-                                            int32_t *Qn, unsigned *qlen, uint32_t stamp,
-                                            unsigned long long &relax)
+__device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S,
+                                             const TileUnit &U, const int (&src)[kPair],
+                                             uint32_t T, int par, const Stage &stage,
+                                             int32_t *Qn, unsigned *qlen, uint32_t stamp,
+                                             unsigned *s_pend, unsigned long long &relax)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
     const int64_t slots = J.g.slots, words = slots >> 5;
-    uint32_t *const dist = J.dist + (int64_t)src * slots;
-    uint32_t *const dcur = J.dirty[par] + (int64_t)src * words + (s0 >> 5);
-    uint32_t *const d = S.d[wid];
-    uint16_t *const list = S.list[wid];
-    uint32_t *const next = S.next[wid];
-    // active: lane q holds word q of the slots whose labels dropped
+    uint32_t *const d = S.d[wid], *const chg = S.chg[wid];
+    const int nw = U.nw;
+    // The dirty words: lanes 0-15 the first source's, 16-31 the second's.
+    const int hs = lane < 16 ? src[0] : src[1];
     uint32_t a = 0;
-    if (lane < nw) {
-        a = __ldcg(dcur + lane);
-        if (a) dcur[lane] = 0u;
+    if (hs >= 0 && (lane & 15) < nw) {
+        uint32_t *p = J.dirty[par] + (int64_t)hs * words + (U.s0 >> 5) + (lane & 15);
+        a = __ldcg(p);
+        if (a) *p = 0u;
     }
-    for (int i = 4 * lane; i < 32 * nw; i += 128)
-        *reinterpret_cast<uint4 *>(d + i) = __ldcg(reinterpret_cast<const uint4 *>(dist + s0 + i));
-    uint32_t changed = 0;
-    for (;;) {
-        const int c = __popc(a);
-        int incl = c;
 #pragma unroll
-        for (int o = 1; o < kTileWords; o <<= 1) {
-            const int y = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int total = __shfl_sync(FULL, incl, kTileWords - 1);
-        if (total == 0) break;
-        changed |= a;
-        int at = incl - c;
-        for (uint32_t b = a; b; b &= b - 1) list[at++] = (uint16_t)(32 * lane + __ffs(b) - 1);
-        if (lane < kTileWords) next[lane] = 0u;
-        __syncwarp();
-        for (int j = lane; j < total; j += 32) {
-            const int u = list[j];
-            const uint32_t du = d[u];
-            const uint32_t e = S.off[u + 1];
-            for (uint32_t x = S.off[u]; x < e; ++x) {
-                const int v = S.col[x];
-                const uint32_t nd = du + (WT ? S.w[x] : 1u);
-                if (nd < du || nd == kInf) {
-                    J.ctl->band_ovf = 1;
-                } else if (nd < d[v] && nd < atomicMin(&d[v], nd)) {
-                    atomicOr(&next[v >> 5], 1u << (v & 31));
+    for (int h = 0; h < kPair; ++h)
+        if (src[h] >= 0)
+            for (int i = 4 * lane; i < 32 * nw; i += 128)
+                *reinterpret_cast<uint4 *>(d + h * kTileCap + i) = __ldcg(
+                    reinterpret_cast<const uint4 *>(J.dist + src[h] * slots + U.s0 + i));
+    chg[lane] = a;
+    // Lists of labels to carry on (entry = source half x kTileCap + slot),
+    // in turns; a list that would not fit is replaced by a sweep over every
+    // slot.
+    int n = __popc(a);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, n, o);
+        if (lane >= o) n += y;
+    }
+    int at = n - __popc(a);
+    n = __shfl_sync(FULL, n, 31);
+    bool sweep = n > kList;
+    int cur = 0;
+    if (!sweep)
+        for (uint32_t b = a; b; b &= b - 1)
+            S.list[wid][0][at++] = (uint16_t)(32 * lane + __ffs(b) - 1);
+    __syncwarp();
+    while (n) {
+        const int todo = sweep ? kPair * 32 * nw : n;
+        int cn = 0;
+        for (int j0 = 0; j0 < todo; j0 += 32) {
+            const int j = j0 + lane;
+            int u = 0;
+            bool on = j < todo;
+            if (on) {
+                if (!sweep) u = S.list[wid][cur][j];
+                else if (j < 32 * nw) u = j;
+                else u = kTileCap + j - 32 * nw, on = src[1] >= 0;
+            }
+            const uint32_t du = on ? d[u] : kInf;
+            int x = 0, e = 0;
+            if (du <= T && du != kInf) {
+                x = S.off[u & (kTileCap - 1)];
+                e = S.off[(u & (kTileCap - 1)) + 1];
+            }
+            const int turns = __reduce_max_sync(FULL, (unsigned)(e - x));
+            for (int t = 0; t < turns; ++t, ++x) {
+                bool imp = false;
+                int v = 0;
+                if (x < e) {
+                    v = (u & kTileCap) | S.col[x];
+                    const uint32_t nd = du + (WT ? S.w[x] : 1u);
+                    if (WT && (nd < du || nd == kInf)) J.ctl->band_ovf = 1;
+                    else if (nd < d[v]) imp = nd < atomicMin(&d[v], nd);
                 }
+                const unsigned m = __ballot_sync(FULL, imp);
+                if (imp) {
+                    const int p = cn + __popc(m & below);
+                    if (p < kList) S.list[wid][cur ^ 1][p] = (uint16_t)v;
+                    atomicOr(&chg[v >> 5], 1u << (v & 31));
+                }
+                cn += __popc(m);
             }
         }
-        if (lane == 0) relax += (unsigned)total;
+        if (lane == 0) relax += (unsigned)n;
         __syncwarp();
-        a = lane < kTileWords ? next[lane] : 0u;
+        n = cn;
+        sweep = cn > kList;
+        cur ^= 1;
     }
     // What dropped goes back (another tile may have lowered a border label
-    // meanwhile: a minimum, not a store), and across the border.
-    for (int q = 0; q < nw; ++q) {
-        const uint32_t cw = __shfl_sync(FULL, changed, q);
-        if (!((cw >> lane) & 1u)) continue;
-        const int i = 32 * q + lane;
-        const uint32_t du = d[i];
-        atomicMin(dist + s0 + i, du);
-        const uint32_t e = J.g.erp[s0 + i + 1];
-        for (uint32_t x = J.g.erp[s0 + i]; x < e; ++x) {
-            const int32_t v = J.g.ecol[x];
-            const uint32_t nd = du + (WT ? J.g.ew[x] : 1u);
-            if (nd < du || nd == kInf) {
-                J.ctl->band_ovf = 1;
-            } else if (nd < __ldcg(dist + v) && nd < atomicMin(dist + v, nd)) {
-                atomicOr(J.dirty[par ^ 1] + (int64_t)src * words + (v >> 5), 1u << (v & 31));
-                const int32_t t = J.g.word_tile[v >> 5];
-                if (atomicOr(J.act[par ^ 1] + (int64_t)t * J.kw + (src >> 5),
-                             1u << (src & 31)) == 0u) {
-                    const int32_t unit = t * J.ku + (src >> 5) / J.uw;
-                    if (atomicExch(J.stamp + unit, stamp) != stamp)
-                        stage_push(stage, unit, Qn, qlen);
+    // meanwhile: a minimum, not a store); what is above T stays dirty.
+    const int base = U.s0 >> 5;
+    uint32_t pend = kInf;
+    unsigned defer = 0;  // bit h: source h has labels left
+#pragma unroll
+    for (int h = 0; h < kPair; ++h) {
+        if (src[h] < 0) continue;
+        uint32_t *const dist = J.dist + src[h] * slots + U.s0;
+        for (int q = 0; q < nw; ++q) {
+            const uint32_t cw = chg[h * kTileWords + q];
+            if (cw == 0u) continue;
+            bool later = false;
+            if ((cw >> lane) & 1u) {
+                const uint32_t du = d[h * kTileCap + 32 * q + lane];
+                atomicMin(dist + 32 * q + lane, du);
+                if (WT && du > T) {
+                    later = true;
+                    pend = min(pend, du);
+                }
+            }
+            if (WT) {
+                const unsigned m = __ballot_sync(FULL, later);
+                if (m) {
+                    defer |= 1u << h;
+                    if (lane == 0)
+                        atomicOr(J.dirty[par ^ 1] + src[h] * words + base + q, m);
                 }
             }
         }
+    }
+    auto activate = [&](int t, int s) {
+        if (atomicOr(J.act[par ^ 1] + (int64_t)t * J.kw + (s >> 5), 1u << (s & 31)) == 0u) {
+            const int32_t unit = t * J.ku + (s >> 5) / J.uw;
+            if (atomicExch(J.stamp + unit, stamp) != stamp) stage_push(stage, unit, Qn, qlen);
+        }
+    };
+    if (WT && lane < kPair && ((defer >> lane) & 1u))
+        activate(J.g.word_tile[base], lane == 0 ? src[0] : src[1]);
+    // ... and across the border, a lane per leaving arc.
+    const bool held = U.ext <= kExt;
+    for (int x = lane; x < U.ext; x += 32) {
+        const int u = held ? S.etail[x] : J.g.etail[U.e0 + x];
+        const int32_t v = held ? S.ecol[x] : J.g.ecol[U.e0 + x];
+        const uint32_t len = !WT ? 1u : held ? S.ew[x] : J.g.ew[U.e0 + x];
+#pragma unroll
+        for (int h = 0; h < kPair; ++h) {
+            if (src[h] < 0 || !((chg[h * kTileWords + (u >> 5)] >> (u & 31)) & 1u)) continue;
+            const uint32_t du = d[h * kTileCap + u], nd = du + len;
+            if (WT && du > T) continue;
+            if (WT && (nd < du || nd == kInf)) {
+                J.ctl->band_ovf = 1;
+                continue;
+            }
+            if (nd < atomicMin(J.dist + src[h] * slots + v, nd)) {
+                pend = min(pend, nd);
+                atomicOr(J.dirty[par ^ 1] + src[h] * words + (v >> 5), 1u << (v & 31));
+                activate(J.g.word_tile[v >> 5], src[h]);
+            }
+        }
+    }
+    if (WT) {
+        pend = __reduce_min_sync(FULL, pend);
+        if (lane == 0 && pend != kInf) atomicMin(s_pend, pend);
     }
     __syncwarp();
 }
 
 // Units (a tile, up to 256 sources) of a round are popped by the CTAs; a CTA
 // loads the tile's arcs once and its warps take the unit's active sources
-// one after another.
+// two by two.
 template <bool WT>
-__global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
+__global__ void __launch_bounds__(kT, WT ? 3 : 4) k_tiles(TileJob J)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
     TileShared<WT> &S = *reinterpret_cast<TileShared<WT> *>(s_raw);
     __shared__ int32_t s_buf[kStage];
-    __shared__ unsigned s_cnt, s_base, s_pop, s_next, s_mask[kUnitWords];
+    __shared__ unsigned s_cnt, s_base, s_pop, s_next, s_pend, s_mask[kUnitWords];
     const Stage stage{s_buf, &s_cnt, &s_base};
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const int64_t gthreads = (int64_t)gridDim.x * kT;
     const int64_t gtid = (int64_t)blockIdx.x * kT + threadIdx.x;
     const int64_t slots = J.g.slots, words = slots >> 5;
@@ -447,16 +537,24 @@ __global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
     }
     if (!grid_sync(ctl, blockIdx.x, gridDim.x, J.timeout_ns)) return;
     unsigned long long relax = 0;
+    uint32_t T = WT ? 0u : kInf;
     int r = 0;
     for (;; ++r) {
         const int par = r & 1;
         LevelCtl *C = &ctl->lev[r & 3];
         const unsigned qn = ((volatile LevelCtl *)C)->qlen;
         if (qn == 0) break;
+        if (WT) {  // T moves on by delta, and to the smallest label at least
+            const uint32_t pend = r ? ~((volatile LevelCtl *)C)->mlen : 0u;
+            const uint32_t from = pend > T ? pend : T;
+            T = from + J.delta < from ? kInf : from + J.delta;
+        }
         if (gtid == 0) {  // round r + 2's counters
             ctl->lev[(r + 2) & 3].qlen = 0;
             ctl->lev[(r + 2) & 3].hnext = 0;
+            ctl->lev[(r + 2) & 3].mlen = 0;  // the complement of its smallest label
         }
+        if (threadIdx.x == 0) s_pend = kInf;
         int32_t *Qn = J.Q[par ^ 1];
         unsigned *qlen = &ctl->lev[(r + 1) & 3].qlen;
         for (;;) {
@@ -479,32 +577,48 @@ __global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
                 s_mask[threadIdx.x] = m;
             }
             const int32_t s0 = J.g.tb[t], nw = (J.g.tb[t + 1] - s0) >> 5;
-            const uint32_t a0 = J.g.irp[s0];
+            const uint32_t a0 = J.g.irp[s0], e0 = J.g.erp[s0];
             const int arcs = (int)(J.g.irp[s0 + 32 * nw] - a0);
-            for (int i = threadIdx.x; i <= 32 * nw; i += kT) S.off[i] = J.g.irp[s0 + i] - a0;
+            const TileUnit U{s0, nw, e0, (int)(J.g.erp[s0 + 32 * nw] - e0)};
+            for (int i = threadIdx.x; i <= 32 * nw; i += kT)
+                S.off[i] = (uint16_t)(J.g.irp[s0 + i] - a0);
             for (int i = threadIdx.x; i < arcs; i += kT) {
                 S.col[i] = J.g.icol[a0 + i];
                 if (WT) S.w[i] = J.g.iw[a0 + i];
             }
+            for (int i = threadIdx.x; i < U.ext && U.ext <= kExt; i += kT) {
+                S.etail[i] = J.g.etail[e0 + i];
+                S.ecol[i] = J.g.ecol[e0 + i];
+                if (WT) S.ew[i] = J.g.ew[e0 + i];
+            }
             __syncthreads();
             for (;;) {
                 unsigned q = 0;
-                if (lane == 0) q = atomicAdd(&s_next, 1u);
+                if (lane == 0) q = atomicAdd(&s_next, (unsigned)kPair);
                 q = __shfl_sync(FULL, q, 0);
-                // the q-th active source
+                // active sources number q and q + 1
+                int src[kPair] = {-1, -1};
                 int w = 0;
                 unsigned m = s_mask[0];
-                while (q >= (unsigned)__popc(m) && w < kUnitWords - 1) {
-                    q -= __popc(m);
-                    m = s_mask[++w];
+#pragma unroll
+                for (int h = 0; h < kPair; ++h) {
+                    while (q >= (unsigned)__popc(m) && w < kUnitWords - 1) {
+                        q -= __popc(m);
+                        m = s_mask[++w];
+                    }
+                    if (q >= (unsigned)__popc(m)) break;
+                    for (; q; --q) m &= m - 1;
+                    src[h] = (w0 + w) * 32 + __ffs(m) - 1;
+                    m &= m - 1;
                 }
-                if (q >= (unsigned)__popc(m)) break;
-                for (; q; --q) m &= m - 1;
-                tile_source<WT>(J, S, (w0 + w) * 32 + __ffs(m) - 1, s0, nw, par, stage, Qn, qlen,
-                                (uint32_t)r + 2u, relax);
+                if (src[0] < 0) break;
+                tile_sources<WT>(J, S, U, src, T, par, stage, Qn, qlen, (uint32_t)r + 2u,
+                                 &s_pend, relax);
             }
             __syncthreads();
         }
+        if (WT && threadIdx.x == 0 && s_pend != kInf)
+            atomicMax(&ctl->lev[(r + 1) & 3].mlen, ~s_pend);
         stage_flush(stage, Qn, qlen);
         if (!grid_sync(ctl, blockIdx.x, gridDim.x, J.timeout_ns)) return;
     }
@@ -811,7 +925,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
                                                          flag.as<uint64_t>());
     T_RC(device_scan_u64(flag.as<uint64_t>(), idx.as<uint64_t>(), (int64_t)tiles, &words, st));
     const int64_t slots = (int64_t)words * 32;
-    Buf perm, iperm, tb, wt, irp, erp, icol, ecol, iw, ew, din, dex;
+    Buf perm, iperm, tb, wt, irp, erp, icol, ecol, etail, iw, ew, din, dex;
     if (slots > 0x7FFFFFE0LL) return CC_OK;
     T_RC(perm.alloc(slots * 4));
     T_RC(iperm.alloc(n * 4));
@@ -834,6 +948,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     T_RC(erp.alloc((slots + 1) * 4));
     T_RC(icol.alloc(in * 2));
     T_RC(ecol.alloc(ex * 4));
+    T_RC(etail.alloc(ex * 2));
     if (w) {
         T_RC(iw.alloc(in * 4));
         T_RC(ew.alloc(ex * 4));
@@ -842,7 +957,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
                                    wt.as<int32_t>(), tb.as<int32_t>(), rp, col, w,
                                    din.as<uint64_t>(), dex.as<uint64_t>(), irp.as<uint32_t>(),
                                    erp.as<uint32_t>(), icol.as<uint16_t>(), ecol.as<int32_t>(),
-                                   iw.as<uint32_t>(), ew.as<uint32_t>());
+                                   etail.as<uint16_t>(), iw.as<uint32_t>(), ew.as<uint32_t>());
     k_tile_stats<<<(int)std::min<uint64_t>(tiles, 152 * 8), 128, 0, st>>>(
         (int64_t)tiles, tb.as<int32_t>(), wt.as<int32_t>(), irp.as<uint32_t>(),
         erp.as<uint32_t>(), ecol.as<int32_t>(), stats.as<unsigned long long>());
@@ -869,6 +984,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     out.erp = erp.take<uint32_t>();
     out.icol = icol.take<uint16_t>();
     out.ecol = ecol.take<int32_t>();
+    out.etail = etail.take<uint16_t>();
     out.iw = iw.take<uint32_t>();
     out.ew = ew.take<uint32_t>();
     *ok = true;
@@ -877,7 +993,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
 
 void tiles_free(TileGraph &g)
 {
-    void *p[] = {g.perm, g.iperm, g.tb, g.word_tile, g.irp, g.erp, g.icol, g.ecol, g.iw, g.ew};
+    void *p[] = {g.perm, g.iperm, g.tb, g.word_tile, g.irp, g.erp, g.icol, g.ecol, g.etail, g.iw, g.ew};
     for (void *x : p)
         if (x) cudaFree(x);
     g = TileGraph{};

@@ -11,7 +11,7 @@ namespace ccg {
 
 constexpr int kTileCap = 512;      // nodes of a tile at most
 constexpr int kTileMean = 256;     // nodes per cluster centre
-constexpr int kTileArcs = 2560;    // arcs inside a tile at most
+constexpr int kTileArcs = 2048;    // arcs inside a tile at most
 constexpr int kUnitWords = 8;      // words of 32 sources a CTA takes at once
 
 // A graph cut into tiles of neighbouring nodes.  Slots are the nodes' numbers
@@ -26,6 +26,7 @@ struct TileGraph {
     uint32_t *irp = nullptr, *erp = nullptr;     // slots + 1: arcs inside, leaving the tile
     uint16_t *icol = nullptr;                    // head's slot within the tile
     int32_t *ecol = nullptr;                     // head's slot
+    uint16_t *etail = nullptr;                   // tail's slot within the tile
     uint32_t *iw = nullptr, *ew = nullptr;       // their lengths (null: unit lengths)
 };
 
@@ -41,6 +42,7 @@ struct TileJob {
     int k;                      // sources
     int kw;                     // words of 32 sources
     int uw, ku;                 // words per unit of work (at most kUnitWords), units per tile
+    uint32_t delta;             // arc lengths: labels a round carries on beyond the last one's
     const int32_t *sources;     // k node ids
     uint32_t *dist;             // k x slots, source-major
     uint32_t *dirty[2];         // k x slots/32: slots lowered from outside, by round parity
