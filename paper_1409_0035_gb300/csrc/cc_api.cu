@@ -43,7 +43,7 @@ constexpr double kDeltaMult = 96.0;
 constexpr int64_t kTileMinNodes = 1024;
 constexpr double kTileMinLevels = 64.0;
 // Mean arc lengths that a round's threshold moves on by: MEASURE2.
-constexpr double kTileDelta = 16.0;
+constexpr double kTileDelta = 10.0;
 constexpr double kMaxHistBytes = 4.0 * (1ull << 30);  // distance histogram cap
 
 // Bumped whenever a device buffer is (re)allocated or freed: a captured

@@ -30,7 +30,7 @@ namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int kT = 256;
-constexpr int kTileWords = kTileCap / 32;
+constexpr uint16_t kNoArc = 0xFFFF, kLongRow = 0xFFFE;
 // Breadth-first growth of the clusters: hops per pass, passes.
 constexpr int kGrowHops = 32;
 constexpr int kGrowPasses = 8;
@@ -87,14 +87,15 @@ struct Buf {
 
 // ---- cutting the graph ----------------------------------------------------
 
-// Clusters: unlabelled nodes picked at random (one in kTileMean) and the
+// Clusters: unlabelled nodes picked at random (one in half a tile's capacity) and the
 // nodes nearest to them in hops (ties to the smallest centre), pass by pass.
 // stamp = the step a node was labelled at (kInf: not yet); a step only reads
 // labels of earlier steps, so the result does not depend on timing.
-__global__ void k_centres(int64_t n, uint64_t seed, uint32_t step, int32_t *lab, uint32_t *stamp)
+__global__ void k_centres(int64_t n, unsigned mean, uint64_t seed, uint32_t step, int32_t *lab,
+                          uint32_t *stamp)
 {
     for (STRIDED(v, n))
-        if (stamp[v] == kInf && splitmix64_out(seed, (uint64_t)v) < ~0ull / kTileMean) {
+        if (stamp[v] == kInf && splitmix64_out(seed, (uint64_t)v) < ~0ull / mean) {
             lab[v] = (int32_t)v;
             stamp[v] = step;
         }
@@ -129,7 +130,7 @@ __global__ void k_keys(int64_t n, const int32_t *lab, const uint32_t *stamp, uin
     unsigned long long h = 0;
     for (STRIDED(v, n)) {
         const uint32_t s = stamp[v];
-        keys[v] = s != kInf ? (uint64_t)lab[v] : (uint64_t)(v & ~(int64_t)(kTileMean - 1));
+        keys[v] = s != kInf ? (uint64_t)lab[v] : (uint64_t)(v & ~255ll);
         vals[v] = (uint32_t)v;
         h += s != kInf ? s % (kGrowHops + 1) : kGrowHops;
     }
@@ -152,14 +153,14 @@ __global__ void k_cluster_first(int64_t n, const uint64_t *keys, const uint64_t 
         if (i == 0 || keys[i] != keys[i - 1]) first[idx[i]] = (int32_t)i;
 }
 
-// A cluster of more than kTileCap nodes is chopped into tiles of that many.
+// A cluster of more than a tile's capacity is chopped into tiles of that many.
 __global__ void k_tile_starts(int64_t n, const uint64_t *keys, const uint64_t *idx,
-                              const int32_t *first, uint64_t *flag)
+                              const int32_t *first, int cap, uint64_t *flag)
 {
     for (STRIDED(i, n)) {
         const bool head = i == 0 || keys[i] != keys[i - 1];
         const int64_t c = (int64_t)idx[i] - (head ? 0 : 1);
-        flag[i] = (i - first[c]) % kTileCap == 0;
+        flag[i] = (i - first[c]) % cap == 0;
     }
 }
 
@@ -216,20 +217,28 @@ __global__ void k_tile_arcs(int64_t slots, const int32_t *perm, const int32_t *i
                             const int32_t *word_tile, const int32_t *tb, const int64_t *rp,
                             const int32_t *col, const uint32_t *w, const uint64_t *ioff,
                             const uint64_t *eoff, uint32_t *irp, uint32_t *erp, uint16_t *icol,
-                            int32_t *ecol, uint16_t *etail, uint32_t *iw, uint32_t *ew)
+                            int32_t *ecol, uint16_t *etail, uint32_t *iw, uint32_t *ew,
+                            ushort4 *icol4, uint4 *iw4)
 {
     for (STRIDED(s, slots + 1)) {
         uint32_t a = (uint32_t)ioff[s], b = (uint32_t)eoff[s];
         irp[s] = a;
         erp[s] = b;
-        const int32_t v = s < slots ? perm[s] : -1;
-        if (v < 0) continue;
-        const int32_t t = word_tile[s >> 5];
-        for (int64_t e = rp[v]; e < rp[v + 1]; ++e) {
+        if (s == slots) continue;
+        const int32_t v = perm[s], t = word_tile[s >> 5];
+        uint16_t c[4] = {kNoArc, kNoArc, kNoArc, kNoArc};
+        uint32_t l[4] = {0u, 0u, 0u, 0u};
+        int m = 0;
+        for (int64_t e = v < 0 ? 0 : rp[v], end = v < 0 ? 0 : rp[v + 1]; e < end; ++e) {
             const int32_t h = iperm[col[e]];
             if (word_tile[h >> 5] == t) {
                 icol[a] = (uint16_t)(h - tb[t]);
                 if (w) iw[a] = w[e];
+                if (m < 4) {
+                    c[m] = (uint16_t)(h - tb[t]);
+                    l[m] = w ? w[e] : 1u;
+                }
+                ++m;
                 ++a;
             } else {
                 ecol[b] = h;
@@ -238,14 +247,18 @@ __global__ void k_tile_arcs(int64_t slots, const int32_t *perm, const int32_t *i
                 ++b;
             }
         }
+        if (m > 4) c[0] = kLongRow;
+        icol4[s] = make_ushort4(c[0], m > 4 ? kNoArc : c[1], m > 4 ? kNoArc : c[2],
+                                m > 4 ? kNoArc : c[3]);
+        if (iw4) iw4[s] = make_uint4(l[0], l[1], l[2], l[3]);
     }
 }
 
-// stats[0] = most arcs inside a tile, stats[1] = neighbouring tiles summed
-// over the tiles (an arc counts when no earlier one of the tile's leads to
-// the same tile; beyond 2048 leaving arcs every one counts).
+// stats[1] = neighbouring tiles summed over the tiles (an arc counts when no
+// earlier one of the tile's leads to the same tile; beyond 2048 leaving arcs
+// every one counts).
 __global__ void k_tile_stats(int64_t tiles, const int32_t *tb, const int32_t *word_tile,
-                             const uint32_t *irp, const uint32_t *erp, const int32_t *ecol,
+                             const uint32_t *erp, const int32_t *ecol,
                              unsigned long long *stats)
 {
     __shared__ int32_t s_t[2048];
@@ -263,8 +276,6 @@ __global__ void k_tile_stats(int64_t tiles, const int32_t *tb, const int32_t *wo
             fresh += !seen;
         }
         if (fresh) atomicAdd(&stats[1], (unsigned long long)fresh);
-        if (threadIdx.x == 0)
-            atomicMax(&stats[0], (unsigned long long)(irp[tb[t + 1]] - irp[tb[t]]));
     }
 }
 
@@ -309,65 +320,82 @@ k_tile_depth(const int32_t *tb, const int32_t *word_tile, const uint32_t *erp,
 
 constexpr int kWarps = kT / 32;
 constexpr int kPair = 2;       // sources a warp takes together
-constexpr int kList = 256;     // labels to carry on that a list holds
-constexpr int kExt = 512;      // leaving arcs of a tile held in shared memory
+constexpr int kList = 192;     // labels to carry on that a list holds
 
+// A warp's labels of its tile for two sources side by side (entry = half x
+// kCap + slot), which of them changed, and two lists of labels to carry
+// on, used in turns.
+template <bool WT>
+struct TileWarp {
+    static constexpr int kCap = tile_cap(WT);
+    uint32_t d[kPair * kCap];
+    uint32_t chg[32];
+    uint16_t list[2][kList];
+};
+
+// A CTA's tile: inline rows, the first kExt leaving arcs.
+constexpr int kExt = 256;
 template <bool WT>
 struct TileShared {
-    uint32_t d[kWarps][kPair * kTileCap];
-    uint32_t chg[kWarps][kPair * kTileWords];
-    uint32_t w[WT ? kTileArcs : 1], ew[WT ? kExt : 1];
+    TileWarp<WT> warp[kWarps];
+    uint4 w4[WT ? tile_cap(WT) : 1];
+    ushort4 c4[tile_cap(WT)];
     int32_t ecol[kExt];
-    uint16_t list[kWarps][2][kList];
-    uint16_t off[kTileCap + 2];
-    uint16_t col[kTileArcs];
+    uint32_t ew[WT ? kExt : 1];
     uint16_t etail[kExt];
+    int32_t s0, nw, ext;
+    uint32_t e0;
 };
 
-// What a unit of work needs of its tile besides the arcs in shared memory.
-struct TileUnit {
-    int32_t s0;   // first slot
-    int nw;       // words
-    uint32_t e0;  // first leaving arc
-    int ext;      // leaving arcs
-};
-
-// A tile and up to two sources (src[1] = -1: one) on one warp, the labels of
-// both side by side: a front inside a tile is a dozen nodes wide, and two
-// fill a warp's lanes better than one.  Labels above T are lowered but not
-// carried on: they stay dirty for the next round (with arc lengths, whose
-// labels would otherwise run ahead of the shortest paths and be carried on
-// again and again).  pend: smallest label left dirty anywhere.
+// A tile and up to two sources (src[1] = -1: one) on one warp: a front inside
+// a tile is a dozen nodes wide, and two fill a warp's lanes better than one.
+// Labels above T are lowered but not carried on: they stay dirty for the next
+// round (with arc lengths, whose labels would otherwise run ahead of the
+// shortest paths and be carried on again and again).  pend: smallest label
+// left dirty anywhere.  Latency is what bounds it, so the arcs are read from
+// shared memory and everything a step can have in flight is: the labels with
+// the dirty words, a node's four arcs, the border's minima.
 template <bool WT>
-__device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S,
-                                             const TileUnit &U, const int (&src)[kPair],
-                                             uint32_t T, int par, const Stage &stage,
-                                             int32_t *Qn, unsigned *qlen, uint32_t stamp,
-                                             unsigned *s_pend, unsigned long long &relax)
+__device__ __forceinline__ void tile_sources(const TileJob &J, const TileShared<WT> &C,
+                                             TileWarp<WT> &S, int t, const int (&src)[kPair],
+                                             uint32_t T, int par,
+                                             const Stage &stage, int32_t *Qn, unsigned *qlen,
+                                             uint32_t stamp, unsigned *s_pend,
+                                             unsigned long long &relax)
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int kCap = TileWarp<WT>::kCap, kWords = kCap / 32;
+    const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     const int64_t slots = J.g.slots, words = slots >> 5;
-    uint32_t *const d = S.d[wid], *const chg = S.chg[wid];
-    const int nw = U.nw;
-    // The dirty words: lanes 0-15 the first source's, 16-31 the second's.
-    const int hs = lane < 16 ? src[0] : src[1];
-    uint32_t a = 0;
-    if (hs >= 0 && (lane & 15) < nw) {
-        uint32_t *p = J.dirty[par] + (int64_t)hs * words + (U.s0 >> 5) + (lane & 15);
-        a = __ldcg(p);
-        if (a) *p = 0u;
-    }
+    uint32_t *const d = S.d, *const chg = S.chg;
+    const int32_t s0 = C.s0;
+    const int nw = C.nw, ext = C.ext;
+    // The dirty words: lanes 0 .. kWords - 1 the first source's, the next
+    // kWords the second's.
+    const int hq = lane < kWords ? lane : lane - kWords;
+    const int hs = lane < kWords ? src[0] : lane < kPair * kWords ? src[1] : -1;
+    uint32_t *const dw = J.dirty[par] + (int64_t)hs * words + (s0 >> 5) + hq;
+    const bool mine = hs >= 0 && hq < nw;
+    const uint32_t a = mine ? __ldcg(dw) : 0u;
+    constexpr int kLoads = (kCap + 127) / 128;
 #pragma unroll
-    for (int h = 0; h < kPair; ++h)
-        if (src[h] >= 0)
-            for (int i = 4 * lane; i < 32 * nw; i += 128)
-                *reinterpret_cast<uint4 *>(d + h * kTileCap + i) = __ldcg(
-                    reinterpret_cast<const uint4 *>(J.dist + src[h] * slots + U.s0 + i));
+    for (int h = 0; h < kPair; ++h) {
+        uint4 x[kLoads];
+#pragma unroll
+        for (int q = 0; q < kLoads; ++q) {
+            const int i = 4 * lane + 128 * q;
+            if (src[h] >= 0 && i < 32 * nw)
+                x[q] = __ldcg(reinterpret_cast<const uint4 *>(J.dist + src[h] * slots + s0 + i));
+        }
+#pragma unroll
+        for (int q = 0; q < kLoads; ++q) {
+            const int i = 4 * lane + 128 * q;
+            if (src[h] >= 0 && i < 32 * nw)
+                *reinterpret_cast<uint4 *>(d + h * kCap + i) = x[q];
+        }
+    }
+    if (a) *dw = 0u;
     chg[lane] = a;
-    // Lists of labels to carry on (entry = source half x kTileCap + slot),
-    // in turns; a list that would not fit is replaced by a sweep over every
-    // slot.
     int n = __popc(a);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -376,11 +404,11 @@ __device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S
     }
     int at = n - __popc(a);
     n = __shfl_sync(FULL, n, 31);
+    // A list that would not fit is replaced by a sweep over every slot.
     bool sweep = n > kList;
     int cur = 0;
     if (!sweep)
-        for (uint32_t b = a; b; b &= b - 1)
-            S.list[wid][0][at++] = (uint16_t)(32 * lane + __ffs(b) - 1);
+        for (uint32_t b = a; b; b &= b - 1) S.list[0][at++] = (uint16_t)(32 * lane + __ffs(b) - 1);
     __syncwarp();
     while (n) {
         const int todo = sweep ? kPair * 32 * nw : n;
@@ -390,33 +418,67 @@ __device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S
             int u = 0;
             bool on = j < todo;
             if (on) {
-                if (!sweep) u = S.list[wid][cur][j];
+                if (!sweep) u = S.list[cur][j];
                 else if (j < 32 * nw) u = j;
-                else u = kTileCap + j - 32 * nw, on = src[1] >= 0;
+                else u = kCap + j - 32 * nw, on = src[1] >= 0;
             }
             const uint32_t du = on ? d[u] : kInf;
-            int x = 0, e = 0;
+            const int hb = u >= kCap ? kCap : 0;
+            uint32_t x = 0, e = 0;  // rows of more than four arcs: the rest of the row
+            ushort4 c = make_ushort4(kNoArc, kNoArc, kNoArc, kNoArc);
+            uint4 w = make_uint4(1u, 1u, 1u, 1u);
             if (du <= T && du != kInf) {
-                x = S.off[u & (kTileCap - 1)];
-                e = S.off[(u & (kTileCap - 1)) + 1];
+                c = C.c4[u - hb];
+                if (WT) w = C.w4[u - hb];
+                if (c.x == kLongRow) {
+                    x = J.g.irp[s0 + u - hb];
+                    e = J.g.irp[s0 + u - hb + 1];
+                    c.x = kNoArc;
+                }
             }
-            const int turns = __reduce_max_sync(FULL, (unsigned)(e - x));
-            for (int t = 0; t < turns; ++t, ++x) {
-                bool imp = false;
-                int v = 0;
-                if (x < e) {
-                    v = (u & kTileCap) | S.col[x];
-                    const uint32_t nd = du + (WT ? S.w[x] : 1u);
-                    if (WT && (nd < du || nd == kInf)) J.ctl->band_ovf = 1;
-                    else if (nd < d[v]) imp = nd < atomicMin(&d[v], nd);
+            const unsigned more = __reduce_max_sync(FULL, (e - x + 3) / 4);
+            for (unsigned r = 0;; ++r) {
+                int v[4] = {c.x, c.y, c.z, c.w};
+                const uint32_t len[4] = {w.x, w.y, w.z, w.w};
+                uint32_t nd[4];
+                bool imp[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    nd[q] = du + (WT ? len[q] : 1u);
+                    imp[q] = v[q] != kNoArc;
+                    if (WT && imp[q] && (nd[q] < du || nd[q] == kInf)) {
+                        J.ctl->band_ovf = 1;
+                        imp[q] = false;
+                    }
+                    v[q] += hb;
+                    if (imp[q]) imp[q] = nd[q] < d[v[q]];
                 }
-                const unsigned m = __ballot_sync(FULL, imp);
-                if (imp) {
-                    const int p = cn + __popc(m & below);
-                    if (p < kList) S.list[wid][cur ^ 1][p] = (uint16_t)v;
-                    atomicOr(&chg[v >> 5], 1u << (v & 31));
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (imp[q]) imp[q] = nd[q] < atomicMin(&d[v[q]], nd[q]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const unsigned m = __ballot_sync(FULL, imp[q]);
+                    if (imp[q]) {
+                        const int p = cn + __popc(m & below);
+                        if (p < kList) S.list[cur ^ 1][p] = (uint16_t)v[q];
+                        atomicOr(&chg[v[q] >> 5], 1u << (v[q] & 31));
+                    }
+                    cn += __popc(m);
                 }
-                cn += __popc(m);
+                if (r == more) break;
+                // the next four of a long row
+                c.x = x < e ? J.g.icol[x] : kNoArc;
+                c.y = x + 1 < e ? J.g.icol[x + 1] : kNoArc;
+                c.z = x + 2 < e ? J.g.icol[x + 2] : kNoArc;
+                c.w = x + 3 < e ? J.g.icol[x + 3] : kNoArc;
+                if (WT) {
+                    w.x = x < e ? J.g.iw[x] : 0u;
+                    w.y = x + 1 < e ? J.g.iw[x + 1] : 0u;
+                    w.z = x + 2 < e ? J.g.iw[x + 2] : 0u;
+                    w.w = x + 3 < e ? J.g.iw[x + 3] : 0u;
+                }
+                x = x + 4 < e ? x + 4 : e;
             }
         }
         if (lane == 0) relax += (unsigned)n;
@@ -427,19 +489,18 @@ __device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S
     }
     // What dropped goes back (another tile may have lowered a border label
     // meanwhile: a minimum, not a store); what is above T stays dirty.
-    const int base = U.s0 >> 5;
     uint32_t pend = kInf;
     unsigned defer = 0;  // bit h: source h has labels left
 #pragma unroll
     for (int h = 0; h < kPair; ++h) {
         if (src[h] < 0) continue;
-        uint32_t *const dist = J.dist + src[h] * slots + U.s0;
+        uint32_t *const dist = J.dist + src[h] * slots + s0;
         for (int q = 0; q < nw; ++q) {
-            const uint32_t cw = chg[h * kTileWords + q];
+            const uint32_t cw = chg[h * kWords + q];
             if (cw == 0u) continue;
             bool later = false;
             if ((cw >> lane) & 1u) {
-                const uint32_t du = d[h * kTileCap + 32 * q + lane];
+                const uint32_t du = d[h * kCap + 32 * q + lane];
                 atomicMin(dist + 32 * q + lane, du);
                 if (WT && du > T) {
                     later = true;
@@ -451,40 +512,82 @@ __device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S
                 if (m) {
                     defer |= 1u << h;
                     if (lane == 0)
-                        atomicOr(J.dirty[par ^ 1] + src[h] * words + base + q, m);
+                        atomicOr(J.dirty[par ^ 1] + src[h] * words + (s0 >> 5) + q, m);
                 }
             }
         }
     }
-    auto activate = [&](int t, int s) {
-        if (atomicOr(J.act[par ^ 1] + (int64_t)t * J.kw + (s >> 5), 1u << (s & 31)) == 0u) {
-            const int32_t unit = t * J.ku + (s >> 5) / J.uw;
-            if (atomicExch(J.stamp + unit, stamp) != stamp) stage_push(stage, unit, Qn, qlen);
-        }
+    auto queue_unit = [&](int tt, int s, uint32_t before) {
+        if (before) return;
+        const int32_t unit = tt * J.ku + (s >> 5) / J.uw;
+        if (atomicExch(J.stamp + unit, stamp) != stamp) stage_push(stage, unit, Qn, qlen);
     };
-    if (WT && lane < kPair && ((defer >> lane) & 1u))
-        activate(J.g.word_tile[base], lane == 0 ? src[0] : src[1]);
-    // ... and across the border, a lane per leaving arc.
-    const bool held = U.ext <= kExt;
-    for (int x = lane; x < U.ext; x += 32) {
-        const int u = held ? S.etail[x] : J.g.etail[U.e0 + x];
-        const int32_t v = held ? S.ecol[x] : J.g.ecol[U.e0 + x];
-        const uint32_t len = !WT ? 1u : held ? S.ew[x] : J.g.ew[U.e0 + x];
+    auto activate = [&](int tt, int s) {
+        return atomicOr(J.act[par ^ 1] + (int64_t)tt * J.kw + (s >> 5), 1u << (s & 31));
+    };
+    if (WT && lane < kPair && ((defer >> lane) & 1u)) {
+        const int s = lane == 0 ? src[0] : src[1];
+        queue_unit(t, s, activate(t, s));
+    }
+    // ... and across the border, a lane per leaving arc, two arcs and both
+    // sources at a time.
+    for (int x0 = 0; x0 < ext; x0 += 64) {
+        uint32_t nd[4], old[4];
+        int32_t v[2];
+        bool go[4];
 #pragma unroll
-        for (int h = 0; h < kPair; ++h) {
-            if (src[h] < 0 || !((chg[h * kTileWords + (u >> 5)] >> (u & 31)) & 1u)) continue;
-            const uint32_t du = d[h * kTileCap + u], nd = du + len;
-            if (WT && du > T) continue;
-            if (WT && (nd < du || nd == kInf)) {
-                J.ctl->band_ovf = 1;
-                continue;
+        for (int y = 0; y < 2; ++y) {
+            const int x = x0 + 32 * y + lane;
+            const bool in = x < ext;
+            int u = 0;
+            uint32_t len = 1u;
+            v[y] = 0;
+            if (in && x < kExt) {
+                u = C.etail[x];
+                v[y] = C.ecol[x];
+                if (WT) len = C.ew[x];
+            } else if (in) {
+                u = J.g.etail[C.e0 + x];
+                v[y] = J.g.ecol[C.e0 + x];
+                if (WT) len = J.g.ew[C.e0 + x];
             }
-            if (nd < atomicMin(J.dist + src[h] * slots + v, nd)) {
-                pend = min(pend, nd);
-                atomicOr(J.dirty[par ^ 1] + src[h] * words + (v >> 5), 1u << (v & 31));
-                activate(J.g.word_tile[v >> 5], src[h]);
+#pragma unroll
+            for (int h = 0; h < kPair; ++h) {
+                const int q = 2 * y + h;
+                go[q] = in && src[h] >= 0 &&
+                        ((chg[h * kWords + (u >> 5)] >> (u & 31)) & 1u) != 0u;
+                const uint32_t du = go[q] ? d[h * kCap + u] : 0u;
+                nd[q] = du + len;
+                if (WT && go[q]) {
+                    if (du > T) go[q] = false;
+                    else if (nd[q] < du || nd[q] == kInf) {
+                        J.ctl->band_ovf = 1;
+                        go[q] = false;
+                    }
+                }
             }
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            old[q] = 0u;
+            if (go[q]) old[q] = atomicMin(J.dist + src[q & 1] * slots + v[q >> 1], nd[q]);
+        }
+        uint32_t before[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            go[q] = go[q] && nd[q] < old[q];
+            before[q] = 1u;
+            if (go[q]) {
+                const int s = src[q & 1];
+                const int32_t vv = v[q >> 1];
+                pend = min(pend, nd[q]);
+                atomicOr(J.dirty[par ^ 1] + s * words + (vv >> 5), 1u << (vv & 31));
+                before[q] = activate(J.g.word_tile[vv >> 5], s);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (go[q]) queue_unit(J.g.word_tile[v[q >> 1] >> 5], src[q & 1], before[q]);
     }
     if (WT) {
         pend = __reduce_min_sync(FULL, pend);
@@ -493,16 +596,17 @@ __device__ __forceinline__ void tile_sources(const TileJob &J, TileShared<WT> &S
     __syncwarp();
 }
 
-// Units (a tile, up to 256 sources) of a round are popped by the CTAs; a CTA
-// loads the tile's arcs once and its warps take the unit's active sources
-// two by two.
+// Units of a round (a tile, up to 32 uw sources) go to the CTAs: the first
+// ones dealt out, the rest taken from a counter.  A CTA loads the tile's arcs
+// once and its warps take the unit's active sources two by two.
 template <bool WT>
-__global__ void __launch_bounds__(kT, WT ? 3 : 4) k_tiles(TileJob J)
+__global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    TileShared<WT> &S = *reinterpret_cast<TileShared<WT> *>(s_raw);
+    TileShared<WT> &Cs = *reinterpret_cast<TileShared<WT> *>(s_raw);
+    TileWarp<WT> &S = Cs.warp[threadIdx.x >> 5];
     __shared__ int32_t s_buf[kStage];
-    __shared__ unsigned s_cnt, s_base, s_pop, s_next, s_pend, s_mask[kUnitWords];
+    __shared__ unsigned s_cnt, s_base, s_pend, s_pop, s_next, s_mask[kUnitWords];
     const Stage stage{s_buf, &s_cnt, &s_base};
     const int lane = threadIdx.x & 31;
     const int64_t gthreads = (int64_t)gridDim.x * kT;
@@ -555,41 +659,43 @@ __global__ void __launch_bounds__(kT, WT ? 3 : 4) k_tiles(TileJob J)
             ctl->lev[(r + 2) & 3].mlen = 0;  // the complement of its smallest label
         }
         if (threadIdx.x == 0) s_pend = kInf;
+        __syncthreads();
         int32_t *Qn = J.Q[par ^ 1];
         unsigned *qlen = &ctl->lev[(r + 1) & 3].qlen;
-        for (;;) {
-            if (threadIdx.x == 0) {
-                const unsigned p = atomicAdd(&C->hnext, 1u);
-                s_pop = p < qn ? (unsigned)__ldcg(J.Q[par] + p) : ~0u;
-                s_next = 0u;
-            }
-            __syncthreads();
-            const unsigned unit = s_pop;
-            if (unit == ~0u) break;
+        for (unsigned p = blockIdx.x; p < qn;) {
+            const unsigned unit = (unsigned)__ldcg(J.Q[par] + p);
             const int t = (int)(unit / (unsigned)J.ku), w0 = (int)(unit % (unsigned)J.ku) * J.uw;
+            if (threadIdx.x == 0) {
+                s_next = 0u;
+                s_pop = qn > gridDim.x ? gridDim.x + atomicAdd(&C->hnext, 1u) : qn;
+            }
             if (threadIdx.x < kUnitWords) {
+                const int w = w0 + (int)threadIdx.x;
                 unsigned m = 0u;
-                if ((int)threadIdx.x < J.uw && w0 + (int)threadIdx.x < J.kw) {
-                    uint32_t *p = J.act[par] + (int64_t)t * J.kw + w0 + threadIdx.x;
-                    m = __ldcg(p);
-                    if (m) *p = 0u;
+                if ((int)threadIdx.x < J.uw && w < J.kw) {
+                    uint32_t *act = J.act[par] + (int64_t)t * J.kw + w;
+                    m = __ldcg(act);
+                    if (m) *act = 0u;
                 }
                 s_mask[threadIdx.x] = m;
             }
-            const int32_t s0 = J.g.tb[t], nw = (J.g.tb[t + 1] - s0) >> 5;
-            const uint32_t a0 = J.g.irp[s0], e0 = J.g.erp[s0];
-            const int arcs = (int)(J.g.irp[s0 + 32 * nw] - a0);
-            const TileUnit U{s0, nw, e0, (int)(J.g.erp[s0 + 32 * nw] - e0)};
-            for (int i = threadIdx.x; i <= 32 * nw; i += kT)
-                S.off[i] = (uint16_t)(J.g.irp[s0 + i] - a0);
-            for (int i = threadIdx.x; i < arcs; i += kT) {
-                S.col[i] = J.g.icol[a0 + i];
-                if (WT) S.w[i] = J.g.iw[a0 + i];
+            const int32_t s0 = J.g.tb[t], size = J.g.tb[t + 1] - s0;
+            const uint32_t e0 = J.g.erp[s0];
+            const int ext = (int)(J.g.erp[s0 + size] - e0);
+            if (threadIdx.x == 0) {
+                Cs.s0 = s0;
+                Cs.nw = size >> 5;
+                Cs.ext = ext;
+                Cs.e0 = e0;
             }
-            for (int i = threadIdx.x; i < U.ext && U.ext <= kExt; i += kT) {
-                S.etail[i] = J.g.etail[e0 + i];
-                S.ecol[i] = J.g.ecol[e0 + i];
-                if (WT) S.ew[i] = J.g.ew[e0 + i];
+            for (int i = threadIdx.x; i < size; i += kT) {
+                Cs.c4[i] = J.g.icol4[s0 + i];
+                if (WT) Cs.w4[i] = J.g.iw4[s0 + i];
+            }
+            for (int i = threadIdx.x; i < ext && i < kExt; i += kT) {
+                Cs.etail[i] = J.g.etail[e0 + i];
+                Cs.ecol[i] = J.g.ecol[e0 + i];
+                if (WT) Cs.ew[i] = J.g.ew[e0 + i];
             }
             __syncthreads();
             for (;;) {
@@ -612,14 +718,15 @@ __global__ void __launch_bounds__(kT, WT ? 3 : 4) k_tiles(TileJob J)
                     m &= m - 1;
                 }
                 if (src[0] < 0) break;
-                tile_sources<WT>(J, S, U, src, T, par, stage, Qn, qlen, (uint32_t)r + 2u,
+                tile_sources<WT>(J, Cs, S, t, src, T, par, stage, Qn, qlen, (uint32_t)r + 2u,
                                  &s_pend, relax);
             }
+            p = s_pop;
             __syncthreads();
         }
+        stage_flush(stage, Qn, qlen);
         if (WT && threadIdx.x == 0 && s_pend != kInf)
             atomicMax(&ctl->lev[(r + 1) & 3].mlen, ~s_pend);
-        stage_flush(stage, Qn, qlen);
         if (!grid_sync(ctl, blockIdx.x, gridDim.x, J.timeout_ns)) return;
     }
     if (lane == 0 && relax) atomicAdd(&ctl->words, relax);
@@ -873,6 +980,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
                 const uint32_t *w, TileGraph &out, bool *ok, cudaStream_t st)
 {
     *ok = false;
+    const int cap = tile_cap(w != nullptr);
     Buf lab, stamp, left, k0, v0, k1, v1, flag, idx, first, tfirst, stats;
     T_RC(lab.alloc(n * 4));
     T_RC(stamp.alloc(n * 4));
@@ -881,8 +989,8 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     T_CK(cudaMemsetAsync(stamp.p, 0xFF, n * 4, st));
     uint32_t step = 0;
     for (int pass = 0; pass < kGrowPasses; ++pass) {
-        k_centres<<<g, kT, 0, st>>>(n, 0x7f4a7c15ull + pass, step++, lab.as<int32_t>(),
-                                    stamp.as<uint32_t>());
+        k_centres<<<g, kT, 0, st>>>(n, (unsigned)(cap / 2), 0x7f4a7c15ull + pass, step++,
+                                    lab.as<int32_t>(), stamp.as<uint32_t>());
         unsigned open = 0;
         T_CK(cudaMemsetAsync(left.p, 0, 4, st));
         for (int h = 0; h < kGrowHops; ++h)
@@ -892,7 +1000,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
         T_CK(cudaStreamSynchronize(st));
         if (open == 0) break;
     }
-    // Nodes sorted by cluster, tiles of at most kTileCap of them.
+    // Nodes sorted by cluster, tiles of at most cap of them.
     T_RC(k0.alloc(n * 8));
     T_RC(v0.alloc(n * 4));
     T_RC(k1.alloc(n * 8));
@@ -916,7 +1024,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     k_cluster_starts<<<g, kT, 0, st>>>(n, keys, flag.as<uint64_t>());
     T_RC(device_scan_u64(flag.as<uint64_t>(), idx.as<uint64_t>(), n, &clusters, st));
     k_cluster_first<<<g, kT, 0, st>>>(n, keys, idx.as<uint64_t>(), first.as<int32_t>());
-    k_tile_starts<<<g, kT, 0, st>>>(n, keys, idx.as<uint64_t>(), first.as<int32_t>(),
+    k_tile_starts<<<g, kT, 0, st>>>(n, keys, idx.as<uint64_t>(), first.as<int32_t>(), cap,
                                     flag.as<uint64_t>());
     T_RC(device_scan_u64(flag.as<uint64_t>(), idx.as<uint64_t>(), n, &tiles, st));
     k_tile_first<<<g, kT, 0, st>>>(n, flag.as<uint64_t>(), idx.as<uint64_t>(),
@@ -925,7 +1033,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
                                                          flag.as<uint64_t>());
     T_RC(device_scan_u64(flag.as<uint64_t>(), idx.as<uint64_t>(), (int64_t)tiles, &words, st));
     const int64_t slots = (int64_t)words * 32;
-    Buf perm, iperm, tb, wt, irp, erp, icol, ecol, etail, iw, ew, din, dex;
+    Buf perm, iperm, tb, wt, irp, erp, icol, ecol, etail, iw, ew, icol4, iw4, din, dex;
     if (slots > 0x7FFFFFE0LL) return CC_OK;
     T_RC(perm.alloc(slots * 4));
     T_RC(iperm.alloc(n * 4));
@@ -949,6 +1057,8 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     T_RC(icol.alloc(in * 2));
     T_RC(ecol.alloc(ex * 4));
     T_RC(etail.alloc(ex * 2));
+    T_RC(icol4.alloc(slots * 8));
+    if (w) T_RC(iw4.alloc(slots * 16));
     if (w) {
         T_RC(iw.alloc(in * 4));
         T_RC(ew.alloc(ex * 4));
@@ -957,10 +1067,11 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
                                    wt.as<int32_t>(), tb.as<int32_t>(), rp, col, w,
                                    din.as<uint64_t>(), dex.as<uint64_t>(), irp.as<uint32_t>(),
                                    erp.as<uint32_t>(), icol.as<uint16_t>(), ecol.as<int32_t>(),
-                                   etail.as<uint16_t>(), iw.as<uint32_t>(), ew.as<uint32_t>());
+                                   etail.as<uint16_t>(), iw.as<uint32_t>(), ew.as<uint32_t>(),
+                                   icol4.as<ushort4>(), iw4.as<uint4>());
     k_tile_stats<<<(int)std::min<uint64_t>(tiles, 152 * 8), 128, 0, st>>>(
-        (int64_t)tiles, tb.as<int32_t>(), wt.as<int32_t>(), irp.as<uint32_t>(),
-        erp.as<uint32_t>(), ecol.as<int32_t>(), stats.as<unsigned long long>());
+        (int64_t)tiles, tb.as<int32_t>(), wt.as<int32_t>(), erp.as<uint32_t>(),
+        ecol.as<int32_t>(), stats.as<unsigned long long>());
     T_CK(cudaMemsetAsync(lab.p, 0xFF, tiles * 4, st));
     k_tile_depth<<<1, 1024, 0, st>>>(tb.as<int32_t>(), wt.as<int32_t>(), erp.as<uint32_t>(),
                                      ecol.as<int32_t>(), lab.as<int32_t>(), first.as<int32_t>(),
@@ -969,7 +1080,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     T_CK(cudaMemcpyAsync(h, stats.p, 32, cudaMemcpyDeviceToHost, st));
     T_CK(cudaStreamSynchronize(st));
     T_CK(cudaGetLastError());
-    if (h[0] > (unsigned long long)kTileArcs || (double)h[1] > kMaxNeighbours * (double)tiles)
+    if ((double)h[1] > kMaxNeighbours * (double)tiles)
         return CC_OK;
     out.n = n;
     out.slots = slots;
@@ -985,6 +1096,8 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     out.icol = icol.take<uint16_t>();
     out.ecol = ecol.take<int32_t>();
     out.etail = etail.take<uint16_t>();
+    out.icol4 = icol4.take<ushort4>();
+    out.iw4 = iw4.take<uint4>();
     out.iw = iw.take<uint32_t>();
     out.ew = ew.take<uint32_t>();
     *ok = true;
@@ -993,7 +1106,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
 
 void tiles_free(TileGraph &g)
 {
-    void *p[] = {g.perm, g.iperm, g.tb, g.word_tile, g.irp, g.erp, g.icol, g.ecol, g.etail, g.iw, g.ew};
+    void *p[] = {g.perm, g.iperm, g.tb, g.word_tile, g.irp, g.erp, g.icol, g.ecol, g.etail, g.iw, g.ew, g.icol4, g.iw4};
     for (void *x : p)
         if (x) cudaFree(x);
     g = TileGraph{};

@@ -9,9 +9,12 @@
 
 namespace ccg {
 
-constexpr int kTileCap = 512;      // nodes of a tile at most
-constexpr int kTileMean = 256;     // nodes per cluster centre
-constexpr int kTileArcs = 2048;    // arcs inside a tile at most
+// Nodes of a tile at most (a cluster centre stands for half as many).  Larger
+// tiles take fewer rounds, smaller ones leave room for more CTAs with their
+// arcs' lengths and correct fewer labels twice: 1024^2 grid, k = 256, 512 /
+// 384 / 256: 17.5 / 19.4 / 24.5 ms an estimate; road-like lattice, 491 K
+// nodes, k = 64: 18.8 / 13.1 / 15.4 ms.
+constexpr int tile_cap(bool lengths) { return lengths ? 384 : 512; }
 constexpr int kUnitWords = 8;      // words of 32 sources a CTA takes at once
 
 // A graph cut into tiles of neighbouring nodes.  Slots are the nodes' numbers
@@ -27,6 +30,8 @@ struct TileGraph {
     uint16_t *icol = nullptr;                    // head's slot within the tile
     int32_t *ecol = nullptr;                     // head's slot
     uint16_t *etail = nullptr;                   // tail's slot within the tile
+    ushort4 *icol4 = nullptr;                    // inside rows of up to four arcs inline
+    uint4 *iw4 = nullptr;                        // and their lengths
     uint32_t *iw = nullptr, *ew = nullptr;       // their lengths (null: unit lengths)
 };
 
