@@ -38,11 +38,14 @@ constexpr int kReachDefaultW = 8;
 // buckets, 391 / 435 ms).
 constexpr double kDeltaMult = 96.0;
 // Tiles pay from about a thousand nodes and, on unit lengths, sixty-four
-// levels on (a level of the bit-packed search costs about 15 us, a round of
-// tiles, which goes on by twenty, about as much): MEASURE.
+// levels on: a level of the bit-packed search costs about 15 us and a round of
+// tiles, which goes on by twenty levels, 30 to 160 (1024^2 grid, k = 256: 1,963
+// levels 85 ms, 90 rounds 16 ms; with arc lengths, 491 K nodes, k = 64: 1,400
+// rounds of buckets 35 ms, 125 rounds of tiles 10 ms).
 constexpr int64_t kTileMinNodes = 1024;
 constexpr double kTileMinLevels = 64.0;
-// Mean arc lengths that a round's threshold moves on by: MEASURE2.
+// Mean arc lengths that a round's threshold moves on by (road-like lattice, 491
+// K nodes, k = 64, before the last cuts: 6 -> 14.0 ms, 10 -> 13.2, 14 -> 14.2).
 constexpr double kTileDelta = 10.0;
 constexpr double kMaxHistBytes = 4.0 * (1ull << 30);  // distance histogram cap
 

@@ -318,7 +318,11 @@ k_tile_depth(const int32_t *tb, const int32_t *word_tile, const uint32_t *erp,
 
 // ---- the search -----------------------------------------------------------
 
-constexpr int kWarps = kT / 32;
+// Threads of a CTA of the search: a unit of the road-like lattice keeps two to
+// four warps busy (64 sources), one of the grid six (256 sources); 256 / 128
+// / 64 threads: grid 17.6 / 17.8 / 22.4 ms, road-like 13.2 / 10.4 / 12.2 ms.
+template <bool WT>
+constexpr int kTileThreads = WT ? 128 : 256;
 constexpr int kPair = 2;       // sources a warp takes together
 constexpr int kList = 192;     // labels to carry on that a list holds
 
@@ -337,7 +341,7 @@ struct TileWarp {
 constexpr int kExt = 256;
 template <bool WT>
 struct TileShared {
-    TileWarp<WT> warp[kWarps];
+    TileWarp<WT> warp[kTileThreads<WT> / 32];
     uint4 w4[WT ? tile_cap(WT) : 1];
     ushort4 c4[tile_cap(WT)];
     int32_t ecol[kExt];
@@ -600,8 +604,9 @@ __device__ __forceinline__ void tile_sources(const TileJob &J, const TileShared<
 // ones dealt out, the rest taken from a counter.  A CTA loads the tile's arcs
 // once and its warps take the unit's active sources two by two.
 template <bool WT>
-__global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
+__global__ void __launch_bounds__(kTileThreads<WT>, WT ? 6 : 4) k_tiles(TileJob J)
 {
+    constexpr int kTT = kTileThreads<WT>;
     extern __shared__ __align__(16) unsigned char s_raw[];
     TileShared<WT> &Cs = *reinterpret_cast<TileShared<WT> *>(s_raw);
     TileWarp<WT> &S = Cs.warp[threadIdx.x >> 5];
@@ -609,8 +614,8 @@ __global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
     __shared__ unsigned s_cnt, s_base, s_pend, s_pop, s_next, s_mask[kUnitWords];
     const Stage stage{s_buf, &s_cnt, &s_base};
     const int lane = threadIdx.x & 31;
-    const int64_t gthreads = (int64_t)gridDim.x * kT;
-    const int64_t gtid = (int64_t)blockIdx.x * kT + threadIdx.x;
+    const int64_t gthreads = (int64_t)gridDim.x * kTT;
+    const int64_t gtid = (int64_t)blockIdx.x * kTT + threadIdx.x;
     const int64_t slots = J.g.slots, words = slots >> 5;
     Ctl *ctl = J.ctl;
     if (threadIdx.x == 0) s_cnt = 0;
@@ -688,11 +693,11 @@ __global__ void __launch_bounds__(kT, 4) k_tiles(TileJob J)
                 Cs.ext = ext;
                 Cs.e0 = e0;
             }
-            for (int i = threadIdx.x; i < size; i += kT) {
+            for (int i = threadIdx.x; i < size; i += kTT) {
                 Cs.c4[i] = J.g.icol4[s0 + i];
                 if (WT) Cs.w4[i] = J.g.iw4[s0 + i];
             }
-            for (int i = threadIdx.x; i < ext && i < kExt; i += kT) {
+            for (int i = threadIdx.x; i < ext && i < kExt; i += kTT) {
                 Cs.etail[i] = J.g.etail[e0 + i];
                 Cs.ecol[i] = J.g.ecol[e0 + i];
                 if (WT) Cs.ew[i] = J.g.ew[e0 + i];
@@ -766,6 +771,7 @@ __global__ void k_tr_nodes(TileReduce R)
 
 // Per source: exact S, the largest distance, whether a node was not reached.
 constexpr int kSeg = 8192;  // slots per CTA
+constexpr int kWarps = kT / 32;
 
 __global__ void k_tr_sources(TileReduce R)
 {
@@ -1124,18 +1130,19 @@ int launch_tiles(const TileJob &job, cudaStream_t st)
     const int q = job.g.iw ? 1 : 0;
     const void *fn = q ? (const void *)k_tiles<true> : (const void *)k_tiles<false>;
     const size_t smem = q ? sizeof(TileShared<true>) : sizeof(TileShared<false>);
+    const int threads = q ? kTileThreads<true> : kTileThreads<false>;
     if (per[q] < 0) {
         int dev = 0, b = 0;
         T_CK(cudaGetDevice(&dev));
         T_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         T_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        T_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kT, smem));
+        T_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem));
         if (b < 1) return CC_ERR_CUDA;
         per[q] = b;
     }
     TileJob j = job;
     void *args[] = {&j};
-    T_CK(cudaLaunchCooperativeKernel(fn, dim3(per[q] * sms), dim3(kT), args, smem, st));
+    T_CK(cudaLaunchCooperativeKernel(fn, dim3(per[q] * sms), dim3(threads), args, smem, st));
     return CC_OK;
 }
 
