@@ -14,6 +14,7 @@
 #include "estimate.h"
 #include "graph_gpu.h"
 #include "nodew.h"
+#include "planes.h"
 #include "reach.h"
 #include "sssp.h"
 #include "tiles.h"
@@ -195,6 +196,11 @@ struct cc_graph {
     // search's rows and queues.  on_tiles: the last first pass ran on them.
     TileGraph tg;
     bool has_tiles = false, on_tiles = false;
+    // Distances as bit planes (planes.cu).  on_planes: the last first pass
+    // left them (on distance rows); deep: a pass found more levels than they
+    // hold, so that the next call does not try first.
+    DevBuf pl_F, pl_R, pl_masks, pl_c;
+    bool on_planes = false, deep = false;
     DevBuf t_dist, t_dirty0, t_dirty1, t_act0, t_act1, t_stamp, t_Q0, t_Q1;
     // workspace
     DevBuf vis, F0, F1, nxt, Q0, Q1, T, tflag, sidx, sum2, pivot, delta, lc2, Lmask, hp,
@@ -630,7 +636,7 @@ void free_graph(cc_graph *g)
         for (DevBuf *b : csr) { b->p = nullptr; b->cap = 0; }
     }
     if (!g->borrowed) tiles_free(g->tg);
-    DevBuf *all[] = {&g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1, &g->t_stamp,
+    DevBuf *all[] = {&g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1, &g->t_stamp,
                      &g->t_Q0, &g->t_Q1, &g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
                      &g->lw_perm, &g->lw_iperm, &g->lw_src, &g->fw.cls.L, &g->fw.cls.M,
                      &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
@@ -685,7 +691,9 @@ int prepare_sq(cc_graph *g, int k, cudaStream_t st)
 // per-source level histogram and the exact S of the sampled nodes.
 // With eps_a > 0 the pass also classifies each arriving bit for the hybrid
 // of eps = eps_a / eps_b (RED_BAND), so that no second pass is needed.
-int bfs_pass1(cc_graph *g, int k, cudaStream_t st, uint32_t eps_a = 0, uint32_t eps_b = 0)
+// With planes it also keeps the distances as bit planes.
+int bfs_pass1(cc_graph *g, int k, cudaStream_t st, uint32_t eps_a = 0, uint32_t eps_b = 0,
+              bool planes = false)
 {
     const int64_t n = g->n;
     const int W = pow2_words(k);
@@ -707,6 +715,11 @@ int bfs_pass1(cc_graph *g, int k, cudaStream_t st, uint32_t eps_a = 0, uint32_t 
         j.lc2 = g->hc2.as<uint64_t>();  // the sums over HC(v) settled on arrival
         j.eps_a = eps_a;
         j.eps_b = eps_b;
+    }
+    if (planes) {
+        RC(g->pl_F.ensure((size_t)n * W * kPlanes * 8));
+        j.red |= RED_PLANES;
+        j.planes = g->pl_F.as<uint64_t>();
     }
     j.pivot = g->pivot.as<int32_t>();
     j.delta = g->delta.as<uint32_t>();
@@ -748,10 +761,61 @@ int check_pass1(cc_graph *g, bool hybrid, int k)
     return CC_OK;
 }
 
+// Whether `sets` sets of planes fit a third of the memory that is free or
+// already held by them.
+bool planes_fit(cc_graph *g, int k, int sets)
+{
+    const double need = (double)sets * (double)g->n * pow2_words(k) * kPlanes * 8.0;
+    const double held = (double)g->pl_F.cap + (double)g->pl_R.cap;
+    if (held >= need) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return need <= ((double)free_b + held) / 3.0;
+}
+
+// The job of the plane kernels; sizes the masks of the hybrid part.
+int plane_job(cc_graph *g, int k, bool roundtrip, PlaneJob &j)
+{
+    const int W = pow2_words(k);
+    RC(g->pl_masks.ensure((size_t)k * plane_rows(roundtrip) * W * 8));
+    RC(g->pl_c.ensure((size_t)k * W * 5 * 8));
+    std::memset(&j, 0, sizeof(j));
+    j.n = g->n;
+    j.k = k;
+    j.W = W;
+    j.F = g->pl_F.as<uint64_t>();
+    j.R = roundtrip ? g->pl_R.as<uint64_t>() : nullptr;
+    j.sources = g->sources.as<int32_t>();
+    j.sidx = g->sidx.as<int32_t>();
+    j.sum2 = g->sum2.as<uint64_t>();
+    j.pivot = g->pivot.as<int32_t>();
+    j.delta = g->delta.as<uint32_t>();
+    j.dcc = g->dcc.as<uint32_t>();
+    j.masks = g->pl_masks.as<uint64_t>();
+    j.cplanes = g->pl_c.as<uint64_t>();
+    j.hp = g->hp.as<HybPrep>();
+    j.lc2 = g->lc2.as<uint64_t>();
+    if (g->sq) {
+        j.sqflag = g->sqflag.as<uint8_t>();
+        j.istar = g->istar.as<int32_t>();
+        j.hcse = g->hcse.as<uint64_t>();
+        j.fdist = g->fdist.as<uint32_t>();
+    }
+    return CC_OK;
+}
+
+// How the hybrid part after bfs_pass1 gets LCsum: by a second pass, from the
+// first pass's classification on arrival, from its planes (the second pass
+// queued in case they overflowed), or from planes known not to have.
+enum class Lc { kPass, kBand, kPlanes, kPlanesOnly };
+
 // The hybrid part of the bit-packed path for eps = a/b, after bfs_pass1:
 // H statistics from the histogram tails, thresholds, L-masks and, where
 // needed, the second pass.
-int bfs_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st, bool band = false)
+int bfs_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st, Lc lc = Lc::kPass)
 {
     const int64_t n = g->n;
     const int W = pow2_words(k);
@@ -787,7 +851,21 @@ int bfs_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st, bool
     // classified on arrival, LCsum is complete once the deferred bits are
     // resolved, and the second pass runs only if a band offset overflowed.
     const unsigned *gate = g->npartial.as<unsigned>();
-    if (band) {
+    if (lc == Lc::kPlanes || lc == Lc::kPlanesOnly) {
+        PlaneJob pj;
+        RC(plane_job(g, k, false, pj));
+        if (lc == Lc::kPlanes) {
+            RC(g->gate2.ensure(8));
+            pj.ovf = &g->ctl.as<Ctl>()->band_ovf;
+            pj.npartial = g->npartial.as<unsigned>();
+            pj.gate = g->gate2.as<unsigned>();
+            gate = g->gate2.as<unsigned>();
+        }
+        run_planes_lc(pj, st);
+        g->call_kernels += 2;
+        if (lc == Lc::kPlanesOnly) return CC_OK;
+    }
+    if (lc == Lc::kBand) {
         RC(g->gate2.ensure(8));
         run_band_resolve(n, k, 64 * W, g->sidx.as<int32_t>(), g->pivot.as<int32_t>(),
                          g->delta.as<uint32_t>(), g->dcc.as<uint32_t>(), g->hp.as<HybPrep>(),
@@ -841,9 +919,11 @@ bool use_band(cc_graph *g, int k, const cc_opts *opts)
 
 int estimate_bfs(cc_graph *g, int k, const cc_opts *opts, bool band, cudaStream_t st)
 {
-    RC(bfs_pass1(g, k, st, band ? opts->eps_num : 0, band ? opts->eps_den : 0));
+    const bool planes = opts->want_hybrid && g->sq && !g->band_off && planes_fit(g, k, 1);
+    RC(bfs_pass1(g, k, st, band ? opts->eps_num : 0, band ? opts->eps_den : 0, planes));
     if (!opts->want_hybrid) return CC_OK;
-    return bfs_hybrid(g, k, opts->eps_num, opts->eps_den, st, band);
+    return bfs_hybrid(g, k, opts->eps_num, opts->eps_den, st,
+                      band ? Lc::kBand : planes ? Lc::kPlanes : Lc::kPass);
 }
 
 // One chunk of shortest paths (forward, and reversed for round trips)
@@ -1323,10 +1403,120 @@ int tiled_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
     return CC_OK;
 }
 
+// Whether the distances from k sources are worth trying as planes: unit
+// lengths, not known (or, on tiles, bound) to be too many levels.
+bool use_planes(cc_graph *g, int k)
+{
+    return !g->weighted && !g->deep && !(g->has_tiles && g->tg.levels >= kTileMinLevels) &&
+           planes_fit(g, k, g->directed ? 2 : 1);
+}
+
+// First pass of all k sources into planes, both ways on a directed graph,
+// reduced into sums, pivots, Delta and delta_cc; waits.  Returns 1 when the
+// planes overflowed (the rows take over).
+int planes_pass1(cc_graph *g, int k, cudaStream_t st)
+{
+    const int64_t n = g->n;
+    const int W = pow2_words(k), dirs = g->directed ? 2 : 1;
+    const size_t bytes = (size_t)n * W * kPlanes * 8;
+    RC(ensure_state(g, W));
+    RC(g->pl_F.ensure(bytes));
+    if (dirs == 2) RC(g->pl_R.ensure(bytes));
+    RC(g->dmax.ensure(8));
+    const DevCSR &gt = g->directed ? g->rv : g->fw;
+    for (int dir = 0; dir < dirs; ++dir) {
+        BfsJob j = base_job(g, W, dir ? gt : g->fw, dir ? g->fw : gt);
+        j.k = k;
+        j.sources = g->sources.as<int32_t>();
+        j.red = RED_PLANES;
+        j.planes = (dir ? g->pl_R : g->pl_F).as<uint64_t>();
+        RC(queue_pass(g, dir, W, j, st));
+    }
+    PlaneJob pj;
+    RC(plane_job(g, k, g->directed, pj));
+    pj.dmax = g->dmax.as<unsigned long long>();
+    CK(cudaMemsetAsync(g->dmax.p, 0, 8, st));
+    run_planes_nodes(pj, st);
+    CK(cudaGetLastError());
+    g->call_kernels += 2;
+    unsigned long long dmax = 0;
+    CK(cudaMemcpyAsync(&dmax, g->dmax.p, 8, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    RC(settle_passes(g));
+    for (int dir = 0; dir < dirs; ++dir)
+        if (g->hctl[dir].band_ovf) {
+            g->deep = true;
+            return 1;
+        }
+    for (int dir = 0; dir < dirs; ++dir)
+        if (g->hctl[dir].ninc_final != 0) return CC_ERR_DISCONNECTED;
+    g->dist_max = (int64_t)dmax;
+    g->D1 = (int64_t)dmax;
+    return CC_OK;
+}
+
+// ... and the level histogram with the exact S of the sampled nodes.
+int planes_hist(cc_graph *g, int k, cudaStream_t st)
+{
+    const size_t bytes = (size_t)(g->D1 + 1) * k * 4;
+    RC(g->hist.ensure(bytes));
+    CK(cudaMemsetAsync(g->hist.p, 0, bytes, st));
+    PlaneJob pj;
+    RC(plane_job(g, k, g->directed, pj));
+    pj.hist = g->hist.as<uint32_t>();
+    pj.D = g->D1;
+    run_planes_hist(pj, st);
+    run_S_sampled(g->hist.as<uint32_t>(), DevCount{nullptr, g->D1}, k, g->dcc.as<uint32_t>(),
+                  g->Ssamp.as<uint64_t>(), st);
+    CK(cudaGetLastError());
+    g->call_kernels += 2;
+    return CC_OK;
+}
+
+// The hybrid part for eps = a/b after planes_pass1 and planes_hist.
+int planes_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
+{
+    const int64_t n = g->n, D = g->D1;
+    RC(g->TN.ensure((size_t)k * (D + 1) * 8));
+    RC(g->TS.ensure((size_t)k * (D + 1) * 8));
+    RC(g->maxd.ensure((size_t)k * 4));
+    RC(g->hp.ensure((size_t)n * sizeof(HybPrep)));
+    RC(g->npartial.ensure(8));
+    RC(g->lc2.ensure(n * 16));
+    CK(cudaMemsetAsync(g->npartial.p, 0, 8, st));
+    run_tail(g->hist.as<uint32_t>(), DevCount{nullptr, D}, D + 1, k, g->TN.as<uint64_t>(),
+             g->TS.as<uint64_t>(), st);
+    run_maxdelta(g->dcc.as<uint32_t>(), k, g->maxd.as<uint32_t>(), st);
+    SqPrep sq{nullptr};
+    if (g->sq) {
+        RC(prepare_sq(g, k, st));
+        sq.flag = g->sqflag.as<uint8_t>();
+    }
+    run_hyb_prep(3, n, k, DevCount{nullptr, D}, D + 1, a, b, g->sidx.as<int32_t>(),
+                 g->pivot.as<int32_t>(), g->delta.as<uint32_t>(), g->dcc.as<uint32_t>(),
+                 g->maxd.as<uint32_t>(), g->TN.as<uint64_t>(), g->TS.as<uint64_t>(),
+                 g->hp.as<HybPrep>(), g->npartial.as<unsigned>(), sq, st);
+    PlaneJob pj;
+    RC(plane_job(g, k, g->directed, pj));
+    run_planes_lc(pj, st);
+    CK(cudaGetLastError());
+    g->call_kernels += 5;
+    return CC_OK;
+}
+
 // First pass and hybrid part on distance rows: tiles where the graph has
-// them (g->on_tiles tells which ran last), else chunks.
+// them (g->on_tiles tells which ran last), planes (g->on_planes), else chunks.
 int rows_pass1(cc_graph *g, int k, cudaStream_t st)
 {
+    g->on_planes = false;
+    if (g->directed && use_planes(g, k)) {
+        const int rc = planes_pass1(g, k, st);
+        if (rc == CC_OK) {
+            g->on_planes = true;
+            return planes_hist(g, k, st);
+        }
+        if (rc != 1) return rc;
+    }
     g->on_tiles = use_tiles(g, k);
     if (g->on_tiles) {
         const int rc = tiled_pass1(g, k, st);
@@ -1338,7 +1528,9 @@ int rows_pass1(cc_graph *g, int k, cudaStream_t st)
 
 int rows_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
 {
-    return g->on_tiles ? tiled_hybrid(g, k, a, b, st) : chunked_hybrid(g, k, a, b, st);
+    return g->on_planes  ? planes_hybrid(g, k, a, b, st)
+           : g->on_tiles ? tiled_hybrid(g, k, a, b, st)
+                         : chunked_hybrid(g, k, a, b, st);
 }
 
 int estimate_chunked(cc_graph *g, int k, const cc_opts *opts, cudaStream_t st)
@@ -1652,7 +1844,7 @@ int ccg::graph_ready_to_borrow(cc_graph_t g) { return ensure_locality(g); }
 
 size_t ccg::graph_workspace_bytes(cc_graph_t g)
 {
-    const DevBuf *ws[] = {&g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1,
+    const DevBuf *ws[] = {&g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1,
                           &g->t_stamp, &g->t_Q0, &g->t_Q1, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1, &g->T, &g->tflag,
                           &g->sidx, &g->sum2, &g->pivot, &g->delta, &g->lc2, &g->Lmask, &g->hp,
                           &g->dcc, &g->hist, &g->TN, &g->TS, &g->Ssamp, &g->maxd, &g->sources,
@@ -1692,10 +1884,11 @@ int ccg::estimate_resident(cc_graph_t g, int32_t k, const cc_opts *opts, cc_out 
     int rc = CC_OK;
     if (hyb) {
         if (chunked) {
-            rc = chunked_hybrid(g, k, opts->eps_num, opts->eps_den, st);
+            rc = rows_hybrid(g, k, opts->eps_num, opts->eps_den, st);
         } else {
             const bool band = !g->sq && g->band_a == opts->eps_num && g->band_b == opts->eps_den;
-            rc = bfs_hybrid(g, k, opts->eps_num, opts->eps_den, st, band);
+            rc = bfs_hybrid(g, k, opts->eps_num, opts->eps_den, st,
+                            band ? Lc::kBand : Lc::kPass);
         }
     }
     if (rc == CC_OK) rc = finish_outputs(g, k, hyb, opts, out, st);  // synchronises
@@ -2072,11 +2265,13 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     g->call_kernels += 2;
     g->on_tiles = use_tiles(g, k);
     const bool chunked = on_rows(g);
+    bool planes = false;
     if (chunked) {
         RC(rows_pass1(g, k, st));
     } else {
+        planes = planes_fit(g, k, 1);
         for (;;) {
-            RC(bfs_pass1(g, k, st));
+            RC(bfs_pass1(g, k, st, 0, 0, planes));
             CK(cudaStreamSynchronize(st));
             RC(settle_passes(g));
             const int c1 = check_pass1(g, true, k);
@@ -2084,12 +2279,14 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
             RC(c1);
             break;
         }
+        planes = planes && !g->hctl[0].band_ovf;
     }
     g->sq = true;
     for (int e = 0; e < n_eps; ++e) {
         RC(chunked ? rows_hybrid(g, k, eps_num[e], eps_den[e], st)
-                   : bfs_hybrid(g, k, eps_num[e], eps_den[e], st));
-        if (!chunked) {
+                   : bfs_hybrid(g, k, eps_num[e], eps_den[e], st,
+                                planes ? Lc::kPlanesOnly : Lc::kPass));
+        if (!chunked && !planes) {
             CK(cudaStreamSynchronize(st));
             RC(settle_passes(g));
         }
@@ -2247,9 +2444,34 @@ int cc_estimate_node_weighted(cc_graph_t g, const int32_t *sample, int32_t k,
     j.sidx = g->sidx.as<int32_t>();
     j.wsum = g->nw_wsum.as<uint64_t>();
     j.S = g->nw_S.as<unsigned long long>();
-    RC(chunked_pass1(g, k, st, &j));  // binds the distance rows it allocates
-    j.distF = g->distF.as<uint32_t>();
-    j.distR = g->directed ? g->distR.as<uint32_t>() : nullptr;
+    // On unit lengths the distances as planes while they fit; else the rows.
+    g->sq = false;
+    bool planes = use_planes(g, k);
+    PlaneJob pj;
+    if (planes) {
+        RC(g->sum2.ensure(n * 16));
+        const int rc = planes_pass1(g, k, st);
+        if (rc == 1) planes = false;
+        else RC(rc);
+    }
+    if (planes) {
+        RC(plane_job(g, k, g->directed, pj));
+        pj.beta = j.beta;
+        pj.bsrc = j.bsrc;
+        pj.mu = j.mu;
+        pj.tau = g->nw_tau.as<uint64_t>();
+        pj.wsum = j.wsum;
+        pj.S = j.S;
+        pj.eps_a = opts->eps_num;
+        pj.eps_b = opts->eps_den;
+        pj.D = g->D1;
+        run_planes_nw1(pj, st);
+        g->call_kernels += 2;
+    } else {
+        RC(chunked_pass1(g, k, st, &j));  // binds the distance rows it allocates
+        j.distF = g->distF.as<uint32_t>();
+        j.distR = g->directed ? g->distR.as<uint32_t>() : nullptr;
+    }
     uint64_t ms[2] = {0, 0};
     CK(cudaMemcpyAsync(ms, g->nw_msum.p, 16, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -2267,6 +2489,15 @@ int cc_estimate_node_weighted(cc_graph_t g, const int32_t *sample, int32_t k,
         RC(g->nw_lc.ensure((size_t)n * 16));
         CK(cudaMemsetAsync(g->nw_hist.p, 0, (size_t)(D + 1) * k * 8, st));
         CK(cudaMemsetAsync(g->nw_lc.p, 0, (size_t)n * 16, st));
+        if (planes) {
+            pj.lc = g->nw_lc.as<uint64_t>();
+            // Delta >= 1 of every unsampled node: from eps D <= 1 on no node
+            // lies beyond its threshold and the tail is empty.
+            if ((uint64_t)opts->eps_den / opts->eps_num < (uint64_t)D)
+                pj.bhist = g->nw_hist.as<unsigned long long>();
+            run_planes_nw2(pj, st);
+            g->call_kernels += 3;
+        }
         j.pivot = g->pivot.as<int32_t>();
         j.delta = g->delta.as<uint32_t>();
         j.dcc = g->dcc.as<uint32_t>();
@@ -2277,7 +2508,7 @@ int cc_estimate_node_weighted(cc_graph_t g, const int32_t *sample, int32_t k,
         const int cw = g->cw;
         j.ld = cw;
         const int32_t *src = g->sources.as<int32_t>();
-        for (int base = 0; base < k; base += cw) {
+        for (int base = 0; !planes && base < k; base += cw) {
             const int kc = std::min(cw, k - base);
             const size_t off = chunk_offset(g, base);
             if (!g->resident) RC(run_chunk(g, src + base, kc, cw, st, off));

@@ -50,7 +50,12 @@ enum : uint32_t {
     // level's offset in that band, l + Delta(v) - floor(Delta(v) eps_b /
     // eps_a), goes to band[v * 64W + i] (valid once bflag[v] & 1)
     RED_BAND = 128u,
+    // planes[(v W + w) kPlanes + b] gets the bits that arrive on a level with
+    // binary digit b set (zeroed by the pass); a level beyond kPlanes digits
+    // sets band_ovf instead, and ends a pass that does nothing else
+    RED_PLANES = 256u,
 };
+constexpr int kPlanes = 4;  // levels 0 .. 15
 
 // Per-level statistics, indexed by level mod 4 (written during level l,
 // read during l+1 and l+2, cleared during l+3).
@@ -77,7 +82,8 @@ constexpr int kTraceLevels = 64;
 struct Ctl {
     unsigned long long bar_arrive;  // grid barrier arrivals (see barrier.cuh)
     int err;                // 0 or a CC_ERR_* code
-    int band_ovf;           // RED_BAND: some band offset did not fit a byte
+    int band_ovf;           // RED_BAND: some band offset did not fit a byte;
+                            // RED_PLANES: a level did not fit the planes
     unsigned far_len[3];    // shortest paths: lengths of the three far queues
     unsigned long long far_min[3];  // and the smallest label each waits with
     int levels;             // last level that produced new bits
@@ -159,6 +165,7 @@ struct BfsJob {
     uint8_t *band;          // RED_BAND: n x 64W band offsets of deferred bits
     uint8_t *bflag;         // RED_BAND: n, zeroed by the pass
     uint32_t eps_a, eps_b;  // RED_BAND: eps
+    uint64_t *planes;       // RED_PLANES: n x W x kPlanes
     Ctl *ctl;
     uint64_t timeout_ns;
     int alpha;              // top-down while ef * alpha < eu

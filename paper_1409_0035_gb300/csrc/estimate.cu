@@ -54,7 +54,7 @@ __global__ void k_hyb_prep(int mode, int64_t n, int k, DevCount D, int64_t strid
 
 __global__ void k_istar(const uint32_t *dcc, int k, int32_t *istar)
 {
-    d_istar(dcc, k, istar, GSTART, GSTRIDE);
+    d_istar(dcc, k, istar, GSTART >> 5, GSTRIDE >> 5);
 }
 
 __global__ void k_lmask(int64_t n, int W, int k, const int32_t *sidx, const int32_t *pivot,
@@ -221,7 +221,7 @@ void run_closeness(int64_t n, const double *s_hat, double *clo, cudaStream_t st)
 
 void run_istar(const uint32_t *dcc, int k, int32_t *istar, cudaStream_t st)
 {
-    k_istar<<<(k + 127) / 128, 128, 0, st>>>(dcc, k, istar);
+    k_istar<<<(k + 7) / 8, 256, 0, st>>>(dcc, k, istar);
 }
 
 void run_lmask(int64_t n, int W, int k, const int32_t *sidx, const int32_t *pivot,

@@ -114,14 +114,26 @@ __device__ __forceinline__ void d_maxdelta(const uint32_t *dcc, int k, uint32_t 
 // Per sampled node p: the sampled node farthest from it other than itself
 // (ties to the smallest index; p itself when k = 1) -- the stand-in for
 // HC(v) in the error estimate of nodes whose HC(v) is empty (section 4).
+// A warp per row (warp w0 of nw): a thread per row read it alone, 40 us at k =
+// 256 against 3.
 __device__ __forceinline__ void d_istar(const uint32_t *dcc, int k, int32_t *istar,
-                                        int64_t i0, int64_t stride)
+                                        int64_t w0, int64_t nw)
 {
-    for (int64_t p = i0; p < k; p += stride) {
-        int best = (int)p;
-        for (int i = 0; i < k; ++i)
-            if (i != (int)p && (best == (int)p || dcc[p * k + i] > dcc[p * k + best])) best = i;
-        istar[p] = best;
+    const int lane = threadIdx.x & 31;
+    for (int64_t p = w0; p < k; p += nw) {
+        unsigned long long best = 0;  // distance, then the complement of the index
+        for (int i = lane; i < k; i += 32)
+            if (i != (int)p) {
+                const unsigned long long key =
+                    ((unsigned long long)dcc[p * k + i] << 32) | (0xFFFFFFFFu - (unsigned)i);
+                best = key > best ? key : best;
+            }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+            best = y > best ? y : best;
+        }
+        if (lane == 0) istar[p] = best ? (int32_t)(0xFFFFFFFFu - (uint32_t)best) : (int32_t)p;
     }
 }
 

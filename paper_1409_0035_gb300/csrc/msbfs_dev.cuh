@@ -247,6 +247,17 @@ __device__ __forceinline__ void tile_reduce(const BfsJob &J, int l, int v, uint6
             }
         }
     }
+    if ((J.red & RED_PLANES) && nw) {
+        if (l >> kPlanes) {
+            J.ctl->band_ovf = 1;
+        } else {
+            unsigned long long *p = (unsigned long long *)J.planes + vw * kPlanes;
+            if (l & 1) atomicOr(p, (unsigned long long)nw);
+            if (l & 2) atomicOr(p + 1, (unsigned long long)nw);
+            if (l & 4) atomicOr(p + 2, (unsigned long long)nw);
+            if (l & 8) atomicOr(p + 3, (unsigned long long)nw);
+        }
+    }
     if ((J.red & RED_LEVELS) && nw) {
         uint64_t b = nw;
         while (b) {
@@ -784,6 +795,11 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
         for (int64_t v = gtid; v < n; v += gthreads) J.bflag[v] = 0;
     if (J.red & RED_LEVELS)
         for (int64_t i = gtid; i < n * J.dist_ld; i += gthreads) J.dist_out[i] = kInf;
+    if (J.red & RED_PLANES) {
+        ulonglong2 *const p = reinterpret_cast<ulonglong2 *>(J.planes);
+        for (int64_t i = gtid; i < n * W * (kPlanes / 2); i += gthreads)
+            p[i] = make_ulonglong2(0ull, 0ull);
+    }
     if (!sync_after(CC_PH_INIT)) return;
     for (int64_t i = gtid; i < J.k; i += gthreads) {
         const int v = J.sources[i];
@@ -846,6 +862,10 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
         if (qprev == 0 || ninc == 0) break;
         if (doHist && l >= J.hist_cap) {
             if (gtid == 0) atomicCAS(&ctl->err, 0, 1);  // histogram too short
+            break;
+        }
+        if (J.red == RED_PLANES && (l >> kPlanes)) {
+            if (gtid == 0) ctl->band_ovf = 1;
             break;
         }
         const bool td = ef * (unsigned long long)J.alpha < (unsigned long long)eu;
