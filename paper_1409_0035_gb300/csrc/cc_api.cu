@@ -81,10 +81,16 @@ struct DevBuf {
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
-// Degree classes of one CSR for the bottom-up scan.
+// Degree classes of one CSR for the bottom-up scan: the nodes by degree (tiny,
+// light, medium and heavy ones one after another), the heavy ones' chunk
+// tasks.
 struct Classes {
-    DevBuf L, M, H, Hn, Hb, T, Tadj, Nadj;
+    DevBuf order, Hn, Hb, Tadj, Nadj;
     int64_t nL = 0, nM = 0, nH = 0, nHch = 0, nT = 0;
+    const int32_t *T() const { return order.as<int32_t>(); }
+    const int32_t *L() const { return T() + nT; }
+    const int32_t *M() const { return L() + nL; }
+    const int32_t *H() const { return M() + nM; }
 };
 
 // Inline adjacency of the tiny nodes (degree <= kTinyMaxDeg): their
@@ -291,48 +297,25 @@ int upload(DevBuf &b, const void *src, size_t bytes)
     return CC_OK;
 }
 
-int build_classes(const std::vector<int64_t> &rp, int64_t n, Classes &c, const int64_t *drp,
-                  const int32_t *dcol)
+// Tiny, light and medium nodes are ordered by degree (ties by id).  A warp
+// scans W-lane groups of nodes in lock step, so equal degrees keep its lanes
+// busy for the same number of steps; and warps take every nwarps-th entry of
+// a list, so a sorted list hands every warp about the same number of CSR
+// entries.  Tiny nodes (degree <= kTinyMaxDeg) carry their neighbours inline
+// (one int4), which takes two dependent loads out of their scan.
+int build_classes(int64_t n, Classes &c, const int64_t *drp, const int32_t *dcol)
 {
-    // Tiny, light and medium nodes are ordered by degree (stable counting
-    // sort, ties by id).  A warp scans W-lane groups of nodes in lock step,
-    // so equal degrees keep its lanes busy for the same number of steps; and
-    // warps take every nwarps-th entry of a list, so a sorted list hands
-    // every warp about the same number of CSR entries.  Tiny nodes (degree
-    // <= kTinyMaxDeg) carry their neighbours inline (one int4), which takes
-    // two dependent loads out of their scan.
-    std::vector<int64_t> start(kMediumMaxDeg + 2, 0);
-    for (int64_t v = 0; v < n; ++v) {
-        const int64_t d = rp[v + 1] - rp[v];
-        if (d <= kMediumMaxDeg) start[d + 1] += 1;
-    }
-    for (int d = 0; d <= kMediumMaxDeg; ++d) start[d + 1] += start[d];
-    const int64_t ntiny = start[kTinyMaxDeg + 1];
-    const int64_t nlight = start[kLightMaxDeg + 1];
-    std::vector<int32_t> T((size_t)ntiny), L((size_t)(nlight - ntiny)),
-        M((size_t)(start[kMediumMaxDeg + 1] - nlight)), H, Hn;
-    std::vector<int64_t> Hb;
-    for (int64_t v = 0; v < n; ++v) {
-        const int64_t d = rp[v + 1] - rp[v];
-        if (d <= kTinyMaxDeg) T[(size_t)start[d]++] = (int32_t)v;
-        else if (d <= kLightMaxDeg) L[(size_t)(start[d]++ - ntiny)] = (int32_t)v;
-        else if (d <= kMediumMaxDeg) M[(size_t)(start[d]++ - nlight)] = (int32_t)v;
-        else {
-            H.push_back((int32_t)v);
-            for (int64_t b = rp[v]; b < rp[v + 1]; b += kChunk) {
-                Hn.push_back((int32_t)v);
-                Hb.push_back(b);
-            }
-        }
-    }
-    c.nL = (int64_t)L.size(); c.nM = (int64_t)M.size(); c.nH = (int64_t)H.size();
-    c.nHch = (int64_t)Hn.size();
-    c.nT = (int64_t)T.size();
-    RC(upload(c.T, T.data(), T.size() * 4));
+    int64_t counts[5];
+    RC(c.order.ensure((size_t)n * 4));
+    RC(degree_order(n, drp, c.order.as<int32_t>(), counts));
+    c.nT = counts[0]; c.nL = counts[1]; c.nM = counts[2]; c.nH = counts[3]; c.nHch = counts[4];
     RC(c.Tadj.ensure((size_t)std::max<int64_t>(c.nT, 1) * 16));
+    RC(c.Hn.ensure((size_t)c.nHch * 4));
+    RC(c.Hb.ensure((size_t)c.nHch * 8));
+    RC(heavy_chunks(c.H(), c.nH, drp, c.Hn.as<int32_t>(), c.Hb.as<int64_t>()));
     if (c.nT > 0) {
         const int64_t g = std::min<int64_t>((c.nT + 255) / 256, 152 * 32);
-        k_tiny_adj<<<(int)g, 256>>>(c.T.as<int32_t>(), c.nT, drp, dcol, c.Tadj.as<int4>());
+        k_tiny_adj<<<(int)g, 256>>>(c.T(), c.nT, drp, dcol, c.Tadj.as<int4>());
         CK(cudaGetLastError());
         if (2 * c.nT >= n) {
             RC(c.Nadj.ensure((size_t)n * 16));
@@ -340,13 +323,8 @@ int build_classes(const std::vector<int64_t> &rp, int64_t n, Classes &c, const i
                 n, drp, dcol, c.Nadj.as<int4>());
             CK(cudaGetLastError());
         }
-        CK(cudaDeviceSynchronize());  // estimates may run on other streams
     }
-    RC(upload(c.L, L.data(), L.size() * 4));
-    RC(upload(c.M, M.data(), M.size() * 4));
-    RC(upload(c.H, H.data(), H.size() * 4));
-    RC(upload(c.Hn, Hn.data(), Hn.size() * 4));
-    RC(upload(c.Hb, Hb.data(), Hb.size() * 8));
+    CK(cudaDeviceSynchronize());  // estimates may run on other streams
     return CC_OK;
 }
 
@@ -406,9 +384,9 @@ BfsJob base_job(cc_graph *g, int W, const DevCSR &push, const DevCSR &pull)
     j.nadj = push.cls.Nadj.as<int4>();
     j.prp = pull.rp.as<int64_t>();
     j.pcol = pull.col.as<int32_t>();
-    j.Llist = csr.cls.L.as<int32_t>();
-    j.Mlist = csr.cls.M.as<int32_t>();
-    j.Hlist = csr.cls.H.as<int32_t>();
+    j.Llist = csr.cls.L();
+    j.Mlist = csr.cls.M();
+    j.Hlist = csr.cls.H();
     j.nL = csr.cls.nL;
     j.nM = csr.cls.nM;
     j.nH = csr.cls.nH;
@@ -426,7 +404,7 @@ BfsJob base_job(cc_graph *g, int W, const DevCSR &push, const DevCSR &pull)
     j.AL1 = g->AL1.as<int32_t>();
     j.ACH0 = g->ACH0.as<int32_t>();
     j.ACH1 = g->ACH1.as<int32_t>();
-    j.Tlist = csr.cls.T.as<int32_t>();
+    j.Tlist = csr.cls.T();
     j.Tadj = csr.cls.Tadj.as<int4>();
     j.nT = csr.cls.nT;
     j.AT0 = g->AT0.as<int32_t>();
@@ -548,8 +526,7 @@ int adopt_device_reverse(cc_graph *g, DeviceCSR &d)
         g->rv.w.cap = (size_t)std::max<int64_t>(d.arcs, 1) * 4;
     }
     d.rp = d.col = d.w = nullptr;
-    return build_classes(d.rp_host, d.n, g->rv.cls, g->rv.rp.as<int64_t>(),
-                         g->rv.col.as<int32_t>());
+    return build_classes(d.n, g->rv.cls, g->rv.rp.as<int64_t>(), g->rv.col.as<int32_t>());
 }
 
 // Take ownership of a CSR built on the device.
@@ -567,15 +544,16 @@ int adopt_device_csr(cc_graph *g, DeviceCSR &d)
         g->fw.w.cap = (size_t)std::max<int64_t>(d.arcs, 1) * 4;
     }
     d.rp = d.col = d.w = nullptr;
-    return build_classes(d.rp_host, d.n, g->fw.cls, g->fw.rp.as<int64_t>(),
-                         g->fw.col.as<int32_t>());
+    return build_classes(d.n, g->fw.cls, g->fw.rp.as<int64_t>(), g->fw.col.as<int32_t>());
 }
 
 // The breadth-first renumbering of an undirected graph with arc lengths
-// (cc_graph::lw), from the host copy of its row offsets.
-int build_locality(cc_graph *g, const std::vector<int64_t> &rp)
+// (cc_graph::lw).
+int build_locality(cc_graph *g)
 {
     const int64_t n = g->n, arcs = g->arcs;
+    std::vector<int64_t> rp((size_t)n + 1);
+    CK(cudaMemcpy(rp.data(), g->fw.rp.p, rp.size() * 8, cudaMemcpyDeviceToHost));
     std::vector<int32_t> col((size_t)arcs);
     if (arcs) CK(cudaMemcpy(col.data(), g->fw.col.p, (size_t)arcs * 4, cudaMemcpyDeviceToHost));
     std::vector<int32_t> perm, iperm((size_t)n);
@@ -607,9 +585,7 @@ int build_locality(cc_graph *g, const std::vector<int64_t> &rp)
 int ensure_locality(cc_graph *g)
 {
     if (!g->has_tiles || !g->weighted || g->has_lw || g->borrowed) return CC_OK;
-    std::vector<int64_t> rp((size_t)g->n + 1);
-    CK(cudaMemcpy(rp.data(), g->fw.rp.p, rp.size() * 8, cudaMemcpyDeviceToHost));
-    return build_locality(g, rp);
+    return build_locality(g);
 }
 
 // Tiles of an undirected graph whose rows are short and mostly tiny
@@ -628,21 +604,17 @@ void free_graph(cc_graph *g)
 {
     if (g->borrowed) {  // drop the borrowed CSR pointers unfreed
         DevBuf *csr[] = {&g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
-                         &g->lw_perm, &g->lw_iperm, &g->fw.cls.L, &g->fw.cls.M,
-                         &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
+                         &g->lw_perm, &g->lw_iperm, &g->fw.cls.order, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
                      &g->rv.rp, &g->rv.col,
-                         &g->rv.w, &g->rv.cls.L, &g->rv.cls.M, &g->rv.cls.H, &g->rv.cls.Hn,
-                         &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj, &g->rv.cls.Nadj};
+                         &g->rv.w, &g->rv.cls.order, &g->rv.cls.Hn, &g->rv.cls.Hb, &g->rv.cls.Tadj, &g->rv.cls.Nadj};
         for (DevBuf *b : csr) { b->p = nullptr; b->cap = 0; }
     }
     if (!g->borrowed) tiles_free(g->tg);
     DevBuf *all[] = {&g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1, &g->t_stamp,
                      &g->t_Q0, &g->t_Q1, &g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
-                     &g->lw_perm, &g->lw_iperm, &g->lw_src, &g->fw.cls.L, &g->fw.cls.M,
-                     &g->fw.cls.H, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.T, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
+                     &g->lw_perm, &g->lw_iperm, &g->lw_src, &g->fw.cls.order, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
                      &g->rv.rp, &g->rv.col,
-                     &g->rv.w, &g->rv.cls.L, &g->rv.cls.M, &g->rv.cls.H, &g->rv.cls.Hn,
-                     &g->rv.cls.Hb, &g->rv.cls.T, &g->rv.cls.Tadj, &g->rv.cls.Nadj, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1,
+                     &g->rv.w, &g->rv.cls.order, &g->rv.cls.Hn, &g->rv.cls.Hb, &g->rv.cls.Tadj, &g->rv.cls.Nadj, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1,
                      &g->T, &g->tflag, &g->sidx, &g->sum2, &g->pivot, &g->delta, &g->lc2,
                      &g->Lmask, &g->hp, &g->dcc, &g->hist, &g->TN, &g->TS, &g->Ssamp,
                      &g->maxd, &g->sources, &g->npartial, &g->ctl, &g->shat, &g->clo,
@@ -1825,8 +1797,8 @@ int ccg::graph_borrow(cc_graph_t dst, cc_graph_t src)
     for (int d = 0; d < 2; ++d) {
         Classes &c = d ? dst->rv.cls : dst->fw.cls;
         const Classes &s = d ? src->rv.cls : src->fw.cls;
-        cp(c.L, s.L); cp(c.M, s.M); cp(c.H, s.H); cp(c.Hn, s.Hn); cp(c.Hb, s.Hb);
-        cp(c.T, s.T); cp(c.Tadj, s.Tadj); cp(c.Nadj, s.Nadj);
+        cp(c.order, s.order); cp(c.Hn, s.Hn); cp(c.Hb, s.Hb);
+        cp(c.Tadj, s.Tadj); cp(c.Nadj, s.Nadj);
         c.nL = s.nL; c.nM = s.nM; c.nH = s.nH; c.nHch = s.nHch; c.nT = s.nT;
     }
     dst->alpha = src->alpha;
@@ -1910,13 +1882,13 @@ int ccg::graph_view(cc_graph_t g, GraphView *v)
     v->weighted = g->weighted;
     v->rp = g->fw.rp.as<int64_t>();
     v->col = g->fw.col.as<int32_t>();
-    v->L = g->fw.cls.L.as<int32_t>();
-    v->T = g->fw.cls.T.as<int32_t>();
+    v->L = g->fw.cls.L();
+    v->T = g->fw.cls.T();
     v->Tadj = g->fw.cls.Tadj.as<int4>();
     v->nadj = g->fw.cls.Nadj.as<int4>();
     v->nT = g->fw.cls.nT;
-    v->M = g->fw.cls.M.as<int32_t>();
-    v->H = g->fw.cls.H.as<int32_t>();
+    v->M = g->fw.cls.M();
+    v->H = g->fw.cls.H();
     v->Hn = g->fw.cls.Hn.as<int32_t>();
     v->Hb = g->fw.cls.Hb.as<int64_t>();
     v->nL = g->fw.cls.nL;
@@ -1986,7 +1958,7 @@ int cc_graph_from_edges(int64_t n, int64_t m, const uint32_t *src, const uint32_
         rc = build_csr_device(n, m, src, dst, w, keep_component != 0, d);
         if (rc == CC_OK) rc = adopt_device_csr(g, d);
         if (rc == CC_OK) rc = cut_tiles(g);
-        if (rc == CC_OK && w && !g->has_tiles) rc = build_locality(g, d.rp_host);
+        if (rc == CC_OK && w && !g->has_tiles) rc = build_locality(g);
         if (d.rp) cudaFree(d.rp);
         if (d.col) cudaFree(d.col);
         if (d.w) cudaFree(d.w);

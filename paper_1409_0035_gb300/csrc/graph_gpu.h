@@ -10,7 +10,6 @@ namespace ccg {
 struct DeviceCSR {
     int64_t n = 0, arcs = 0;
     void *rp = nullptr, *col = nullptr, *w = nullptr;  // device, caller frees
-    std::vector<int64_t> rp_host;
     std::vector<int32_t> old_id;
 };
 
@@ -25,6 +24,14 @@ int build_csr_device(int64_t n, int64_t m, const uint32_t *src, const uint32_t *
 int build_csr_device_directed(int64_t n, int64_t m, const uint32_t *src, const uint32_t *dst,
                               const uint32_t *w, bool keep_component, DeviceCSR &F,
                               DeviceCSR &R);
+
+// Nodes by degree (stable, ids ascending; kMediumMaxDeg + 1 and more alike)
+// into order[n] (device), and on the host the counts of tiny, light, medium
+// and heavy nodes and of the heavy ones' chunk tasks.  Synchronises.
+int degree_order(int64_t n, const int64_t *rp, int32_t *order, int64_t (&counts)[5]);
+
+// Chunk tasks of the heavy nodes H (device): the node and first arc of each.
+int heavy_chunks(const int32_t *H, int64_t nH, const int64_t *rp, int32_t *Hn, int64_t *Hb);
 
 // Exclusive scan of n uint64 values (in -> out, may alias); *total = the sum.
 // Synchronises the stream.
