@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -49,21 +50,54 @@ constexpr double kTileMinLevels = 64.0;
 // K nodes, k = 64, before the last cuts: 6 -> 14.0 ms, 10 -> 13.2, 14 -> 14.2).
 constexpr double kTileDelta = 10.0;
 constexpr double kMaxHistBytes = 4.0 * (1ull << 30);  // distance histogram cap
+constexpr size_t kSlabBytes = 512u << 20;  // above, the allocations no longer count
+constexpr size_t kPinBytes = 1 << 20;  // host outputs staged in pinned memory
 
 // Bumped whenever a device buffer is (re)allocated or freed: a captured
 // estimate graph holds raw pointers and is valid only while it is unchanged.
 std::atomic<uint64_t> g_alloc_gen{1};
 
+// One allocation that a handle's first estimate carves its buffers from: some
+// forty of them cost 0.85 ms to allocate one by one and a millisecond to free
+// (R-MAT 18, edges to host results 4.54 -> 3.60 ms).  Current for the
+// thread while an estimate sizes its buffers (SlabScope); a buffer that
+// outgrows its part leaves it unused until the handle goes.
+struct Slab {
+    void *p = nullptr;
+    size_t cap = 0, off = 0;
+    void *take(size_t bytes)
+    {
+        const size_t b = (bytes + 255) & ~size_t(255);
+        if (off + b > cap) return nullptr;
+        void *q = static_cast<char *>(p) + off;
+        off += b;
+        return q;
+    }
+};
+thread_local Slab *t_slab = nullptr;
+struct SlabScope {
+    Slab *before;
+    explicit SlabScope(Slab *s) : before(t_slab) { t_slab = s; }
+    ~SlabScope() { t_slab = before; }
+};
+
 struct DevBuf {
     void *p = nullptr;
     size_t cap = 0;
+    bool part = false;  // of a slab
     int ensure(size_t bytes)
     {
         if (bytes <= cap) return CC_OK;
         g_alloc_gen.fetch_add(1);
-        if (p) cudaFree(p);
+        if (p && !part) cudaFree(p);
         p = nullptr;
         cap = 0;
+        part = false;
+        if (t_slab && bytes && (p = t_slab->take(bytes))) {
+            part = true;
+            cap = bytes;
+            return CC_OK;
+        }
         if (cudaMalloc(&p, bytes ? bytes : 16) != cudaSuccess) {
             cudaGetLastError();
             return CC_ERR_OOM;
@@ -74,9 +108,10 @@ struct DevBuf {
     void release()
     {
         if (p) g_alloc_gen.fetch_add(1);
-        if (p) cudaFree(p);
+        if (p && !part) cudaFree(p);
         p = nullptr;
         cap = 0;
+        part = false;
     }
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
@@ -213,6 +248,12 @@ struct cc_graph {
         dcc, hist, TN, TS, Ssamp, maxd, sources, npartial, ctl, shat, clo, hyb, ssum,
         distF, distR, mask, best, dmax, errflag, AL0, AL1, ACH0, ACH1, fstamp, AT0, AT1, ATa0,
         ATa1, band, bflag, gate2, hc2, sp_far0, sp_far1, sp_far2, sp_nst, sp_fst;
+    Slab slab;               // see Slab
+    DevBuf sc_cand, sc_cnt, sc_out;  // cc_sample_choose
+    std::mutex sc_mu;
+    // Small host outputs go through one pinned buffer, from the third call on.
+    char *pin = nullptr;
+    int host_calls = 0;
     // error estimate of the hybrid (SqErrEst): squared errors, fallback
     // distances, per-node flags, farthest-sample table, staged output
     DevBuf hcse, fdist, sqflag, istar, sqe;
@@ -610,7 +651,7 @@ void free_graph(cc_graph *g)
         for (DevBuf *b : csr) { b->p = nullptr; b->cap = 0; }
     }
     if (!g->borrowed) tiles_free(g->tg);
-    DevBuf *all[] = {&g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1, &g->t_stamp,
+    DevBuf *all[] = {&g->sc_cand, &g->sc_cnt, &g->sc_out, &g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1, &g->t_stamp,
                      &g->t_Q0, &g->t_Q1, &g->fw.rp, &g->fw.col, &g->fw.w, &g->lw.rp, &g->lw.col, &g->lw.w,
                      &g->lw_perm, &g->lw_iperm, &g->lw_src, &g->fw.cls.order, &g->fw.cls.Hn, &g->fw.cls.Hb, &g->fw.cls.Tadj, &g->fw.cls.Nadj,
                      &g->rv.rp, &g->rv.col,
@@ -631,6 +672,9 @@ void free_graph(cc_graph *g)
                      &g->rc_dsum, &g->rc_T, &g->rc_qstamp, &g->rc_vis, &g->rc_F, &g->rc_nxt,
                      &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
     for (DevBuf *b : all) b->release();
+    if (g->slab.p) cudaFree(g->slab.p);
+    g->slab = Slab{};
+    if (g->pin) { cudaFreeHost(g->pin); g->pin = nullptr; }
     if (g->ev0) cudaEventDestroy(g->ev0);
     if (g->ev1) cudaEventDestroy(g->ev1);
     g->ev0 = g->ev1 = nullptr;
@@ -1622,30 +1666,54 @@ int copy_outputs(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *out,
     const int64_t n = g->n;
     const bool dev_out = opts->device_outputs != 0;
     const cudaMemcpyKind kind = dev_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    struct Copy {
+        void *to;
+        const void *from;
+        size_t bytes;
+    };
+    Copy copies[2 * CC_NUM_EST + 8];
+    int nc = 0;
+    size_t total = 0;
+    auto put = [&](void *to, const void *from, size_t bytes) {
+        if (!to) return;
+        copies[nc++] = Copy{to, from, bytes};
+        total += (bytes + 63) & ~size_t(63);
+    };
     if (!dev_out) {
         for (int e = 0; e < CC_NUM_EST; ++e) {
             if (e == CC_EST_HYBRID && !hyb) continue;
-            if (out->s_hat[e])
-                CK(cudaMemcpyAsync(out->s_hat[e], fa.s_hat[e], n * 8, kind, st));
-            if (out->closeness[e])
-                CK(cudaMemcpyAsync(out->closeness[e], fa.clo[e], n * 8, kind, st));
+            put(out->s_hat[e], fa.s_hat[e], n * 8);
+            put(out->closeness[e], fa.clo[e], n * 8);
         }
-        if (out->hyb_int && hyb)
-            CK(cudaMemcpyAsync(out->hyb_int, fa.hyb_int, n * 48, kind, st));
-        if (out->sample_sum)
-            CK(cudaMemcpyAsync(out->sample_sum, fa.sample_sum, n * 8, kind, st));
-        if (fa.sq_err) CK(cudaMemcpyAsync(out->sq_err, fa.sq_err, n * 8, kind, st));
+        if (hyb) put(out->hyb_int, fa.hyb_int, n * 48);
+        put(out->sample_sum, fa.sample_sum, n * 8);
+        if (fa.sq_err) put(out->sq_err, fa.sq_err, n * 8);
     }
-    if (out->pivot && !fa.pivot_out)
-        CK(cudaMemcpyAsync(out->pivot, g->pivot.p, n * 4, kind, st));
-    if (out->delta && !fa.delta_out)
-        CK(cudaMemcpyAsync(out->delta, g->delta.p, n * 4, kind, st));
-    if (out->S_sampled)
-        CK(cudaMemcpyAsync(out->S_sampled, g->Ssamp.p, (size_t)k * 8, kind, st));
-    if (out->delta_cc)
-        CK(cudaMemcpyAsync(out->delta_cc, g->dcc.p, (size_t)k * k * 4, kind, st));
+    if (!fa.pivot_out) put(out->pivot, g->pivot.p, n * 4);
+    if (!fa.delta_out) put(out->delta, g->delta.p, n * 4);
+    put(out->S_sampled, g->Ssamp.p, (size_t)k * 8);
+    put(out->delta_cc, g->dcc.p, (size_t)k * k * 4);
+    // A copy into pageable memory is waited for by itself, about 10 us each
+    // however small: small outputs are queued into a pinned buffer, waited
+    // for once and handed on from there (R-MAT 12, sample and host outputs:
+    // with the
+    // sample's buffers kept, 455 -> 356 us a call).
+    const bool stage = !dev_out && total <= kPinBytes && g->host_calls >= 2;
+    if (!dev_out && g->host_calls < 2) g->host_calls += 1;
+    if (stage && !g->pin) CK(cudaMallocHost(&g->pin, kPinBytes));
+    size_t at = 0;
+    for (int i = 0; i < nc; ++i) {
+        void *to = stage ? g->pin + at : copies[i].to;
+        CK(cudaMemcpyAsync(to, copies[i].from, copies[i].bytes, kind, st));
+        at += (copies[i].bytes + 63) & ~size_t(63);
+    }
     CK(cudaStreamSynchronize(st));
     CK(cudaGetLastError());
+    at = 0;
+    for (int i = 0; stage && i < nc; ++i) {
+        std::memcpy(copies[i].to, g->pin + at, copies[i].bytes);
+        at += (copies[i].bytes + 63) & ~size_t(63);
+    }
     return CC_OK;
 }
 
@@ -1812,11 +1880,22 @@ int ccg::graph_borrow(cc_graph_t dst, cc_graph_t src)
 
 cc_graph_t ccg::graph_new_empty() { return new (std::nothrow) cc_graph(); }
 
+int ccg::graph_choose_sample(cc_graph_t g, int64_t n, int k, uint64_t seed, int32_t *host_out)
+{
+    // Needs no more of the handle than its buffers: two threads may ask at once.
+    std::lock_guard<std::mutex> lock(g->sc_mu);
+    RC(g->sc_cand.ensure(sample_candidate_bytes()));
+    RC(g->sc_cnt.ensure(4));
+    RC(g->sc_out.ensure((size_t)k * 4));
+    return choose_sample_ws(n, k, seed, host_out, g->sc_cand.p, g->sc_cnt.as<unsigned>(),
+                            g->sc_out.as<int32_t>(), 0);
+}
+
 int ccg::graph_ready_to_borrow(cc_graph_t g) { return ensure_locality(g); }
 
 size_t ccg::graph_workspace_bytes(cc_graph_t g)
 {
-    const DevBuf *ws[] = {&g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1,
+    const DevBuf *ws[] = {&g->sc_cand, &g->sc_cnt, &g->sc_out, &g->pl_F, &g->pl_R, &g->pl_masks, &g->pl_c, &g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1,
                           &g->t_stamp, &g->t_Q0, &g->t_Q1, &g->vis, &g->F0, &g->F1, &g->nxt, &g->Q0, &g->Q1, &g->T, &g->tflag,
                           &g->sidx, &g->sum2, &g->pivot, &g->delta, &g->lc2, &g->Lmask, &g->hp,
                           &g->dcc, &g->hist, &g->TN, &g->TS, &g->Ssamp, &g->maxd, &g->sources,
@@ -2147,6 +2226,39 @@ int cc_selftest_barrier_timeout(uint64_t timeout_ns)
     return err;
 }
 
+namespace {
+
+// A handle's slab, sized for its first estimate when that is a bit-packed one
+// (what does not fit is allocated by itself).  Server slots keep separate
+// buffers: their sizes are what the server accounts.
+int make_slab(cc_graph *g, int k, const cc_opts *opts)
+{
+    if (g->slab.p || g->borrowed || g->vis.p || g->weighted || g->directed || use_tiles(g, k))
+        return CC_OK;
+    const size_t n = (size_t)g->n, W = (size_t)pow2_words(k), K = (size_t)k;
+    const size_t nt = (size_t)g->fw.cls.nT, nch = (size_t)g->fw.cls.nHch;
+    const size_t cap = g->hist_cap ? (size_t)g->hist_cap : std::min<size_t>(n + 1, 4096);
+    const size_t c0 = std::min<size_t>(K * cap, 1 << 20), ts = std::min<size_t>(cap, 256);
+    // words and queues, lists, per-node sums and outputs; per-source tables
+    size_t bytes = n * (32 * W + 20 + 12 + 16 + 8) + nt * 40 + nch * 8 + sizeof(Ctl) * 2;
+    bytes += K * K * 4 + K * 64 + cap * K * 4 + 16 * K + 16 * K * ts + 16 * c0;
+    if (opts->want_hybrid) bytes += n * (64 * W + 1 + 16 + 16 + 32 + 8 * W) + 16 * K * cap;
+    if (!opts->device_outputs) bytes += n * (64 + 48 + 8);
+    bytes += 64 * 256;  // alignment
+    size_t free_b = 0, total_b = 0;
+    CK(cudaMemGetInfo(&free_b, &total_b));
+    if (bytes > std::min(free_b / 4, kSlabBytes)) return CC_OK;
+    if (cudaMalloc(&g->slab.p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        g->slab.p = nullptr;
+        return CC_OK;
+    }
+    g->slab.cap = bytes;
+    return CC_OK;
+}
+
+}  // namespace
+
 int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *opts,
                 cc_out *out)
 {
@@ -2157,6 +2269,8 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     reset_timing(g);
     cudaStream_t st = (cudaStream_t)opts->stream;
     const int64_t n = g->n;
+    RC(make_slab(g, k, opts));
+    const SlabScope scope(g->slab.p ? &g->slab : nullptr);
     RC(g->sidx.ensure(n * 4));
     RC(g->sum2.ensure(n * 16));
     RC(g->pivot.ensure(n * 4));

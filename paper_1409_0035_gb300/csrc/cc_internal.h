@@ -238,6 +238,8 @@ void graph_set_max_ctas(cc_graph_t g, int ctas);
 int choose_sample_ws(int64_t n, int k, uint64_t seed, int32_t *host_out, void *cand,
                      unsigned *count, int32_t *dout, cudaStream_t st);
 size_t sample_candidate_bytes();
+// The same in the handle's own buffers.
+int graph_choose_sample(cc_graph_t g, int64_t n, int k, uint64_t seed, int32_t *host_out);
 
 
 }  // namespace ccg

@@ -123,24 +123,6 @@ int choose_sample_ws(int64_t n, int k, uint64_t seed, int32_t *host_out, void *c
     return rc;
 }
 
-int choose_sample_device(int64_t n, int k, uint64_t seed, int32_t *host_out)
-{
-    Cand *buf = nullptr;
-    unsigned *cnt = nullptr;
-    int32_t *dout = nullptr;
-    if (cudaMalloc(&buf, sizeof(Cand) * kCap) != cudaSuccess ||
-        cudaMalloc(&cnt, 4) != cudaSuccess || cudaMalloc(&dout, (size_t)k * 4) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(buf); cudaFree(cnt); cudaFree(dout);
-        return CC_ERR_OOM;
-    }
-    const int rc = choose_sample_ws(n, k, seed, host_out, buf, cnt, dout, 0);
-    cudaFree(buf);
-    cudaFree(cnt);
-    cudaFree(dout);
-    return rc;
-}
-
 }  // namespace ccg
 
 extern "C" int cc_sample_choose(cc_graph_t g, int32_t k, uint64_t seed, int32_t *sample_out)
@@ -149,5 +131,5 @@ extern "C" int cc_sample_choose(cc_graph_t g, int32_t k, uint64_t seed, int32_t 
     if (!g || !sample_out || cc_graph_info(g, &n, nullptr, nullptr, nullptr) != CC_OK)
         return CC_ERR_ARG;
     if (k < 1 || k > CC_MAX_K || k > n) return CC_ERR_ARG;
-    return ccg::choose_sample_device(n, k, seed, sample_out);
+    return ccg::graph_choose_sample(g, n, k, seed, sample_out);
 }
