@@ -268,7 +268,7 @@ struct cc_graph {
     bool has_beta = false;
     // outbound / inbound reachability samples: order, per-node state, queues
     DevBuf rc_order, rc_rank, rc_cnt, rc_sat, rc_dsum, rc_T, rc_qstamp, rc_vis, rc_F, rc_nxt,
-        rc_lev, rc_Q0, rc_Q1, rc_QB0, rc_QB1, rc_TL, rc_out;
+        rc_lev, rc_planes, rc_Q0, rc_Q1, rc_QB0, rc_QB1, rc_TL, rc_out;
     bool sq = false;       // the current cc_estimate call wants SqErrEst
     int64_t D1 = 0;        // levels (largest distance) of the last first pass
     int cw = 32;           // sources per chunk of the last chunked first pass
@@ -670,7 +670,7 @@ void free_graph(cc_graph *g)
                      &g->nw_msum, &g->nw_wsum, &g->nw_S, &g->nw_hist, &g->nw_TS, &g->nw_lc,
                      &g->nw_out, &g->rc_order, &g->rc_rank, &g->rc_cnt, &g->rc_sat,
                      &g->rc_dsum, &g->rc_T, &g->rc_qstamp, &g->rc_vis, &g->rc_F, &g->rc_nxt,
-                     &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
+                     &g->rc_lev, &g->rc_planes, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
     for (DevBuf *b : all) b->release();
     if (g->slab.p) cudaFree(g->slab.p);
     g->slab = Slab{};
@@ -1911,7 +1911,7 @@ size_t ccg::graph_workspace_bytes(cc_graph_t g)
                      &g->nw_msum, &g->nw_wsum, &g->nw_S, &g->nw_hist, &g->nw_TS, &g->nw_lc,
                      &g->nw_out, &g->rc_order, &g->rc_rank, &g->rc_cnt, &g->rc_sat,
                      &g->rc_dsum, &g->rc_T, &g->rc_qstamp, &g->rc_vis, &g->rc_F, &g->rc_nxt,
-                     &g->rc_lev, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
+                     &g->rc_lev, &g->rc_planes, &g->rc_Q0, &g->rc_Q1, &g->rc_QB0, &g->rc_QB1, &g->rc_TL, &g->rc_out};
     size_t t = 0;
     for (const DevBuf *b : ws) t += b->cap;
     return t;
@@ -2700,12 +2700,13 @@ int cc_reach_estimate(cc_graph_t g, int32_t k, uint64_t seed, int32_t inbound, v
     RC(g->rc_F.ensure(n * W * 8));
     RC(g->rc_nxt.ensure(n * W * 8));
     RC(g->rc_lev.ensure(n * 64 * W * 4));
+    if (!g->weighted) RC(g->rc_planes.ensure(n * W * 8 * kReachPlanes));
     RC(g->rc_Q0.ensure(n * 4));
     RC(g->rc_Q1.ensure(n * 4));
     RC(g->rc_TL.ensure(n * 4));
-    const size_t nbig = (size_t)g->arcs / kReachBigDeg + 1;
-    RC(g->rc_QB0.ensure(nbig * 4));
-    RC(g->rc_QB1.ensure(nbig * 4));
+    const size_t nbig = 2 * ((size_t)g->arcs / kReachBigDeg) + 1;  // parts of rows
+    RC(g->rc_QB0.ensure(nbig * 8));
+    RC(g->rc_QB1.ensure(nbig * 8));
     RC(g->rc_out.ensure(n * 16));
     RC(g->ctl.ensure(sizeof(Ctl)));
     CK(cudaMemsetAsync(g->rc_cnt.p, 0, n * 4, st));
@@ -2739,11 +2740,12 @@ int cc_reach_estimate(cc_graph_t g, int32_t k, uint64_t seed, int32_t inbound, v
     j.F = g->rc_F.as<uint64_t>();
     j.nxt = g->rc_nxt.as<uint64_t>();
     j.lev = g->rc_lev.as<uint32_t>();
+    j.planes = g->weighted ? nullptr : g->rc_planes.as<uint64_t>();
     j.Q[0] = g->rc_Q0.as<int32_t>();
     j.Q[1] = g->rc_Q1.as<int32_t>();
     j.TL = g->rc_TL.as<int32_t>();
-    j.QB[0] = g->rc_QB0.as<int32_t>();
-    j.QB[1] = g->rc_QB1.as<int32_t>();
+    j.QB[0] = g->rc_QB0.as<uint64_t>();
+    j.QB[1] = g->rc_QB1.as<uint64_t>();
     j.ctl = g->ctl.as<Ctl>();
     j.timeout_ns = kTimeoutNs;
     if (!g->ev0) {

@@ -8,10 +8,12 @@
 
 namespace ccg {
 
+constexpr int kReachPlanes = 4;  // bit planes for levels below 1 << kReachPlanes
 constexpr int kReachMaxW = 16;  // words per node: groups of up to 1024 sources
-// Frontier nodes with more arcs are expanded by every warp of the grid (a
-// hub's row would take one warp milliseconds while the others wait).
-constexpr int kReachBigDeg = 2048;
+// Longer rows are queued and expanded in parts of so many arcs (a hub's row
+// would take one warp milliseconds while the others wait; 512, 256, 128, 64 and
+// 32 arcs: 1.95, 1.90, 1.77, 1.76, 1.80 ms on directed R-MAT 18).
+constexpr int kReachBigDeg = 128;
 
 struct ReachJob {
     int64_t n;
@@ -28,11 +30,13 @@ struct ReachJob {
     int64_t *T;                   // rank position of the k-th sample, mark rule
     uint32_t *qstamp;             // level stamp of the last push to the queue
     uint64_t *vis, *F, *nxt;      // n x W
+    uint64_t *planes;             // kReachPlanes x n x W: the low levels (see
+                                  // reach.cu; null with arc lengths)
     uint32_t *lev;                // n x 64 W: first-arrival level of each bit
-                                  // (arc lengths: tentative distance, kInf
-                                  // outside a group's search)
+                                  // beyond them (arc lengths: tentative
+                                  // distance, kInf outside a group's search)
     int32_t *Q[2], *TL;           // frontier queues, touched list (n each)
-    int32_t *QB[2];               // frontier nodes of more than kReachBigDeg arcs
+    uint64_t *QB[2];              // parts of longer rows: part << 32 | node
     Ctl *ctl;                     // barrier counter and error code
     uint64_t timeout_ns;
 };

@@ -160,3 +160,34 @@ def test_reach_hubs_and_dropped_sources(cc, leaves, k, inbound, words):
     for key in ("count", "distsum", "T"):
         assert np.array_equal(r[key], ref[key]), key
     assert close(r["avg"], ref["avg"]).all() and close(r["R_hat"], ref["R_hat"]).all()
+
+
+@pytest.mark.parametrize("words", [1, 8])
+@pytest.mark.parametrize("n,deg,k", [(200_000, 0.7, 5), (140_000, 6.0, 16)])
+def test_reach_wide_windows(cc, n, deg, k, words):
+    """Graphs of more nodes than one window of the order, with sets of every
+    size: count, distance sum and T of some nodes from their own searches."""
+    from scipy.sparse import csr_matrix
+    from scipy.sparse.csgraph import dijkstra
+    rng = np.random.default_rng(n)
+    m = int(n * deg)
+    s, d = rng.integers(0, n, (2, m))
+    keep = s != d
+    s, d = np.append(s[keep], n - 1), np.append(d[keep], 0)
+    g, _ = cc.cc_graph_from_edges(n, s.astype(np.uint32), d.astype(np.uint32), directed=True,
+                                  keep_component=False)
+    try:
+        cc.cc_set_param(g, cc.CC_PARAM_REACH_WORDS, words)
+        r = cc.cc_reach_estimate(g, k, 11, False)
+    finally:
+        cc.cc_graph_free(g)
+    order = orc.sample_order(n, 11)
+    A = csr_matrix((np.ones(s.size), (s, d)), shape=(n, n))
+    for v in rng.integers(0, n, 12):
+        D = dijkstra(A, indices=v, unweighted=True)
+        others = order[order != v]
+        at = np.flatnonzero(np.isfinite(D[others]))[:k]
+        assert r["count"][v] == at.size
+        assert r["distsum"][v] == int(D[others[at]].sum())
+        if at.size == k:
+            assert r["T"][v] == at[-1] + 1
