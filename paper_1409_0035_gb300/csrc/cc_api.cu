@@ -824,9 +824,9 @@ int plane_job(cc_graph *g, int k, bool roundtrip, PlaneJob &j)
 }
 
 // How the hybrid part after bfs_pass1 gets LCsum: by a second pass, from the
-// first pass's classification on arrival, from its planes (the second pass
-// queued in case they overflowed), or from planes known not to have.
-enum class Lc { kPass, kBand, kPlanes, kPlanesOnly };
+// first pass's classification on arrival, or from its planes (the second pass
+// queued in case they overflowed).
+enum class Lc { kPass, kBand, kPlanes };
 
 // The hybrid part of the bit-packed path for eps = a/b, after bfs_pass1:
 // H statistics from the histogram tails, thresholds, L-masks and, where
@@ -867,19 +867,16 @@ int bfs_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st, Lc l
     // classified on arrival, LCsum is complete once the deferred bits are
     // resolved, and the second pass runs only if a band offset overflowed.
     const unsigned *gate = g->npartial.as<unsigned>();
-    if (lc == Lc::kPlanes || lc == Lc::kPlanesOnly) {
+    if (lc == Lc::kPlanes) {
         PlaneJob pj;
         RC(plane_job(g, k, false, pj));
-        if (lc == Lc::kPlanes) {
-            RC(g->gate2.ensure(8));
-            pj.ovf = &g->ctl.as<Ctl>()->band_ovf;
-            pj.npartial = g->npartial.as<unsigned>();
-            pj.gate = g->gate2.as<unsigned>();
-            gate = g->gate2.as<unsigned>();
-        }
+        RC(g->gate2.ensure(8));
+        pj.ovf = &g->ctl.as<Ctl>()->band_ovf;
+        pj.npartial = g->npartial.as<unsigned>();
+        pj.gate = g->gate2.as<unsigned>();
+        gate = g->gate2.as<unsigned>();
         run_planes_lc(pj, st);
         g->call_kernels += 2;
-        if (lc == Lc::kPlanesOnly) return CC_OK;
     }
     if (lc == Lc::kBand) {
         RC(g->gate2.ensure(8));
@@ -1515,6 +1512,43 @@ int planes_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
     PlaneJob pj;
     RC(plane_job(g, k, g->directed, pj));
     run_planes_lc(pj, st);
+    CK(cudaGetLastError());
+    g->call_kernels += 5;
+    return CC_OK;
+}
+
+// The adaptive hybrid on planes after a first pass whose level count is D
+// (tail tables of tstride entries per source): ad_best, ad_bsq, ad_clo and
+// ad_choice of every node.
+int planes_adaptive(cc_graph *g, int k, bool roundtrip, DevCount D, int64_t tstride, int n_eps,
+                    const uint32_t *num, const uint32_t *den, cudaStream_t st)
+{
+    RC(g->TN.ensure((size_t)k * tstride * 8));
+    RC(g->TS.ensure((size_t)k * tstride * 8));
+    RC(g->maxd.ensure((size_t)k * 4));
+    RC(g->istar.ensure((size_t)k * 4));
+    run_tail(g->hist.as<uint32_t>(), D, tstride, k, g->TN.as<uint64_t>(), g->TS.as<uint64_t>(),
+             st);
+    run_maxdelta(g->dcc.as<uint32_t>(), k, g->maxd.as<uint32_t>(), st);
+    run_istar(g->dcc.as<uint32_t>(), k, g->istar.as<int32_t>(), st);
+    PlaneJob pj;
+    RC(plane_job(g, k, roundtrip, pj));
+    pj.istar = g->istar.as<int32_t>();
+    AdaptiveJob a;
+    a.D = D;
+    a.tstride = tstride;
+    a.maxd = g->maxd.as<uint32_t>();
+    a.TN = g->TN.as<uint64_t>();
+    a.TS = g->TS.as<uint64_t>();
+    a.S_samp = g->Ssamp.as<uint64_t>();
+    a.n_eps = n_eps;
+    std::copy(num, num + n_eps, a.num);
+    std::copy(den, den + n_eps, a.den);
+    a.est = g->ad_best.as<double>();
+    a.sq = g->ad_bsq.as<double>();
+    a.clo = g->ad_clo.as<double>();
+    a.choice = g->ad_choice.as<int32_t>();
+    run_planes_adaptive(pj, a, st);
     CK(cudaGetLastError());
     g->call_kernels += 5;
     return CC_OK;
@@ -2339,8 +2373,6 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     RC(g->Ssamp.ensure((size_t)k * 8));
     RC(g->sources.ensure((size_t)k * 4));
     RC(g->ctl.ensure(sizeof(Ctl)));
-    RC(g->ad_est.ensure((size_t)n * 8));
-    RC(g->ad_sq.ensure((size_t)n * 8));
     RC(g->ad_best.ensure((size_t)n * 8));
     RC(g->ad_bsq.ensure((size_t)n * 8));
     RC(g->ad_clo.ensure((size_t)n * 8));
@@ -2367,12 +2399,21 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
         }
         planes = planes && !g->hctl[0].band_ovf;
     }
+    const bool fused = planes || (chunked && g->on_planes);
+    if (fused)
+        RC(chunked ? planes_adaptive(g, k, true, DevCount{nullptr, g->D1}, g->D1 + 1, n_eps,
+                                     eps_num, eps_den, st)
+                   : planes_adaptive(g, k, false, DevCount{&g->ctl.as<Ctl>()->levels, 0},
+                                     g->hist_cap, n_eps, eps_num, eps_den, st));
+    else {
+        RC(g->ad_est.ensure((size_t)n * 8));
+        RC(g->ad_sq.ensure((size_t)n * 8));
+    }
     g->sq = true;
-    for (int e = 0; e < n_eps; ++e) {
+    for (int e = 0; e < (fused ? 0 : n_eps); ++e) {
         RC(chunked ? rows_hybrid(g, k, eps_num[e], eps_den[e], st)
-                   : bfs_hybrid(g, k, eps_num[e], eps_den[e], st,
-                                planes ? Lc::kPlanesOnly : Lc::kPass));
-        if (!chunked && !planes) {
+                   : bfs_hybrid(g, k, eps_num[e], eps_den[e], st));
+        if (!chunked) {
             CK(cudaStreamSynchronize(st));
             RC(settle_passes(g));
         }
@@ -2400,8 +2441,10 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
         g->call_kernels += 2;
     }
     g->sq = false;
-    run_closeness(n, g->ad_best.as<double>(), g->ad_clo.as<double>(), st);
-    g->call_kernels += 1;
+    if (!fused) {
+        run_closeness(n, g->ad_best.as<double>(), g->ad_clo.as<double>(), st);
+        g->call_kernels += 1;
+    }
     const cudaMemcpyKind kind =
         opts->device_outputs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (s_hat) CK(cudaMemcpyAsync(s_hat, g->ad_best.p, n * 8, kind, st));

@@ -23,7 +23,6 @@ __global__ void k_scatter_sidx(int32_t *sidx, const int32_t *src, int k)
     d_scatter_sidx(sidx, src, k, GSTART, GSTRIDE);
 }
 
-__device__ __forceinline__ int64_t count_of(DevCount c) { return c.p ? (int64_t)*c.p : c.h; }
 
 __global__ void k_S_sampled(const uint32_t *hist, DevCount D, int k, const uint32_t *dcc,
                             uint64_t *S)

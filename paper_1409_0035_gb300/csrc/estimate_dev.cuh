@@ -13,6 +13,8 @@ namespace {
 typedef unsigned __int128 u128;
 constexpr int kTailThreads = 256;
 
+__device__ __forceinline__ int64_t count_of(DevCount c) { return c.p ? (int64_t)*c.p : c.h; }
+
 // Round-to-nearest-even conversion of an unsigned 128-bit integer: the top
 // 64 significant bits with every lower bit folded into a sticky bit are
 // converted by the hardware (correctly rounded), then scaled by a power of
@@ -262,6 +264,19 @@ __device__ __forceinline__ void d_band_resolve(int64_t n, int k, int rowb, const
     }
 }
 
+// SqErrEst (Algorithm 1's last loop; section 4): the sampling term |L| var(L n
+// C) / |L n C| and the pivoting term |H| * mean over HC of (d(c_i, v) -
+// d(c(v), c_i))^2, whose numerator is t2num (HCnum = 0: that of one sample).
+__device__ __forceinline__ double sq_err_of(uint64_t LCnum, uint64_t LCsum, uint64_t LCsq,
+                                            uint64_t Lnum, uint64_t HCnum, u128 t2num)
+{
+    const u128 var_num = (u128)LCsq * LCnum - (u128)LCsum * LCsum;
+    const double t1 = u128_to_double(var_num * Lnum) /
+                      ((double)LCnum * (double)LCnum * (double)LCnum);
+    const double t2 = u128_to_double(t2num);
+    return t1 + (HCnum > 0 ? t2 / (double)HCnum : t2);
+}
+
 __device__ __forceinline__ void d_finalize(FinalizeArgs A, int64_t i0,
                                 int64_t stride)
 {
@@ -326,24 +341,18 @@ __device__ __forceinline__ void d_finalize(FinalizeArgs A, int64_t i0,
                 h6[0] = h.Hsum; h6[1] = h.Hnum; h6[2] = HCsum;
                 h6[3] = LCsum; h6[4] = LCnum; h6[5] = LCsq;
                 if (A.sq_err) {
-                    // SqErrEst (Algorithm 1's last loop; section 4): the
-                    // sampling term |L| var(L n C) / |L n C| and the pivoting
-                    // term |H| * mean over HC of (d(c_i, v) - d(c(v), c_i))^2.
-                    const u128 var_num = (u128)LCsq * LCnum - (u128)LCsum * LCsum;
-                    const double t1 = u128_to_double(var_num * Lnum) /
-                                      ((double)LCnum * (double)LCnum * (double)LCnum);
-                    double t2 = 0.0;
+                    u128 t2num = 0;
                     if (HCnum > 0) {
                         const u128 e2 = ((u128)A.hcse[2 * v + 1] << 64) | A.hcse[2 * v];
-                        t2 = u128_to_double(e2 * h.Hnum) / (double)HCnum;
+                        t2num = e2 * h.Hnum;
                     } else if (h.Hnum > 0) {
                         const int is = A.istar[p];
                         const int64_t e = (int64_t)A.fdist[v] -
                                           (int64_t)A.dcc[(int64_t)p * A.k + is];
                         const uint64_t ae = (uint64_t)(e < 0 ? -e : e);
-                        t2 = u128_to_double((u128)ae * ae * h.Hnum);
+                        t2num = (u128)ae * ae * h.Hnum;
                     }
-                    A.sq_err[v] = t1 + t2;
+                    A.sq_err[v] = sq_err_of(LCnum, LCsum, LCsq, Lnum, HCnum, t2num);
                 }
             }
         }

@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "estimate_dev.cuh"
 #include "planes.h"
 
 namespace ccg {
@@ -334,6 +335,139 @@ __global__ void k_pl_lc(PlaneJob J)
     });
 }
 
+// The adaptive hybrid, W lanes a node.  Thresholds at or beyond the largest
+// distance give the same classes (most small eps do), and a later eps wins
+// only by a smaller squared error, so an eps whose threshold equals the one
+// before it is passed over; the others' sums are collected lane by lane until
+// W are together, since the FP64 of one estimate takes a warp as long as that
+// of 32.  One pass over the planes for all eps in place of five kernels and
+// 150 bytes of state per node and eps (R-MAT 18, k = 256, seven eps: 594 of
+// 920 us of kernels before, 150 now).
+template <bool RT>
+__global__ void k_pl_adaptive(PlaneJob J, AdaptiveJob A)
+{
+    constexpr int kRows = plane_rows_dev<RT>;
+    const int W = J.W, lane = threadIdx.x & 31, g0 = lane & ~(W - 1);
+    const int64_t D = count_of(A.D);
+    const uint64_t nm1 = (uint64_t)(J.n - 1);
+    for_nodes(J.n, W, [&](int64_t v, int w, bool ok) {
+        const int j = ok ? J.sidx[v] : 0;
+        const bool live = ok && j < 0;
+        uint64_t S[kB] = {0, 0, 0, 0, 0};
+        int p = 0;
+        uint32_t delta = 0, maxd = 0;
+        uint64_t sum = 0, sumsq = 0;
+        if (live) {
+            load_planes<RT>(J, v * W + w, S);
+            p = J.pivot[v];
+            delta = J.delta[v];
+            maxd = A.maxd[p];
+            sum = J.sum2[2 * v];
+            sumsq = J.sum2[2 * v + 1];
+        }
+        double best = live || !ok ? 0.0 : (double)A.S_samp[j], bsq = 0.0;
+        int choice = -1;
+        int64_t before = -1;  // threshold of the eps last taken
+        int held = 0;         // estimates collected, lane w the w-th
+        // the one of this lane: LCnum, sums over L n C, the pivoting term's
+        // sum (or the one distance), threshold, eps
+        uint64_t c_lc = 0, c_s = 0, c_sq = 0, c_e2 = 0;
+        int64_t c_tt = 0;
+        int c_e = 0;
+        for (int e = 0; e <= A.n_eps; ++e) {
+            const bool end = e == A.n_eps;
+            if (!end) {
+                const uint64_t thr = (uint64_t)delta * A.den[e] / A.num[e];
+                const int64_t tt = thr < (uint64_t)D ? (int64_t)thr : D;
+                const bool take = live && tt != before;
+                if (!__any_sync(FULL, take)) continue;
+                const bool part = take && thr < maxd;
+                unsigned lc = 0, s = 0, sq = 0, e2 = 0;
+                if (part) {
+                    const uint64_t L = J.masks[((int64_t)p * kRows + tt) * W + w];
+                    lc = __popcll(L);
+                    sums<RT>(S, L, s, sq);
+                    const uint64_t H = valid_mask(J.k, w) & ~L;
+                    uint64_t C[kB];
+#pragma unroll
+                    for (int b = 0; b < kB; ++b) C[b] = J.cplanes[((int64_t)p * W + w) * kB + b];
+                    unsigned a0, dd, cc, x = 0;
+                    sums<RT>(S, H, a0, dd);
+                    sums<RT>(C, H, a0, cc);
+#pragma unroll
+                    for (int a = 0; a < kB; ++a)
+#pragma unroll
+                        for (int b = 0; b < kB; ++b)
+                            x += (unsigned)__popcll(S[a] & C[b] & H) << (a + b);
+                    e2 = dd + cc - 2u * x;
+                } else if (take) {
+                    const int is = J.istar[p];
+                    if ((is >> 6) == w) {
+#pragma unroll
+                        for (int b = 0; b < kB; ++b)
+                            e2 |= (unsigned)((S[b] >> (is & 63)) & 1ull) << b;
+                    }
+                }
+                lc = group_sum(lc, W);
+                s = group_sum(s, W);
+                sq = group_sum(sq, W);
+                e2 = group_sum(e2, W);
+                if (take) {
+                    if (w == held) {
+                        c_lc = part ? lc : (uint64_t)J.k;
+                        c_s = part ? s : sum;
+                        c_sq = part ? sq : sumsq;
+                        c_e2 = e2;
+                        c_tt = tt;
+                        c_e = e;
+                    }
+                    ++held;
+                    before = tt;
+                }
+            }
+            if (!(end ? __any_sync(FULL, held > 0) : __any_sync(FULL, held == W))) continue;
+            double est = 0.0, err = 0.0;
+            if (w < held) {
+                const uint64_t Hnum = A.TN[(int64_t)p * A.tstride + c_tt];
+                const uint64_t Hsum = A.TS[(int64_t)p * A.tstride + c_tt];
+                const uint64_t HCsum = sum - c_s, HCnum = (uint64_t)J.k - c_lc;
+                const uint64_t Lnum = nm1 - Hnum - HCnum;
+                const u128 N = (u128)(Hsum + HCsum) * c_lc + (u128)c_s * Lnum;
+                est = u128_to_double(N) / (double)c_lc;
+                if (c_lc == (uint64_t)J.k && Hnum == 0)
+                    est = u128_to_double((u128)nm1 * sum) / (double)J.k;
+                u128 t2num = 0;
+                if (HCnum > 0) {
+                    t2num = (u128)c_e2 * Hnum;
+                } else if (Hnum > 0) {
+                    const int64_t x = (int64_t)c_e2 -
+                                      (int64_t)J.dcc[(int64_t)p * J.k + J.istar[p]];
+                    const uint64_t ax = (uint64_t)(x < 0 ? -x : x);
+                    t2num = (u128)ax * ax * Hnum;
+                }
+                err = sq_err_of(c_lc, c_s, c_sq, Lnum, HCnum, t2num);
+            }
+            for (int i = 0; i < W; ++i) {
+                const double xe = __shfl_sync(FULL, est, g0 + i);
+                const double xq = __shfl_sync(FULL, err, g0 + i);
+                const int xi = __shfl_sync(FULL, c_e, g0 + i);
+                if (i < held && (choice < 0 || xq < bsq)) {
+                    best = xe;
+                    bsq = xq;
+                    choice = xi;
+                }
+            }
+            held = 0;
+        }
+        if (ok && w == 0) {
+            A.est[v] = best;
+            A.sq[v] = bsq;
+            A.clo[v] = (double)nm1 / best;
+            A.choice[v] = choice;
+        }
+    });
+}
+
 // ---- node weights ---------------------------------------------------------
 
 // S[i] += sum over v of beta(v) d(c_i, v): a warp per node, lane l the
@@ -524,6 +658,14 @@ void run_planes_lc(const PlaneJob &j, cudaStream_t st)
 {
     PLANES(k_pl_masks, grid_of((int64_t)j.k * j.W), j, st);
     PLANES(k_pl_lc, grid_of(j.n * j.W), j, st);
+}
+
+void run_planes_adaptive(const PlaneJob &j, const AdaptiveJob &a, cudaStream_t st)
+{
+    PLANES(k_pl_masks, grid_of((int64_t)j.k * j.W), j, st);
+    const int grid = grid_of(j.n * j.W);
+    if (j.R) k_pl_adaptive<true><<<grid, kT, 0, st>>>(j, a);
+    else k_pl_adaptive<false><<<grid, kT, 0, st>>>(j, a);
 }
 
 void run_planes_nw1(const PlaneJob &j, cudaStream_t st)

@@ -47,6 +47,18 @@ struct PlaneJob {
     int64_t D;
 };
 
+// The adaptive hybrid over n_eps values of eps = num / den.
+struct AdaptiveJob {
+    DevCount D;
+    int64_t tstride;           // of the tail tables
+    const uint32_t *maxd;      // k: largest distance between samples
+    const uint64_t *TN, *TS, *S_samp;
+    int n_eps;
+    uint32_t num[64], den[64];
+    double *est, *sq, *clo;    // n: of the eps of smallest squared error
+    int32_t *choice;           // n: its index (-1: sampled node)
+};
+
 // Sums, pivots, Delta, the largest distance and delta_cc from the planes.
 void run_planes_nodes(const PlaneJob &j, cudaStream_t st);
 // Per-source distance histogram over V \ C, rows 0 .. D.
@@ -54,6 +66,9 @@ void run_planes_hist(const PlaneJob &j, cudaStream_t st);
 // Sums over L(v) n C and the error estimate's inputs of the nodes that need
 // them (after the thresholds).
 void run_planes_lc(const PlaneJob &j, cudaStream_t st);
+// The adaptive hybrid from the planes, the tail tables and istar: for every
+// node the estimate, squared error and closeness of its best eps.
+void run_planes_adaptive(const PlaneJob &j, const AdaptiveJob &a, cudaStream_t st);
 // Node weights: per node sum_i mu_i d(c_i, v), per source sum_v beta(v) d.
 void run_planes_nw1(const PlaneJob &j, cudaStream_t st);
 // The hybrid's sums per node, and (bhist set) the beta mass per (distance,

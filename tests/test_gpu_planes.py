@@ -97,6 +97,34 @@ def test_every_width(cc, k, directed):
         cc.cc_graph_free(g)
 
 
+@pytest.mark.parametrize("k", [5, 100, 300])
+@pytest.mark.parametrize("directed", [False, True])
+def test_adaptive_eps_in_any_order(cc, k, directed):
+    """More eps than a node's words, unsorted and repeated: the first of the
+    smallest squared error."""
+    n, s, d = synth.watts_strogatz_edges(900, 6, 0.3, seed=8)
+    eps = [(1, 2), (1, 9), (9, 10), (1, 2), (1, 3), (3, 4), (1, 1), (2, 3), (1, 1000), (5, 7),
+           (4, 9)]
+    g, _ = cc.cc_graph_from_edges(n, s, d, directed=directed)
+    og = orc.csr_from_edges(n, s, d, directed=directed)
+    try:
+        C = cc.cc_sample_choose(g, k, 2)
+        T = orc.dist_table(og, C, roundtrip=directed)
+        o = cc.cc_opts_default(k)
+        o.roundtrip = int(directed)
+        ad = cc.cc_estimate_adaptive(g, C, o, eps)
+        hq = [orc.sqerr_from_table(T, C, e) for e in eps]
+        at = np.argmin(np.stack([q for _, q in hq]), axis=0)
+        other = np.setdiff1d(np.arange(og.n), C)
+        got = ad["choice"][other]
+        for v, e in zip(other, got):  # ties within rounding may fall to either
+            assert e == at[v] or close(hq[e][1][v], hq[at[v]][1][v])
+            assert close(ad["s_hat"][v], hq[e][0][v]) and close(ad["sq_err"][v], hq[e][1][v])
+        assert (ad["choice"][C] == -1).all()
+    finally:
+        cc.cc_graph_free(g)
+
+
 @pytest.mark.parametrize("k", [3, 64, 130, 300, 600])
 @pytest.mark.parametrize("eps", [(1, 16), (1, 2), (9, 10)])
 @pytest.mark.parametrize("directed", [False, True])
