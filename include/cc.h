@@ -252,8 +252,9 @@ typedef struct {
  * p counts beta(w) d(p, w), each sampled c_i with d(p, c_i) beyond counts
  * beta(c_i) d(c_i, v), each other sampled node max(tau, beta(c_i)) d(c_i, v).
  * Every estimate is an integer numerator over tau[1] divided once in FP64.
- * Runs the sources in chunks of shortest-path rows for every graph kind
- * (a second sweep for the hybrid when opts->want_hybrid).  opts: eps,
+ * Runs on the distances as bit planes on unit lengths while they stay below
+ * 16, else the sources in chunks of shortest-path rows (a second sweep for
+ * the hybrid when opts->want_hybrid).  opts: eps,
  * want_hybrid, roundtrip (must match the graph), device_outputs, stream.
  * Errors: CC_ERR_ARG (no weights attached, bad sample or tau = 0/x),
  * CC_ERR_DISCONNECTED, CC_ERR_OOM, CC_ERR_TIMEOUT, CC_ERR_CUDA,
@@ -369,7 +370,10 @@ typedef struct cc_batch *cc_batch_t;
  *                  two block shapes (the kernel's full residency per SM and
  *                  half of it) and time the six best plans;
  *                  0: default alpha, plan from CSR sizes only
- * The graphs fall into classes by their word width W (1, 2, 4 or 8 64-bit
+ * Graphs that cc_estimate would search tile by tile (under the parameters set
+ * on their handles at this call) do so in a run too, one after another behind
+ * the classes; the plan shows them as team 0 of 1 with switch 0.
+ * The others fall into classes by their word width W (1, 2, 4 or 8 64-bit
  * words per node).  A run is one cooperative launch per class, specialised
  * for its W and covering the GPU, the classes one after another: the CTAs
  * of a class form equal teams, each team estimating its graphs one after
@@ -481,7 +485,8 @@ int cc_server_free(cc_server_t s);
  * is at least 8, else 14): a level
  * runs top-down while (CSR entries of the frontier) * alpha < (CSR entries
  * of the nodes some source has not reached yet), bottom-up otherwise.
- * Results do not depend on it, only the time. */
+ * A value other than 0 also keeps this search where the graph would be
+ * searched tile by tile.  Results do not depend on it, only the time. */
 int cc_set_tuning(cc_graph_t g, int32_t alpha);
 
 /* Parameters of a graph's estimates (cc_set_param); results never depend
@@ -499,7 +504,7 @@ int cc_set_tuning(cc_graph_t g, int32_t alpha);
  *                             band offset exceeds a byte, the error estimate
  *                             is asked for, or the rows do not fit a third
  *                             of the free memory; 0: always the two-pass
- *                             form
+ *                             form (no tiles)
  *   CC_PARAM_SSSP_DELTA       bucket width of the shortest-path rounds with
  *                             arc lengths (delta-stepping with a near and a
  *                             far queue: labels below the threshold relax
@@ -508,7 +513,9 @@ int cc_set_tuning(cc_graph_t g, int32_t alpha);
  *                             0 restores the default (96 mean arc
  *                             lengths), a negative value relaxes every
  *                             label at once (plain label-correcting
- *                             rounds)
+ *                             rounds); any value but 0 keeps these rounds
+ *                             where the graph would be searched tile by
+ *                             tile
  *   CC_PARAM_REACH_WORDS      words per node of cc_reach_estimate's groups
  *                             (1, 2, 4, 8 or 16: groups of 64 x that many
  *                             sources searched together); 0 restores the

@@ -15,6 +15,12 @@
 // single-graph path, with team-wide bounded barriers (sections 2-3 of the
 // paper, applied to every graph of the batch).
 //
+// Members that an estimate of their own would search tile by tile (grids, road
+// networks) do so here too, one after another behind the class kernels: their
+// hundreds of levels at 13 to 16 us each are what a class would wait for (157 x
+// 157 grid, 16 sources: 4.8 ms of levels, 0.48 ms on tiles; twelve mixed graphs
+// with three grids 4.8 -> 3.1 ms a batch).
+//
 // The autotuner (cc_batch_create with autotune = 1) times every graph
 // alone under several direction switches alpha and keeps the fastest per
 // graph; per class it models the time of every team count P on a team of s
@@ -197,8 +203,21 @@ struct BatchClass {
     DBuf dteams, dcta, dorder;
 };
 
+// Handle on which the members searched by tiles run, each in turn.
+struct TileHandle {
+    cc_graph_t g = nullptr;
+    TileHandle() = default;
+    TileHandle(const TileHandle &) = delete;
+    TileHandle &operator=(const TileHandle &) = delete;
+    ~TileHandle() { if (g) cc_graph_free(g); }
+};
+
 struct cc_batch {
     int ngraphs = 0;
+    std::vector<char> tiled;                    // per graph: by tiles
+    std::vector<int> tstatus;                   // and its last status
+    std::vector<std::vector<int32_t>> samples;  // of those
+    TileHandle th;
     std::vector<cc_graph_t> graphs;
     std::vector<int> k, W, cls, alpha, cached;
     std::vector<int64_t> n;
@@ -414,13 +433,39 @@ int upload_plan(cc_batch *b, int c, int per_sm, int P, const std::vector<int> &t
     return CC_OK;
 }
 
+// Member i by tiles into its result buffers; synchronises the stream.
+int run_tiled(cc_batch *b, int i, cudaStream_t st)
+{
+    const BatchJob &J = b->hjobs[i];
+    B_RC(graph_borrow_tiles(b->th.g, b->graphs[i]));
+    cc_opts o;
+    cc_opts_default(&o, b->k[i]);
+    o.eps_num = J.a;
+    o.eps_den = J.b;
+    o.device_outputs = 1;
+    o.stream = st;
+    cc_out out;
+    std::memset(&out, 0, sizeof(out));
+    for (int e = 0; e < CC_NUM_EST; ++e) {
+        out.s_hat[e] = J.shat + (int64_t)e * b->n[i];
+        out.closeness[e] = J.clo + (int64_t)e * b->n[i];
+    }
+    out.pivot = J.j.pivot;
+    out.delta = J.j.delta;
+    out.hyb_int = J.hyb;
+    out.S_sampled = J.Ssamp;
+    out.delta_cc = J.j.dcc;
+    out.sample_sum = J.ssum;
+    return cc_estimate(b->th.g, b->samples[i].data(), b->k[i], &o, &out);
+}
+
 // Memsets and the class launches (the classes in `mask`), in stream order.
 int enqueue(cc_batch *b, cudaStream_t st, unsigned mask = 0xFu)
 {
     B_CK(cudaMemsetAsync(b->dctl.p, 0, b->ctl_bytes, st));
     B_CK(cudaMemsetAsync(b->dstatus.p, 0xFF, sizeof(int) * b->ngraphs, st));
     for (int i = 0; i < b->ngraphs; ++i) {
-        if (!((mask >> b->cls[i]) & 1u)) continue;
+        if (b->tiled[i] || !((mask >> b->cls[i]) & 1u)) continue;
         const BatchJob &J = b->hjobs[i];
         const int64_t n = b->n[i];
         const int k = b->k[i];
@@ -469,6 +514,8 @@ int run_once(cc_batch *b, cudaStream_t st, bool use_graph, unsigned mask = 0xFu)
     } else {
         B_RC(enqueue(b, st, mask));
     }
+    for (int i = 0; i < b->ngraphs && mask == 0xFu; ++i)
+        if (b->tiled[i]) b->tstatus[i] = run_tiled(b, i, st);
     B_CK(cudaEventRecord(b->e1, st));
     B_CK(cudaStreamSynchronize(st));
     float ms = 0.f;
@@ -499,6 +546,9 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
     b->graphs.assign(graphs, graphs + ngraphs);
     b->bufs.resize(ngraphs);
     b->hjobs.resize(ngraphs);
+    b->tiled.assign(ngraphs, 0);
+    b->tstatus.assign(ngraphs, CC_OK);
+    b->samples.resize(ngraphs);
     B_RC(batch_residency(b));
     b->ctl_bytes = sizeof(Ctl) * (size_t)(kClasses * b->P_max + 2 * ngraphs);
     B_RC(dalloc(b->dctl, b->ctl_bytes));
@@ -530,9 +580,8 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
         const int c = W == 1 ? 0 : W == 2 ? 1 : W == 4 ? 2 : 3;
         b->cls.push_back(c);
         b->alpha.push_back(v.alpha);
-        b->classes[c].graphs.push_back(i);
         auto &bf = b->bufs[i];
-        bf.resize(40);
+        bf.resize(48);
         int q = 0;
         auto take = [&](size_t bytes) -> void * {
             if (dalloc(bf[q], bytes) != CC_OK) return nullptr;
@@ -541,6 +590,30 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
         BatchJob J;
         std::memset(&J, 0, sizeof(J));
         BfsJob &j = J.j;
+        J.W = W;
+        J.k = k;
+        J.a = a;
+        J.b = bb;
+        j.pivot = (int32_t *)take(n * 4);
+        j.delta = (uint32_t *)take(n * 4);
+        j.dcc = (uint32_t *)take((size_t)k * k * 4);
+        J.Ssamp = (uint64_t *)take((size_t)k * 8);
+        J.shat = (double *)take((size_t)n * 8 * CC_NUM_EST);
+        J.clo = (double *)take((size_t)n * 8 * CC_NUM_EST);
+        J.hyb = (uint64_t *)take((size_t)n * 48);
+        J.ssum = (uint64_t *)take((size_t)n * 8);
+        if (!j.pivot || !j.delta || !j.dcc || !J.Ssamp || !J.shat || !J.clo || !J.hyb || !J.ssum)
+            return CC_ERR_OOM;
+        if (graph_takes_tiles(graphs[i], k)) {
+            // Run once to size the handle; what refuses goes to its class.
+            if (!b->th.g) b->th.g = graph_new_empty();
+            if (!b->th.g) return CC_ERR_OOM;
+            b->samples[i].assign(samples[i], samples[i] + k);
+            b->hjobs[i] = J;
+            b->tiled[i] = run_tiled(b, i, 0) == CC_OK;
+            if (b->tiled[i]) continue;
+        }
+        b->classes[c].graphs.push_back(i);
         j.n = n;
         j.arcs = v.arcs;
         j.rp = v.rp;
@@ -558,18 +631,16 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
         p[0] = take(n * W * 8); p[1] = take(n * W * 8); p[2] = take(n * W * 8);
         p[3] = take(n * W * 8); p[4] = take(n * 4); p[5] = take(n * 4); p[6] = take(n * 4);
         p[7] = take(n * 4); p[8] = take(n * 4); p[9] = take(n * 4); p[10] = take(n * 4);
-        p[11] = take(n * 4); p[12] = take(n * 16); p[13] = take(n * 4); p[14] = take(n * 4);
-        p[15] = take((size_t)k * k * 4); p[16] = take((size_t)k * 4);
-        for (int z = 0; z < 17; ++z)
+        p[11] = take(n * 4); p[12] = take(n * 16); p[13] = take((size_t)k * 4);
+        for (int z = 0; z < 14; ++z)
             if (!p[z]) return CC_ERR_OOM;
         j.vis = (uint64_t *)p[0]; j.F0 = (uint64_t *)p[1]; j.F1 = (uint64_t *)p[2];
         j.nxt = (uint64_t *)p[3];
         j.Q0 = (int32_t *)p[4]; j.Q1 = (int32_t *)p[5]; j.T = (int32_t *)p[6];
         j.tflag = (unsigned *)p[7]; j.sidx = (int32_t *)p[8]; j.AL0 = (int32_t *)p[9];
         j.AL1 = (int32_t *)p[10]; j.fstamp = (uint32_t *)p[11]; j.sum2 = (uint64_t *)p[12];
-        j.pivot = (int32_t *)p[13]; j.delta = (uint32_t *)p[14]; j.dcc = (uint32_t *)p[15];
         j.dcc_k = k;
-        j.sources = (int32_t *)p[16];
+        j.sources = (int32_t *)p[13];
         j.ACH0 = (int32_t *)take((size_t)std::max<int64_t>(1, v.nHch) * 4);
         j.ACH1 = (int32_t *)take((size_t)std::max<int64_t>(1, v.nHch) * 4);
         j.AT0 = (int32_t *)take((size_t)std::max<int64_t>(1, v.nT) * 4);
@@ -582,35 +653,25 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
         j.band = (uint8_t *)take((size_t)n * 64 * W);
         j.bflag = j.band ? (uint8_t *)take((size_t)n) : nullptr;
         if (!j.bflag) j.band = nullptr;
-        B_CK(cudaMemcpy(p[16], samples[i], (size_t)k * 4, cudaMemcpyHostToDevice));
+        B_CK(cudaMemcpy(p[13], samples[i], (size_t)k * 4, cudaMemcpyHostToDevice));
         j.red = RED_SUM | RED_PIVOT | RED_DCC | RED_HIST | (j.band ? RED_BAND : 0u);
         j.eps_a = a;
         j.eps_b = bb;
         j.timeout_ns = 10ull * 1000 * 1000 * 1000;
         j.alpha = v.alpha ? v.alpha : default_alpha(W, j.n, j.arcs);
         j.ctl = ctl_jobs + 2 * i;
-        J.W = W;
-        J.k = k;
         J.want_hybrid = 1;
-        J.a = a;
-        J.b = bb;
         J.hist_cap = cap;
         J.hist = (uint32_t *)take((size_t)cap * k * 4);
         J.TN = (uint64_t *)take((size_t)cap * k * 8);
         J.TS = (uint64_t *)take((size_t)cap * k * 8);
-        J.Ssamp = (uint64_t *)take((size_t)k * 8);
         J.maxd = (uint32_t *)take((size_t)k * 4);
         J.hp = (HybPrep *)take((size_t)n * sizeof(HybPrep));
         J.Lmask = (uint64_t *)take((size_t)n * W * 8);
         J.lc2 = (uint64_t *)take((size_t)n * 16);
         j.lc2 = J.lc2;
         J.npartial = (unsigned *)take(4);
-        J.shat = (double *)take((size_t)n * 8 * CC_NUM_EST);
-        J.clo = (double *)take((size_t)n * 8 * CC_NUM_EST);
-        J.hyb = (uint64_t *)take((size_t)n * 48);
-        J.ssum = (uint64_t *)take((size_t)n * 8);
-        if (!J.hist || !J.TN || !J.TS || !J.Ssamp || !J.maxd || !J.hp || !J.Lmask ||
-            !J.lc2 || !J.npartial || !J.shat || !J.clo || !J.hyb || !J.ssum)
+        if (!J.hist || !J.TN || !J.TS || !J.maxd || !J.hp || !J.Lmask || !J.lc2 || !J.npartial)
             return CC_ERR_OOM;
         j.hist = J.hist;
         j.hist_cap = cap;
@@ -650,6 +711,7 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
     if (autotune) {
         const int alphas[] = {0, 2, 4, 8, 14};
         for (int i = 0; i < ngraphs; ++i) {
+            if (b->tiled[i]) continue;
             TuneEntry key;
             if (!tpath.empty()) {
                 GraphView v;
@@ -683,7 +745,9 @@ int cc_batch_create(int32_t ngraphs, const cc_graph_t *graphs, const int32_t *co
             int best_a = 0;
             int64_t best_lv = 0;
             for (int al : alphas) {
-                B_RC(cc_set_tuning(graphs[i], al));
+                // (never 0, which may choose tiles)
+                B_RC(cc_set_tuning(graphs[i], al ? al : default_alpha(b->W[i], b->n[i],
+                                                                      b->hjobs[i].j.arcs)));
                 B_RC(cc_estimate(graphs[i], samples[i], b->k[i], &o, &none));
                 int32_t nl = 0, kern = 0;
                 double ms = 0, bytes = 0;
@@ -772,8 +836,10 @@ int cc_batch_run(cc_batch_t b, void *stream)
     B_RC(run_once(b, (cudaStream_t)stream, true));
     std::vector<int> st(b->ngraphs);
     B_CK(cudaMemcpy(st.data(), b->dstatus.p, sizeof(int) * b->ngraphs, cudaMemcpyDeviceToHost));
-    for (int s : st)
+    for (int i = 0; i < b->ngraphs; ++i) {
+        const int s = b->tiled[i] ? b->tstatus[i] : st[i];
         if (s != CC_OK) return s < 0 ? s : CC_ERR_CUDA;
+    }
     return CC_OK;
 }
 
@@ -813,6 +879,12 @@ int cc_batch_info(cc_batch_t b, int32_t *teams, int32_t *grid, double *last_ms,
         t += K.teams;
         g = std::max(g, K.grid);
     }
+    for (int i = 0; i < b->ngraphs; ++i)
+        if (b->tiled[i]) {  // one team of the whole GPU for all of them
+            t += 1;
+            g = std::max(g, b->sms * b->classes[b->cls[i]].max_per_sm);
+            break;
+        }
     if (teams) *teams = t;
     if (grid) *grid = g;
     if (last_ms) *last_ms = b->last_ms;
@@ -834,6 +906,15 @@ int cc_batch_plan(cc_batch_t b, int32_t i, int32_t *words, int32_t *alpha, int32
     if (!b || i < 0 || i >= b->ngraphs) return CC_ERR_ARG;
     if (from_cache) *from_cache = i < (int)b->cached.size() ? b->cached[i] : 0;
     const BatchClass &K = b->classes[b->cls[i]];
+    if (b->tiled[i]) {
+        if (words) *words = b->W[i];
+        if (alpha) *alpha = 0;
+        if (team) *team = 0;
+        if (class_teams) *class_teams = 1;
+        if (class_ctas) *class_ctas = b->sms * K.max_per_sm;
+        if (ctas_per_sm) *ctas_per_sm = K.max_per_sm;
+        return CC_OK;
+    }
     int x = 0;
     while (x < (int)K.graphs.size() && K.graphs[x] != i) ++x;
     if (words) *words = b->W[i];

@@ -282,6 +282,7 @@ struct cc_graph {
     double w_mean = 0.0;     // mean arc length (weighted graphs)
     int max_ctas = 0;    // cap on the CTAs of each launch (0: whole GPU)
     bool borrowed = false;  // CSR buffers belong to another handle
+    bool tiles_lent = false;  // and so do its tiles
     int hist_cap = 0;
     Ctl last{};
     // Traversal launches of the last API call: count, device time (CUDA
@@ -1253,11 +1254,11 @@ int chunked_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
 // setting of the search they replace (the direction switch or the two-pass
 // form on unit lengths, the bucket width with arc lengths), not in a server
 // slot (its launches are capped and its footprint is admitted for the other
-// path), and while the labels fit a third of the memory that is free or
+// path; a batch lends its handle the tiles), and while the labels fit a third of the memory that is free or
 // already held by them.
 bool use_tiles(cc_graph *g, int64_t k)
 {
-    if (!g->has_tiles || g->borrowed || g->max_ctas > 0) return false;
+    if (!g->has_tiles || (g->borrowed && !g->tiles_lent) || g->max_ctas > 0) return false;
     if (g->weighted ? g->sssp_delta != 0
                     : g->band_off || g->alpha != 0 || g->tg.levels < kTileMinLevels)
         return false;
@@ -1732,9 +1733,13 @@ int copy_outputs(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *out,
     // for once and handed on from there (R-MAT 12, sample and host outputs:
     // with the
     // sample's buffers kept, 455 -> 356 us a call).
-    const bool stage = !dev_out && total <= kPinBytes && g->host_calls >= 2;
+    bool stage = !dev_out && total <= kPinBytes && g->host_calls >= 2;
     if (!dev_out && g->host_calls < 2) g->host_calls += 1;
-    if (stage && !g->pin) CK(cudaMallocHost(&g->pin, kPinBytes));
+    if (stage && !g->pin && cudaMallocHost(&g->pin, kPinBytes) != cudaSuccess) {
+        cudaGetLastError();
+        g->pin = nullptr;
+        stage = false;
+    }
     size_t at = 0;
     for (int i = 0; i < nc; ++i) {
         void *to = stage ? g->pin + at : copies[i].to;
@@ -1913,6 +1918,16 @@ int ccg::graph_borrow(cc_graph_t dst, cc_graph_t src)
 }
 
 cc_graph_t ccg::graph_new_empty() { return new (std::nothrow) cc_graph(); }
+
+int ccg::graph_borrow_tiles(cc_graph_t dst, cc_graph_t src)
+{
+    RC(graph_borrow(dst, src));
+    dst->tg = src->tg;
+    dst->has_tiles = dst->tiles_lent = src->has_tiles;
+    return CC_OK;
+}
+
+bool ccg::graph_takes_tiles(cc_graph_t src, int64_t k) { return use_tiles(src, k); }
 
 int ccg::graph_choose_sample(cc_graph_t g, int64_t n, int k, uint64_t seed, int32_t *host_out)
 {

@@ -227,6 +227,10 @@ __device__ __forceinline__ uint64_t splitmix64_out(uint64_t seed, uint64_t c)
 // resident CSR of another handle per request.
 cc_graph_t graph_new_empty();
 int graph_borrow(cc_graph_t dst, cc_graph_t src);
+// The same with the tiles of `src`, and whether an estimate of k sources on
+// `src` runs on them.
+int graph_borrow_tiles(cc_graph_t dst, cc_graph_t src);
+bool graph_takes_tiles(cc_graph_t src, int64_t k);
 // Called once per graph before its first borrow: lays out what a borrowing
 // handle uses and this one may not have needed yet.
 int graph_ready_to_borrow(cc_graph_t g);

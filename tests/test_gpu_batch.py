@@ -113,3 +113,38 @@ def test_autotune_cache(cc, tmp_path):
     finally:
         for g in handles:
             cc.cc_graph_free(g)
+
+
+@pytest.mark.parametrize("autotune", [True, False])
+@pytest.mark.parametrize("which", [slice(0, 5), slice(0, 3), slice(1, 2)])
+def test_batch_members_on_tiles(cc, autotune, which):
+    """Members searched by tiles (long grids, 1 to 200 sources) beside members
+    that are not: every result equals the bit-packed search's."""
+    gens = [synth.grid_edges(40, 41), synth.grid_edges(300, 20), synth.grid_edges(64, 64),
+            synth.rmat_edges(10, 8, seed=2), synth.path_edges(300)][which]
+    ks = [1, 64, 200, 30, 17][which]
+    handles, samples, ns = [], [], []
+    try:
+        for (n, s, d), k in zip(gens, ks):
+            g, _ = cc.cc_graph_from_edges(n, s, d)
+            handles.append(g)
+            ns.append(cc.cc_graph_info(g)[0])
+            samples.append(cc.cc_sample_choose(g, k, 5 + k))
+        b = cc.cc_batch_create(handles, samples, autotune=autotune)
+        try:
+            assert cc.cc_batch_plan(b, 0)["class_teams"] >= 1
+            assert cc.cc_batch_info(b)["teams"] >= 1
+            for _ in range(3):
+                cc.cc_batch_run(b)
+            got = [cc.cc_batch_result(b, i, n, C.size)
+                   for i, (n, C) in enumerate(zip(ns, samples))]
+        finally:
+            cc.cc_batch_free(b)
+        for i, g in enumerate(handles):
+            cc.cc_set_tuning(g, 14)
+            want = cc.cc_estimate(g, samples[i])
+            for key in want:
+                assert (got[i][key] == want[key]).all(), (i, key)
+    finally:
+        for g in handles:
+            cc.cc_graph_free(g)
