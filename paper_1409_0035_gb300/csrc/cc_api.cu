@@ -1370,7 +1370,10 @@ int tiled_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
     const int64_t n = g->n;
     const int W = pow2_words(k);
     const int64_t D = g->D1, hs = (D + 64) / 64 * 64;
-    if ((double)(D + 1) * k * 4.0 > (double)kMaxHistBytes) return CC_ERR_TOO_LARGE;
+    // The limit of the shortest-path rounds' histogram.  On unit lengths, where
+    // the level-synchronous search has none, D < n: the counters are no more
+    // than the labels that are there already.
+    if (g->weighted && (double)(D + 1) * k * 4.0 > (double)kMaxHistBytes) return CC_ERR_TOO_LARGE;
     // Sums of squared distances (LCsumSq) stay in 64 bits.
     if ((double)D * (double)D * (double)k >= 1.8e19) return CC_ERR_TOO_LARGE;
     const size_t blocks = (size_t)k * (hs / 64 + 1) * 8;

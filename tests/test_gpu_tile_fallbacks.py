@@ -1,0 +1,67 @@
+"""Graphs cut into tiles at the limits of another search: what the
+level-synchronous search answered before stays answered."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+RTOL = 1e-12  # one conversion and one division of the same integers
+
+
+@pytest.fixture(scope="module")
+def cc():
+    from paper_1409_0035_gb300 import build
+    build.build()
+    import paper_1409_0035_gb300 as m
+    return m
+
+
+def path_hybrid(n, C, v, eps):
+    """Hybrid of node v of a path, C the sampled positions, from the
+    definitions: (Hsum, Hnum, HCsum, LCsum, LCnum, estimate)."""
+    d = np.abs(C.astype(np.int64) - v)
+    i = int(d.argmin())
+    p, t = int(C[i]), int(d[i]) * eps[1] // eps[0]
+    num = tot = 0
+    for side in (p, n - 1 - p):  # nodes beyond t on each side
+        if side > t:
+            num += side - t
+            tot += (side * (side + 1) - t * (t + 1)) // 2
+    dc = np.abs(C.astype(np.int64) - p)
+    far = dc > t
+    num -= int(far.sum())
+    tot -= int(dc[far].sum())
+    hc, lc, L = int(d[far].sum()), int(d[~far].sum()), int((~far).sum())
+    est = ((tot + hc) * L + lc * (n - 1 - num - int(far.sum()))) / L
+    return (tot, num, hc, lc, L), est
+
+
+def test_more_distances_than_a_row_histogram(cc):
+    """(D + 1) k counters of four bytes, over 4 GiB: a path of 1.1 million
+    nodes and 1024 sources."""
+    n, s, d = synth.path_edges(1_100_000)
+    k = 1024
+    g, _ = cc.cc_graph_from_edges(n, s, d)
+    try:
+        C = cc.cc_sample_choose(g, k, 2)
+        o = cc.cc_opts_default(k)
+        r = cc.cc_estimate(g, C, o)
+        assert (int(r["delta_cc"].max()) + 1) * k * 4 > 4 << 30
+        eps = [(1, 2), (1, 40)]
+        ad = cc.cc_estimate_adaptive(g, C, o, eps)
+    finally:
+        cc.cc_graph_free(g)
+    rng = np.random.default_rng(3)
+    inC = np.zeros(n, bool)
+    inC[C] = True
+    for v in np.concatenate([[0, n - 1], rng.integers(0, n, 60)]):
+        if inC[v]:
+            continue
+        dv = np.abs(C.astype(np.int64) - v)
+        assert r["sum"][v] == dv.sum() and r["delta"][v] == dv.min() and r["pivot"][v] == dv.argmin()
+        ints, est = path_hybrid(n, C, int(v), (o.eps_num, o.eps_den))
+        assert tuple(int(x) for x in r["hyb"][v][:5]) == ints
+        assert abs(r["s_hat"][3][v] - est) <= RTOL * est
+        est = path_hybrid(n, C, int(v), eps[ad["choice"][v]])[1]
+        assert abs(ad["s_hat"][v] - est) <= RTOL * est
