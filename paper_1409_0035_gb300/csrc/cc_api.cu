@@ -631,13 +631,17 @@ int ensure_locality(cc_graph *g)
 }
 
 // Tiles of an undirected graph whose rows are short and mostly tiny
-// (tiles.cu decides whether they are local).
+// (tiles.cu decides whether they are local).  The graph serves every call
+// without them: where memory is short of the 60 to 100 bytes a node that
+// cutting takes, there are none.
 int cut_tiles(cc_graph *g)
 {
     const Classes &c = g->fw.cls;
     if (g->directed || g->n < kTileMinNodes || c.nM + c.nH > 0 || 2 * c.nT < g->n) return CC_OK;
-    RC(tiles_build(g->n, g->arcs, g->fw.rp.as<int64_t>(), g->fw.col.as<int32_t>(),
-                   g->weighted ? g->fw.w.as<uint32_t>() : nullptr, g->tg, &g->has_tiles, 0));
+    const int rc = tiles_build(g->n, g->arcs, g->fw.rp.as<int64_t>(), g->fw.col.as<int32_t>(),
+                               g->weighted ? g->fw.w.as<uint32_t>() : nullptr, g->tg,
+                               &g->has_tiles, 0);
+    if (rc != CC_OK && rc != CC_ERR_OOM) return rc;
     CK(cudaDeviceSynchronize());  // estimates may run on other streams
     return CC_OK;
 }

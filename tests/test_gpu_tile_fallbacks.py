@@ -1,4 +1,5 @@
-"""Graphs cut into tiles at the limits of another search: what the
+"""Graphs cut into tiles where the tiles cannot serve: more distances than
+another search's histogram limit, memory too short to cut them.  What the
 level-synchronous search answered before stays answered."""
 import numpy as np
 import pytest
@@ -65,3 +66,50 @@ def test_more_distances_than_a_row_histogram(cc):
         assert abs(r["s_hat"][3][v] - est) <= RTOL * est
         est = path_hybrid(n, C, int(v), eps[ad["choice"][v]])[1]
         assert abs(ad["s_hat"][v] - est) <= RTOL * est
+
+
+class Short:
+    """All device memory but `left` bytes taken, while it lives."""
+
+    def __init__(self, left):
+        import torch
+        torch.cuda.empty_cache()
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        self.t = torch.empty(free - left, dtype=torch.uint8, device="cuda")
+
+    def give_back(self):
+        import torch
+        self.t = None
+        torch.cuda.empty_cache()
+
+
+def test_no_memory_to_cut_tiles(cc):
+    """From the memory that holds the graph and its tiles down to what does not
+    hold the graph: in between the graph is there without tiles."""
+    n, s, d = synth.grid_edges(2048, 1024)
+    rounds = []
+    for left in range(480, 160, -20):
+        m = Short(left << 20)
+        try:
+            g, _ = cc.cc_graph_from_edges(n, s, d)
+        except cc.CCError as e:
+            assert e.code == cc.CC_ERR_OOM
+            rounds.append(0)
+            continue
+        finally:
+            m.give_back()
+        try:
+            C = np.array([0, 7777, n - 1], np.int32)
+            r = cc.cc_estimate(g, C)
+            x, y = np.arange(n) % 2048, np.arange(n) // 2048
+            T = np.stack([np.abs(x - c % 2048) + np.abs(y - c // 2048) for c in C])
+            assert np.array_equal(r["sum"], T.sum(0).astype(np.uint64))
+            rounds.append(int(cc.cc_last_pass_stats(g)["levels"]))
+        finally:
+            cc.cc_graph_free(g)
+    levels = 2048 + 1024 - 2
+    assert rounds[0] > 0 and rounds[0] < levels  # tiles
+    assert levels in rounds                      # none: a round per level
+    at = rounds.index(levels)
+    assert all(0 < x < levels for x in rounds[:at])
