@@ -1562,8 +1562,9 @@ int planes_adaptive(cc_graph *g, int k, bool roundtrip, DevCount D, int64_t tstr
     return CC_OK;
 }
 
-// First pass and hybrid part on distance rows: tiles where the graph has
-// them (g->on_tiles tells which ran last), planes (g->on_planes), else chunks.
+// First pass and hybrid part on distance rows: tiles where the caller chose
+// them (g->on_tiles), planes (g->on_planes tells whether they ran), else
+// chunks.  Returns 1 when the tiles' labels came near 2^32.
 int rows_pass1(cc_graph *g, int k, cudaStream_t st)
 {
     g->on_planes = false;
@@ -1575,13 +1576,7 @@ int rows_pass1(cc_graph *g, int k, cudaStream_t st)
         }
         if (rc != 1) return rc;
     }
-    g->on_tiles = use_tiles(g, k);
-    if (g->on_tiles) {
-        const int rc = tiled_pass1(g, k, st);
-        if (rc != 1) return rc;
-        g->on_tiles = false;
-    }
-    return chunked_pass1(g, k, st);
+    return g->on_tiles ? tiled_pass1(g, k, st) : chunked_pass1(g, k, st);
 }
 
 int rows_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
@@ -1596,6 +1591,23 @@ int estimate_chunked(cc_graph *g, int k, const cc_opts *opts, cudaStream_t st)
     RC(rows_pass1(g, k, st));
     if (!opts->want_hybrid) return CC_OK;
     return rows_hybrid(g, k, opts->eps_num, opts->eps_den, st);
+}
+
+// Whether a call that ended with rc on the tiles goes to the search that they
+// replace: labels near 2^32 (the shortest-path rounds decide), or memory
+// short, whose labels are then given back (4 bytes a node and source, where a
+// bit-packed search takes half a byte).
+bool leave_tiles(cc_graph *g, int rc, cudaStream_t st)
+{
+    if (!g->on_tiles || (rc != 1 && rc != CC_ERR_OOM)) return false;
+    g->on_tiles = false;
+    if (rc == CC_ERR_OOM) {
+        cudaStreamSynchronize(st);
+        for (DevBuf *b : {&g->t_dist, &g->t_dirty0, &g->t_dirty1, &g->t_act0, &g->t_act1,
+                          &g->t_stamp, &g->t_Q0, &g->t_Q1})
+            b->release();
+    }
+    return true;
 }
 
 // Whether an estimate's first pass leaves distance rows (arc lengths, round
@@ -2339,24 +2351,25 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     const bool hyb = opts->want_hybrid != 0;
     g->sq = hyb && out->sq_err != nullptr;
     g->on_tiles = use_tiles(g, k);
-    const bool chunked = on_rows(g);
-    if (g->on_tiles) g->eg.replayed = 0;
     int rc = CC_OK;
-    if (chunked) {
+    do {
+        if (!on_rows(g)) {
+            rc = run_bfs_estimate(g, k, hyb, opts, out, st);  // synchronises
+            break;
+        }
+        g->eg.replayed = 0;
         run_fill_i32(g->sidx.as<int32_t>(), n, -1, st);
         run_scatter_sidx(g->sidx.as<int32_t>(), g->sources.as<int32_t>(), k, st);
         g->call_kernels += 2;
         rc = estimate_chunked(g, k, opts, st);
         if (rc == CC_OK) rc = finish_outputs(g, k, hyb, opts, out, st);  // synchronises
-    } else {
-        rc = run_bfs_estimate(g, k, hyb, opts, out, st);  // synchronises
-    }
+    } while (leave_tiles(g, rc, st));
     if (rc != CC_OK) {
         cudaStreamSynchronize(st);
         g->pend = 0;
         return rc;
     }
-    if (chunked) return CC_OK;
+    if (on_rows(g)) return CC_OK;
     // The bit-packed passes were queued without waiting: account them and
     // check the first pass now.
     rc = settle_passes(g);
@@ -2366,26 +2379,13 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     return c1;
 }
 
-int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *opts,
-                         int32_t n_eps, const uint32_t *eps_num, const uint32_t *eps_den,
-                         double *s_hat, double *closeness, double *sq_err, int32_t *choice)
+namespace {
+
+// An adaptive estimate on the search chosen (g->on_tiles).
+int adaptive_run(cc_graph *g, const int32_t *sample, int k, const cc_opts *opts, int n_eps,
+                 const uint32_t *eps_num, const uint32_t *eps_den, double *s_hat,
+                 double *closeness, double *sq_err, int32_t *choice, cudaStream_t st)
 {
-    static const uint32_t kNum[] = {1, 1, 1, 1, 1, 1, 99};
-    static const uint32_t kDen[] = {1000, 40, 20, 10, 5, 2, 100};
-    if (!g || !opts) return CC_ERR_ARG;
-    if (!eps_num || !eps_den) {
-        if (eps_num || eps_den) return CC_ERR_ARG;
-        n_eps = 7;
-        eps_num = kNum;
-        eps_den = kDen;
-    }
-    if (n_eps < 1 || n_eps > 64) return CC_ERR_ARG;
-    for (int e = 0; e < n_eps; ++e)
-        if (eps_num[e] == 0 || eps_num[e] > eps_den[e]) return CC_ERR_ARG;
-    if ((opts->roundtrip != 0) != g->directed) return CC_ERR_ARG;
-    RC(validate_sample(g, sample, k));
-    reset_timing(g);
-    cudaStream_t st = (cudaStream_t)opts->stream;
     const int64_t n = g->n;
     RC(g->sidx.ensure(n * 4));
     RC(g->sum2.ensure(n * 16));
@@ -2403,7 +2403,6 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     run_fill_i32(g->sidx.as<int32_t>(), n, -1, st);
     run_scatter_sidx(g->sidx.as<int32_t>(), g->sources.as<int32_t>(), k, st);
     g->call_kernels += 2;
-    g->on_tiles = use_tiles(g, k);
     const bool chunked = on_rows(g);
     bool planes = false;
     if (chunked) {
@@ -2475,6 +2474,37 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     if (choice) CK(cudaMemcpyAsync(choice, g->ad_choice.p, n * 4, kind, st));
     CK(cudaStreamSynchronize(st));
     return CC_OK;
+}
+
+}  // namespace
+
+int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *opts,
+                         int32_t n_eps, const uint32_t *eps_num, const uint32_t *eps_den,
+                         double *s_hat, double *closeness, double *sq_err, int32_t *choice)
+{
+    static const uint32_t kNum[] = {1, 1, 1, 1, 1, 1, 99};
+    static const uint32_t kDen[] = {1000, 40, 20, 10, 5, 2, 100};
+    if (!g || !opts) return CC_ERR_ARG;
+    if (!eps_num || !eps_den) {
+        if (eps_num || eps_den) return CC_ERR_ARG;
+        n_eps = 7;
+        eps_num = kNum;
+        eps_den = kDen;
+    }
+    if (n_eps < 1 || n_eps > 64) return CC_ERR_ARG;
+    for (int e = 0; e < n_eps; ++e)
+        if (eps_num[e] == 0 || eps_num[e] > eps_den[e]) return CC_ERR_ARG;
+    if ((opts->roundtrip != 0) != g->directed) return CC_ERR_ARG;
+    RC(validate_sample(g, sample, k));
+    reset_timing(g);
+    cudaStream_t st = (cudaStream_t)opts->stream;
+    g->on_tiles = use_tiles(g, k);
+    int rc;
+    do
+        rc = adaptive_run(g, sample, k, opts, n_eps, eps_num, eps_den, s_hat, closeness, sq_err,
+                          choice, st);
+    while (leave_tiles(g, rc, st));
+    return rc;
 }
 
 int cc_graph_set_node_weights(cc_graph_t g, const uint32_t *beta)

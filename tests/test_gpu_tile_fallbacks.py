@@ -1,5 +1,5 @@
 """Graphs cut into tiles where the tiles cannot serve: more distances than
-another search's histogram limit, memory too short to cut them.  What the
+another search's histogram limit, memory too short to cut or to search them.  What the
 level-synchronous search answered before stays answered."""
 import numpy as np
 import pytest
@@ -113,3 +113,37 @@ def test_no_memory_to_cut_tiles(cc):
     assert levels in rounds                      # none: a round per level
     at = rounds.index(levels)
     assert all(0 < x < levels for x in rounds[:at])
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("call", ["hybrid", "adaptive"])
+def test_no_memory_to_search_tiles(cc, weighted, call):
+    """The labels of an earlier call are held, the hybrid's tables do not fit
+    beside them: the search that the tiles replace runs in their place."""
+    n, s, d = synth.grid_edges(64, 3900)
+    w = np.full(s.size, 1, np.uint32) if weighted else None
+    k = 512
+    g, _ = cc.cc_graph_from_edges(n, s, d, w)
+    try:
+        C = cc.cc_sample_choose(g, k, 2)
+        o = cc.cc_opts_default(k)
+
+        def run():
+            if call == "adaptive":
+                return cc.cc_estimate_adaptive(g, C, o)
+            return cc.cc_estimate(g, C, o)
+
+        o.want_hybrid = 0
+        cc.cc_estimate(g, C, o)
+        o.want_hybrid = 1
+        m = Short(12 << 20)
+        try:
+            r = run()
+        finally:
+            m.give_back()
+        want = run()
+        assert cc.cc_last_pass_stats(g)["levels"] < 3000  # tiles again
+    finally:
+        cc.cc_graph_free(g)
+    for key in want:
+        assert np.array_equal(r[key], want[key]), key
