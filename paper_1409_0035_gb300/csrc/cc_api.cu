@@ -935,13 +935,22 @@ bool use_band(cc_graph *g, int k, const cc_opts *opts)
     return need <= ((double)free_b + (double)g->band.cap) / 3.0;
 }
 
-int estimate_bfs(cc_graph *g, int k, const cc_opts *opts, bool band, cudaStream_t st)
+// The form of a bit-packed estimate's hybrid part: with the error estimate the
+// planes, unless the two-pass form is set.
+Lc choose_lc(cc_graph *g, int k, const cc_opts *opts)
 {
-    const bool planes = opts->want_hybrid && g->sq && !g->band_off && planes_fit(g, k, 1);
-    RC(bfs_pass1(g, k, st, band ? opts->eps_num : 0, band ? opts->eps_den : 0, planes));
+    if (use_band(g, k, opts)) return Lc::kBand;
+    if (opts->want_hybrid && g->sq && !g->band_off && planes_fit(g, k, 1)) return Lc::kPlanes;
+    return Lc::kPass;
+}
+
+int estimate_bfs(cc_graph *g, int k, const cc_opts *opts, Lc lc, cudaStream_t st)
+{
+    const bool band = lc == Lc::kBand;
+    RC(bfs_pass1(g, k, st, band ? opts->eps_num : 0, band ? opts->eps_den : 0,
+                 lc == Lc::kPlanes));
     if (!opts->want_hybrid) return CC_OK;
-    return bfs_hybrid(g, k, opts->eps_num, opts->eps_den, st,
-                      band ? Lc::kBand : planes ? Lc::kPlanes : Lc::kPass);
+    return bfs_hybrid(g, k, opts->eps_num, opts->eps_den, st, lc);
 }
 
 // One chunk of shortest paths (forward, and reversed for round trips)
@@ -1788,12 +1797,12 @@ int finish_outputs(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *ou
 // output copies.  The finalisation's arguments are taken after the passes
 // are queued, once every buffer they point to is sized.
 int enqueue_bfs_estimate(cc_graph *g, int k, bool hyb, const cc_opts *opts, const cc_out *out,
-                         bool band, FinalizeArgs &fa, cudaStream_t st)
+                         Lc lc, FinalizeArgs &fa, cudaStream_t st)
 {
     run_fill_i32(g->sidx.as<int32_t>(), g->n, -1, st);
     run_scatter_sidx(g->sidx.as<int32_t>(), g->sources.as<int32_t>(), k, st);
     g->call_kernels += 2;
-    RC(estimate_bfs(g, k, opts, band, st));
+    RC(estimate_bfs(g, k, opts, lc, st));
     RC(prepare_finalize(g, k, hyb, opts, out, fa));
     enqueue_finalize(g, k, fa, st);
     return CC_OK;
@@ -1801,11 +1810,11 @@ int enqueue_bfs_estimate(cc_graph *g, int k, bool hyb, const cc_opts *opts, cons
 
 // The arguments a captured estimate graph depends on.
 std::vector<uint64_t> est_key(const cc_graph *g, int k, const cc_opts *opts, const cc_out *out,
-                              bool band)
+                              Lc lc)
 {
     std::vector<uint64_t> key = {g_alloc_gen.load(), (uint64_t)k, (uint64_t)opts->want_hybrid,
                                  opts->eps_num, opts->eps_den, (uint64_t)opts->device_outputs,
-                                 (uint64_t)g->sq, (uint64_t)band, (uint64_t)g->hist_cap,
+                                 (uint64_t)g->sq, (uint64_t)lc, (uint64_t)g->hist_cap,
                                  (uint64_t)g->alpha, (uint64_t)g->max_ctas};
     // The finalisation writes device outputs in place (their addresses are
     // in the graph); host outputs are copied after it, from the library's
@@ -1833,12 +1842,12 @@ int run_bfs_estimate(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *
 {
     if (g->hist_cap == 0) g->hist_cap = (int)std::min<int64_t>(g->n + 1, 4096);
     FinalizeArgs fa;
-    const bool band = use_band(g, k, opts);
-    std::vector<uint64_t> key = est_key(g, k, opts, out, band);
+    const Lc lc = choose_lc(g, k, opts);
+    std::vector<uint64_t> key = est_key(g, k, opts, out, lc);
     auto &E = g->eg;
     E.replayed = 0;
     if (E.off) {
-        RC(enqueue_bfs_estimate(g, k, hyb, opts, out, band, fa, st));
+        RC(enqueue_bfs_estimate(g, k, hyb, opts, out, lc, fa, st));
         return copy_outputs(g, k, hyb, opts, out, fa, st);
     }
     if (E.exec && E.key != key) {
@@ -1850,12 +1859,12 @@ int run_bfs_estimate(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *
         if (!E.cap) CK(cudaStreamCreateWithFlags(&E.cap, cudaStreamNonBlocking));
         const int kernels0 = g->call_kernels;
         bool ok = cudaStreamBeginCapture(E.cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) ok = enqueue_bfs_estimate(g, k, hyb, opts, out, band, fa, E.cap) == CC_OK;
+        if (ok) ok = enqueue_bfs_estimate(g, k, hyb, opts, out, lc, fa, E.cap) == CC_OK;
         cudaGraph_t gr = nullptr;
         if (cudaStreamEndCapture(E.cap, &gr) != cudaSuccess) ok = false;
         // Buffers must not have moved during the capture (nothing is sized
         // there once the previous call ran with the same arguments).
-        ok = ok && gr && est_key(g, k, opts, out, band) == key;
+        ok = ok && gr && est_key(g, k, opts, out, lc) == key;
         if (ok && cudaGraphInstantiate(&E.exec, gr, 0) != cudaSuccess) {
             E.exec = nullptr;
             ok = false;
@@ -1892,7 +1901,7 @@ int run_bfs_estimate(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *
         g->pend_red[0] = E.pend_red[0]; g->pend_red[1] = E.pend_red[1];
         g->call_kernels += E.kernels;
     } else {
-        RC(enqueue_bfs_estimate(g, k, hyb, opts, out, band, fa, st));
+        RC(enqueue_bfs_estimate(g, k, hyb, opts, out, lc, fa, st));
     }
     return copy_outputs(g, k, hyb, opts, out, fa, st);
 }
