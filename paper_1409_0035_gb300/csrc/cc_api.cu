@@ -238,8 +238,8 @@ struct cc_graph {
     TileGraph tg;
     bool has_tiles = false, on_tiles = false;
     // Distances as bit planes (planes.cu).  on_planes: the last first pass
-    // left them (on distance rows); deep: a pass found more levels than they
-    // hold, so that the next call does not try first.
+    // left them (on distance rows); deep: the last pass whose depth is known
+    // found more levels than they hold, so that the next call does not try.
     DevBuf pl_F, pl_R, pl_masks, pl_c;
     bool on_planes = false, deep = false;
     DevBuf t_dist, t_dirty0, t_dirty1, t_act0, t_act1, t_stamp, t_Q0, t_Q1;
@@ -797,6 +797,16 @@ bool planes_fit(cc_graph *g, int k, int sets)
     return need <= ((double)free_b + held) / 3.0;
 }
 
+// After a first pass over an undirected graph of unit lengths that found
+// `levels` levels.  Beyond twice as many as the planes hold, no node reaches
+// all others within them, and their memory goes back.
+void note_depth(cc_graph *g, int64_t levels)
+{
+    constexpr int64_t top = (1 << kPlanes) - 1;
+    g->deep = levels > top;
+    if (levels > 2 * top) g->pl_F.release();
+}
+
 // The job of the plane kernels; sizes the masks of the hybrid part.
 int plane_job(cc_graph *g, int k, bool roundtrip, PlaneJob &j)
 {
@@ -940,7 +950,8 @@ bool use_band(cc_graph *g, int k, const cc_opts *opts)
 Lc choose_lc(cc_graph *g, int k, const cc_opts *opts)
 {
     if (use_band(g, k, opts)) return Lc::kBand;
-    if (opts->want_hybrid && g->sq && !g->band_off && planes_fit(g, k, 1)) return Lc::kPlanes;
+    if (opts->want_hybrid && g->sq && !g->band_off && !g->deep && planes_fit(g, k, 1))
+        return Lc::kPlanes;
     return Lc::kPass;
 }
 
@@ -1186,6 +1197,7 @@ int chunked_pass1(cc_graph *g, int k, cudaStream_t st, const NwJob *nw = nullptr
     g->call_kernels += 1;
     g->dist_max = (int64_t)dmax;
     g->D1 = (int64_t)dmax;
+    if (!g->weighted && !g->directed) note_depth(g, g->D1);
     return CC_OK;
 }
 
@@ -1476,6 +1488,8 @@ int planes_pass1(cc_graph *g, int k, cudaStream_t st)
     for (int dir = 0; dir < dirs; ++dir)
         if (g->hctl[dir].band_ovf) {
             g->deep = true;
+            g->pl_F.release();
+            g->pl_R.release();
             return 1;
         }
     for (int dir = 0; dir < dirs; ++dir)
@@ -1941,6 +1955,7 @@ int ccg::graph_borrow(cc_graph_t dst, cc_graph_t src)
     dst->sssp_delta = src->sssp_delta;
     dst->reach_words = src->reach_words;
     dst->w_mean = src->w_mean;
+    dst->deep = src->deep;
     dst->borrowed = true;
     return CC_OK;
 }
@@ -2385,6 +2400,7 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     const int c1 = check_pass1(g, hyb, k);
     if (rc != CC_OK) return rc;
     if (c1 == 1) return cc_estimate(g, sample, k, opts, out);  // histogram grown: again
+    if (c1 == CC_OK) note_depth(g, g->D1);
     return c1;
 }
 
@@ -2417,7 +2433,7 @@ int adaptive_run(cc_graph *g, const int32_t *sample, int k, const cc_opts *opts,
     if (chunked) {
         RC(rows_pass1(g, k, st));
     } else {
-        planes = planes_fit(g, k, 1);
+        planes = !g->deep && planes_fit(g, k, 1);
         for (;;) {
             RC(bfs_pass1(g, k, st, 0, 0, planes));
             CK(cudaStreamSynchronize(st));
@@ -2427,6 +2443,7 @@ int adaptive_run(cc_graph *g, const int32_t *sample, int k, const cc_opts *opts,
             RC(c1);
             break;
         }
+        note_depth(g, g->D1);
         planes = planes && !g->hctl[0].band_ovf;
     }
     const bool fused = planes || (chunked && g->on_planes);

@@ -1,5 +1,6 @@
 """What the bit planes leave on a handle: the captured estimate follows the
-parameter that chooses them."""
+parameter that chooses them, graphs too deep for them do not keep their
+memory."""
 import numpy as np
 import pytest
 
@@ -41,3 +42,47 @@ def test_captured_estimate_follows_the_parameter(cc):
                 assert np.array_equal(r[key], seen[0][1][key]), key
     finally:
         cc.cc_graph_free(g)
+
+
+def comet(head, tail, directed):
+    """A dense head with a tail of `tail` nodes; directed: arcs both ways in
+    the tail, a cycle with chords in the head."""
+    rng = np.random.default_rng(head + tail)
+    ring = np.arange(head)
+    s = np.concatenate([ring, rng.integers(0, head, 6 * head), np.arange(head - 1, head + tail - 1)])
+    d = np.concatenate([(ring + 1) % head, rng.integers(0, head, 6 * head),
+                        np.arange(head, head + tail)])
+    if directed:
+        t = np.arange(head - 1, head + tail - 1)
+        s, d = np.concatenate([s, t + 1]), np.concatenate([d, t])
+    return head + tail, s.astype(np.uint32), d.astype(np.uint32)
+
+
+@pytest.mark.parametrize("directed", [False, True])
+def test_planes_of_deep_graphs_are_given_back(cc, directed):
+    """The planes of 1000 sources take 512 bytes a node and direction.  A graph
+    of 60 levels cannot use them: its handle holds less than a shallow one's
+    by more than half of that, other buffers (about 290 and, round trip, the
+    distance rows) set aside."""
+    import torch
+    k, head = 1000, 150_000
+    held = []
+    for tail in (1, 60):
+        n, s, d = comet(head, tail, directed)
+        g, _ = cc.cc_graph_from_edges(n, s, d, directed=directed)
+        try:
+            C = cc.cc_sample_choose(g, k, 4)
+            o = cc.cc_opts_default(k)
+            o.roundtrip = int(directed)
+            torch.cuda.synchronize()
+            before = torch.cuda.mem_get_info()[0]
+            ad = [cc.cc_estimate_adaptive(g, C, o) for _ in range(2)]
+            torch.cuda.synchronize()
+            held.append(before - torch.cuda.mem_get_info()[0])
+            for key in ad[0]:
+                assert np.array_equal(ad[0][key], ad[1][key]), key
+        finally:
+            cc.cc_graph_free(g)
+    if directed:
+        held[1] -= 2 * head * 1024 * 4  # the rows of all sources, both ways
+    assert held[1] < held[0], held
