@@ -85,6 +85,16 @@ size_t footprint(int64_t n, int k, bool directed_or_weighted, bool hybrid)
     return b;
 }
 
+// ... and with its distances as bit planes (round trips on unit lengths): two
+// sets of four words per node and 64 sources, the masks and planes of the
+// distances between sampled nodes.
+size_t plane_bytes(int64_t n, int k)
+{
+    size_t W = 1;
+    while (W * 64 < (size_t)k) W <<= 1;
+    return (size_t)n * W * 64 + (size_t)k * W * (32 * 8 + 40);
+}
+
 }  // namespace
 
 struct cc_server {
@@ -313,6 +323,10 @@ int cc_server_submit(cc_server_t s, int32_t graph, int32_t estimator, int32_t k,
     r->b = eps_den;
     r->footprint = footprint(s->n[graph], k, directed || weighted, estimator == CC_EST_HYBRID);
     if (r->footprint > s->budget) return CC_ERR_TOO_LARGE;
+    // A budget that does not hold the planes besides is charged whole: the
+    // request is taken as ever, and runs alone.
+    if (directed && !weighted)
+        r->footprint += std::min(plane_bytes(s->n[graph], k), s->budget - r->footprint);
     r->arrive = Clock::now();
     {
         std::lock_guard<std::mutex> lk(s->mu);

@@ -1,6 +1,6 @@
 """What the bit planes leave on a handle: the captured estimate follows the
 parameter that chooses them, graphs too deep for them do not keep their
-memory."""
+memory, a server admits requests with them in the account."""
 import numpy as np
 import pytest
 
@@ -86,3 +86,31 @@ def test_planes_of_deep_graphs_are_given_back(cc, directed):
     if directed:
         held[1] -= 2 * head * 1024 * 4  # the rows of all sources, both ways
     assert held[1] < held[0], held
+
+
+def test_server_counts_the_planes(cc):
+    """Two round-trip requests whose workspaces do not fit the budget together
+    do not run together."""
+    n, s, d = synth.watts_strogatz_edges(400_000, 10, 0.5, seed=6)
+    s, d = np.concatenate([s, d]), np.concatenate([d, s])
+    k = 1024
+    g, _ = cc.cc_graph_from_edges(n, s, d, directed=True)
+    try:
+        srv = cc.cc_server_create([g], slots=2)
+        try:
+            rid = cc.cc_server_submit(srv, 0, 0, k, 1)
+            assert cc.cc_server_wait(srv, rid, 60000) == cc.CC_OK
+            one = cc.cc_server_cache_stats(srv)["resident_bytes"]
+        finally:
+            cc.cc_server_free(srv)
+        srv = cc.cc_server_create([g], slots=2, hbm_budget=int(1.7 * one))
+        try:
+            ids = [cc.cc_server_submit(srv, 0, 0, k, 10 + i) for i in range(6)]
+            for rid in ids:
+                assert cc.cc_server_wait(srv, rid, 60000) == cc.CC_OK
+            assert cc.cc_server_stats(srv)["peak_running"] == 1
+            assert cc.cc_server_cache_stats(srv)["resident_bytes"] <= int(1.7 * one)
+        finally:
+            cc.cc_server_free(srv)
+    finally:
+        cc.cc_graph_free(g)
