@@ -1777,6 +1777,16 @@ int copy_outputs(cc_graph *g, int k, bool hyb, const cc_opts *opts, cc_out *out,
     // sample's buffers kept, 455 -> 356 us a call).
     bool stage = !dev_out && total <= kPinBytes && g->host_calls >= 2;
     if (!dev_out && g->host_calls < 2) g->host_calls += 1;
+    // (a device address among them is left to the copies, which take it)
+    for (int i = 0; stage && i < nc; ++i) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, copies[i].to) != cudaSuccess) {
+            cudaGetLastError();
+            stage = false;
+        } else {
+            stage = a.type != cudaMemoryTypeDevice;
+        }
+    }
     if (stage && !g->pin && cudaMallocHost(&g->pin, kPinBytes) != cudaSuccess) {
         cudaGetLastError();
         g->pin = nullptr;
