@@ -28,6 +28,7 @@
 
 
 #include "msbfs_dev.cuh"
+#include "per_device.h"
 
 namespace ccg {
 
@@ -61,20 +62,21 @@ __global__ void barrier_selftest_kernel(Ctl *ctl, uint64_t timeout_ns)
 template <int W>
 int launch_w(const BfsJob &job, cudaStream_t st, int *grid_used)
 {
-    static int blocks_per_sm = -1, sms = 0;
+    static PerDevice<Residency> residency;
     const size_t smem = (size_t)W * 64 * sizeof(unsigned);
-    if (blocks_per_sm < 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return CC_ERR_CUDA;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return CC_ERR_CUDA;
+    Residency fit;
+    const int rc = residency.get(dev, &fit, [&](Residency &r) -> int {
+        if (cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return CC_ERR_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm,
-                                                          msbfs_kernel<W>, kBlock,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.per_sm, msbfs_kernel<W>, kBlock,
                                                           smem) != cudaSuccess)
             return CC_ERR_CUDA;
-        if (blocks_per_sm < 1) return CC_ERR_CUDA;
-    }
-    int grid = blocks_per_sm * sms;
+        return r.per_sm < 1 ? CC_ERR_CUDA : CC_OK;
+    });
+    if (rc != CC_OK) return rc;
+    int grid = fit.per_sm * fit.sms;
     if (job.max_ctas > 0 && job.max_ctas < grid) grid = job.max_ctas;
     if (grid_used) *grid_used = grid;
     BfsJob j = job;

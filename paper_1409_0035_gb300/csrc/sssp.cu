@@ -21,6 +21,7 @@
 
 #include "barrier.cuh"
 #include "cc_internal.h"
+#include "per_device.h"
 #include "sssp.h"
 
 namespace ccg {
@@ -450,22 +451,24 @@ int grid_of(int64_t n)
 
 int launch_mssp(const SsspJob &job, cudaStream_t st)
 {
-    static int blocks_per_sm[2] = {-1, -1}, sms = 0;
+    static PerDevice<Residency> residency[2];
     const int q = job.spl == 2 ? 1 : 0;
     const void *fn = q ? (const void *)mssp_kernel<2> : (const void *)mssp_kernel<1>;
-    if (blocks_per_sm[q] < 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return CC_ERR_CUDA;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return CC_ERR_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[q], fn, kBlock, 0) !=
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return CC_ERR_CUDA;
+    Residency fit;
+    const int rc = residency[q].get(dev, &fit, [&](Residency &r) -> int {
+        if (cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.per_sm, fn, kBlock, 0) !=
                 cudaSuccess ||
-            blocks_per_sm[q] < 1)
+            r.per_sm < 1)
             return CC_ERR_CUDA;
-    }
+        return CC_OK;
+    });
+    if (rc != CC_OK) return rc;
     SsspJob j = job;
     void *args[] = {&j};
-    int grid = blocks_per_sm[q] * sms;
+    int grid = fit.per_sm * fit.sms;
     if (job.max_ctas > 0 && job.max_ctas < grid) grid = job.max_ctas;
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBlock), args, 0, st) == cudaSuccess
                ? CC_OK

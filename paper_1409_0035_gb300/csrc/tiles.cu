@@ -23,6 +23,7 @@
 
 #include "barrier.cuh"
 #include "graph_gpu.h"
+#include "per_device.h"
 #include "tiles.h"
 
 namespace ccg {
@@ -1139,23 +1140,24 @@ int tile_unit_words(const TileGraph &g, int k)
 
 int launch_tiles(const TileJob &job, cudaStream_t st)
 {
-    static int per[2] = {-1, -1}, sms = 0;
+    // The shared memory opted into is a device's, like the residency.
+    static PerDevice<Residency> residency[2];
     const int q = job.g.iw ? 1 : 0;
     const void *fn = q ? (const void *)k_tiles<true> : (const void *)k_tiles<false>;
     const size_t smem = q ? sizeof(TileShared<true>) : sizeof(TileShared<false>);
     const int threads = q ? kTileThreads<true> : kTileThreads<false>;
-    if (per[q] < 0) {
-        int dev = 0, b = 0;
-        T_CK(cudaGetDevice(&dev));
-        T_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int dev = 0;
+    T_CK(cudaGetDevice(&dev));
+    Residency fit;
+    T_RC(residency[q].get(dev, &fit, [&](Residency &r) -> int {
+        T_CK(cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev));
         T_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        T_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem));
-        if (b < 1) return CC_ERR_CUDA;
-        per[q] = b;
-    }
+        T_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.per_sm, fn, threads, smem));
+        return r.per_sm < 1 ? CC_ERR_CUDA : CC_OK;
+    }));
     TileJob j = job;
     void *args[] = {&j};
-    T_CK(cudaLaunchCooperativeKernel(fn, dim3(per[q] * sms), dim3(threads), args, smem, st));
+    T_CK(cudaLaunchCooperativeKernel(fn, dim3(fit.per_sm * fit.sms), dim3(threads), args, smem, st));
     return CC_OK;
 }
 
