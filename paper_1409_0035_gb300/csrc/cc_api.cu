@@ -1275,18 +1275,20 @@ int chunked_hybrid(cc_graph *g, int k, uint32_t a, uint32_t b, cudaStream_t st)
     return CC_OK;
 }
 
-// Whether an estimate of k sources runs on the graph's tiles: not under a
-// setting of the search they replace (the direction switch or the two-pass
-// form on unit lengths, the bucket width with arc lengths), not in a server
-// slot (its launches are capped and its footprint is admitted for the other
-// path; a batch lends its handle the tiles), and while the labels fit a third of the memory that is free or
+// Whether an estimate of k sources (passes: see tiles_pay) runs on the graph's
+// tiles: where they are the faster search; not under a setting of the search
+// they replace (the direction switch or the two-pass form on unit lengths, the
+// bucket width with arc lengths), not in a server slot (its launches are capped
+// and its footprint is admitted for the other path; a batch lends its handle
+// the tiles), and while the labels fit a third of the memory that is free or
 // already held by them.
-bool use_tiles(cc_graph *g, int64_t k)
+bool use_tiles(cc_graph *g, int64_t k, int passes)
 {
     if (!g->has_tiles || (g->borrowed && !g->tiles_lent) || g->max_ctas > 0) return false;
     if (g->weighted ? g->sssp_delta != 0
                     : g->band_off || g->alpha != 0 || g->tg.levels < kTileMinLevels)
         return false;
+    if (!tiles_pay(g->tg, k, passes)) return false;
     const double need = (double)k * (double)g->tg.slots * 4.25;
     if ((double)g->t_dist.cap + (double)g->t_dirty0.cap * 2.0 >= need) return true;
     size_t free_b = 0, total_b = 0;
@@ -1980,7 +1982,7 @@ int ccg::graph_borrow_tiles(cc_graph_t dst, cc_graph_t src)
     return CC_OK;
 }
 
-bool ccg::graph_takes_tiles(cc_graph_t src, int64_t k) { return use_tiles(src, k); }
+bool ccg::graph_takes_tiles(cc_graph_t src, int64_t k) { return use_tiles(src, k, 1); }
 
 int ccg::graph_choose_sample(cc_graph_t g, int64_t n, int k, uint64_t seed, int32_t *host_out)
 {
@@ -2139,7 +2141,7 @@ int cc_graph_from_edges(int64_t n, int64_t m, const uint32_t *src, const uint32_
         rc = build_csr_device(n, m, src, dst, w, keep_component != 0, d);
         if (rc == CC_OK) rc = adopt_device_csr(g, d);
         if (rc == CC_OK) rc = cut_tiles(g);
-        if (rc == CC_OK && w && !g->has_tiles) rc = build_locality(g);
+        if (rc == CC_OK && w && !(g->has_tiles && tiles_pay(g->tg, 1, 1))) rc = build_locality(g);
         if (d.rp) cudaFree(d.rp);
         if (d.col) cudaFree(d.col);
         if (d.w) cudaFree(d.w);
@@ -2335,7 +2337,7 @@ namespace {
 // buffers: their sizes are what the server accounts.
 int make_slab(cc_graph *g, int k, const cc_opts *opts)
 {
-    if (g->slab.p || g->borrowed || g->vis.p || g->weighted || g->directed || use_tiles(g, k))
+    if (g->slab.p || g->borrowed || g->vis.p || g->weighted || g->directed || g->on_tiles)
         return CC_OK;
     const size_t n = (size_t)g->n, W = (size_t)pow2_words(k), K = (size_t)k;
     const size_t nt = (size_t)g->fw.cls.nT, nch = (size_t)g->fw.cls.nHch;
@@ -2371,6 +2373,9 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     reset_timing(g);
     cudaStream_t st = (cudaStream_t)opts->stream;
     const int64_t n = g->n;
+    const bool hyb = opts->want_hybrid != 0;
+    g->sq = hyb && out->sq_err != nullptr;
+    g->on_tiles = use_tiles(g, k, g->sq ? 2 : 1);
     RC(make_slab(g, k, opts));
     const SlabScope scope(g->slab.p ? &g->slab : nullptr);
     RC(g->sidx.ensure(n * 4));
@@ -2382,9 +2387,6 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k, const cc_opts *o
     RC(g->sources.ensure((size_t)k * 4));
     RC(g->ctl.ensure(sizeof(Ctl)));
     CK(cudaMemcpyAsync(g->sources.p, sample, (size_t)k * 4, cudaMemcpyHostToDevice, st));
-    const bool hyb = opts->want_hybrid != 0;
-    g->sq = hyb && out->sq_err != nullptr;
-    g->on_tiles = use_tiles(g, k);
     int rc = CC_OK;
     do {
         if (!on_rows(g)) {
@@ -2534,7 +2536,7 @@ int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k, const c
     RC(validate_sample(g, sample, k));
     reset_timing(g);
     cudaStream_t st = (cudaStream_t)opts->stream;
-    g->on_tiles = use_tiles(g, k);
+    g->on_tiles = use_tiles(g, k, 1 + n_eps);
     int rc;
     do
         rc = adaptive_run(g, sample, k, opts, n_eps, eps_num, eps_den, s_hat, closeness, sq_err,

@@ -1096,8 +1096,7 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     // sides of arcs to each, five to seven rounds per tile across; 464 K nodes,
     // k = 64: tiles 77 ms, buckets 47).  Street lattices have 4 to 6 neighbours
     // or borders of 0.2 to 0.4 sides, two and a half rounds (478 K: 9.4
-    // against 35 ms).  On unit lengths tiles stay ahead on both (464 K: 60
-    // against 119 ms).
+    // against 35 ms).  tiles_pay decides on the others by the call.
     // (Below 64 tiles most lie at the rim and have few neighbours anyway.)
     if (w && tiles >= 64 && (double)h[1] < 4.0 * (double)tiles &&
         (double)ex > 0.5 * std::sqrt((double)n / (double)tiles) * (double)h[1])
@@ -1107,6 +1106,10 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     out.tiles = (int32_t)tiles;
     // a tile is about two mean radii across
     out.levels = 2.0 * (double)h[2] / (double)n * (double)h[3];
+    out.depth = (double)h[3];
+    out.neighbours = (double)h[1] / (double)tiles;
+    out.border = (double)ex / (double)std::max(1ull, h[1]) /
+                 std::sqrt((double)n / (double)tiles);
     out.perm = perm.take<int32_t>();
     out.iperm = iperm.take<int32_t>();
     out.tb = tb.take<int32_t>();
@@ -1130,6 +1133,43 @@ void tiles_free(TileGraph &g)
     for (void *x : p)
         if (x) cudaFree(x);
     g = TileGraph{};
+}
+
+// Tiles whose borders to each neighbour are longer than a side interleave:
+// fronts cross them to and fro, 5 to 10 levels a round in place of 16 to 32,
+// and once there are enough tiles to fill the GPU a label costs five times as
+// much (120 to 200 ns a tile and source, elsewhere 14 to 35).  Tiles against
+// the other search on thinned random geometric graphs:
+// - one bit-packed pass: 60 K nodes of degree 2.6 (2.5 neighbours, 1.5 sides)
+//   k = 64 13.4 / 13.7 ms, k = 256 22 / 16, k = 1024 55 / 21; of degree 4 (5.6,
+//   1.6) k = 8 8.3 / 5.7, k = 256 19 / 6.6;
+// - two passes (the error estimate): degree 2.6 k = 128 18 / 37, degree 4 k = 8
+//   8.4 / 11.9; from four on (the adaptive hybrid) tiles were ahead
+//   everywhere, 64 / 76 ms at the least;
+// - few tiles run side by side at any k: degree 2.6, 14 K nodes k = 256 5.8 /
+//   10.2, 18 K (2.5 sides) k = 128 5.1 / 5.7, but 7 K (3.3 sides) 7.3 / 5.4;
+// - with arc lengths the other search takes 64 sources at a time: degree 4,
+//   60 K nodes k = 64 11.9 / 7.5, k = 200 17 / 26, 16 K 11.0 / 3.1, 12.6 / 11.2.
+// Shortcuts (more tiles than three times the square of the tiles across)
+// leave few levels: 200 K-node rings, 0.5 % rewired, k = 64 3.0 / 4.6 ms, k =
+// 256 10.0 / 6.0; 20 K nodes, 1 %, k = 512 2.0 / 2.5, k = 2048 5.7 / 3.3.
+// Lattices with or without gaps, mazes, honeycombs and trees (borders of 0.1 to
+// 0.9 sides, below 64 tiles, most of them at the rim, up to 1.4) gain 1.2 to 16
+// times from k = 1 to 2048; so do strips a tile or two wide (0.6 to 1.03), told
+// by the levels for their tiles (30 x 2000, 11: k = 2048 20 / 62 ms).
+bool tiles_pay(const TileGraph &g, int64_t k, int passes)
+{
+    if (g.border > (g.tiles < 64 ? 1.7 : 1.0) && g.levels < 8.0 * (double)g.tiles) {
+        const bool thin = g.neighbours < 2.7 &&
+                          (g.border < 1.6 || (g.tiles < 128 && g.border < 2.5));
+        if (g.iw) return thin || k > 192;
+        if (passes >= 4) return true;
+        if (thin) return k <= 64 * passes || g.tiles * k <= 24576 * passes;
+        return k <= 32 * (passes - 1);
+    }
+    if (!g.iw && (double)g.tiles > 3.0 * g.depth * g.depth)
+        return (double)g.tiles * (double)k <= 1000.0 * passes * g.levels;
+    return true;
 }
 
 int tile_unit_words(const TileGraph &g, int k)

@@ -23,6 +23,9 @@ struct TileGraph {
     int64_t n = 0, slots = 0;
     int32_t tiles = 0;
     double levels = 0.0;                         // estimated hops across the graph
+    double depth = 0.0;                          // tiles across it, from one of them
+    double neighbours = 0.0;                     // neighbouring tiles of a tile, mean
+    double border = 0.0;                         // arcs to each over the nodes of a side
     int32_t *perm = nullptr, *iperm = nullptr;   // slot -> node, node -> slot
     int32_t *tb = nullptr;                       // tiles + 1: first slot of each
     int32_t *word_tile = nullptr;                // slots / 32: the word's tile
@@ -57,6 +60,10 @@ struct TileJob {
     Ctl *ctl;                   // band_ovf: some candidate label reached 2^32 - 1
     uint64_t timeout_ns;
 };
+
+// Whether a search of k sources by tiles is the faster one; passes: traversals
+// of all sources that a level-synchronous estimate would make in its place.
+bool tiles_pay(const TileGraph &g, int64_t k, int passes);
 
 // Words per unit for k sources: as many as leave every CTA of the GPU two
 // units of a fully active round.
