@@ -280,11 +280,11 @@ k_digit_scatter(const uint64_t *keys, const uint32_t *vals, int64_t n, int shift
 
 // ---------------------------------------------------------------- arcs
 
-// Arc keys (tail << b | head) with their lengths: both ways for undirected
-// input, one way (second slot unused) for directed input.
+// Arc keys (tail << b | head) of directed input with their lengths; flags: the
+// arcs to keep (no self-loops).
 __global__ void k_make_arcs(const uint32_t *src, const uint32_t *dst, const uint32_t *w,
                             int64_t m, int64_t n, int b, uint64_t *keys, uint32_t *vals,
-                            uint64_t *flags, int *err, int both)
+                            uint64_t *flags, int *err)
 {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -292,13 +292,9 @@ __global__ void k_make_arcs(const uint32_t *src, const uint32_t *dst, const uint
         const uint32_t ww = w ? w[e] : 1u;
         if ((int64_t)u >= n || (int64_t)v >= n) atomicExch(err, CC_ERR_GRAPH);
         if (ww == 0) atomicExch(err, CC_ERR_ARG);
-        const uint64_t keep = u != v && (int64_t)u < n && (int64_t)v < n;
-        keys[2 * e] = (u << b) | v;
-        keys[2 * e + 1] = (v << b) | u;
-        vals[2 * e] = ww;
-        vals[2 * e + 1] = ww;
-        flags[2 * e] = keep;
-        flags[2 * e + 1] = both ? keep : 0;
+        keys[e] = (u << b) | v;
+        vals[e] = ww;
+        flags[e] = u != v && (int64_t)u < n && (int64_t)v < n;
     }
 }
 
@@ -1479,16 +1475,15 @@ int build_csr_device_directed(int64_t n, int64_t m, const uint32_t *h_src, const
     cudaStream_t st = 0;
     int b = 1;
     while ((1ll << b) < n) ++b;
-    const int64_t A0 = 2 * m;  // k_make_arcs writes two slots per input edge
     Buf dsrc, ddst, dw, k0, v0, k1, v1, fl, pos, err;
     G_RC(dsrc.alloc(m * 4));
     G_RC(ddst.alloc(m * 4));
     if (h_w) G_RC(dw.alloc(m * 4));
-    G_RC(k0.alloc(std::max<int64_t>(A0, 1) * 8));
-    G_RC(v0.alloc(std::max<int64_t>(A0, 1) * 4));
-    G_RC(k1.alloc(std::max<int64_t>(A0, 1) * 8));
-    G_RC(v1.alloc(std::max<int64_t>(A0, 1) * 4));
-    const int64_t FL = std::max<int64_t>(A0, n) + 1;
+    G_RC(k0.alloc(std::max<int64_t>(m, 1) * 8));
+    G_RC(v0.alloc(std::max<int64_t>(m, 1) * 4));
+    G_RC(k1.alloc(std::max<int64_t>(m, 1) * 8));
+    G_RC(v1.alloc(std::max<int64_t>(m, 1) * 4));
+    const int64_t FL = std::max<int64_t>(m, n) + 1;
     G_RC(fl.alloc(FL * 8));
     G_RC(pos.alloc(FL * 8));
     G_RC(err.alloc(4));
@@ -1504,16 +1499,16 @@ int build_csr_device_directed(int64_t n, int64_t m, const uint32_t *h_src, const
         k_make_arcs<<<gsz(m), 256, 0, st>>>(dsrc.as<uint32_t>(), ddst.as<uint32_t>(),
                                             h_w ? dw.as<uint32_t>() : nullptr, m, n, b,
                                             k0.as<uint64_t>(), v0.as<uint32_t>(),
-                                            fl.as<uint64_t>(), err.as<int>(), 0);
+                                            fl.as<uint64_t>(), err.as<int>());
     int herr = 0;
     G_CK(cudaMemcpy(&herr, err.p, 4, cudaMemcpyDeviceToHost));
     if (herr) return herr;
     uint64_t A1 = 0;
-    G_RC(scan_u64(fl.as<uint64_t>(), pos.as<uint64_t>(), A0, &A1, st));
-    if (A0 > 0)
-        k_compact<<<gsz(A0), 256, 0, st>>>(k0.as<uint64_t>(), v0.as<uint32_t>(),
-                                           fl.as<uint64_t>(), pos.as<uint64_t>(), A0,
-                                           k1.as<uint64_t>(), v1.as<uint32_t>());
+    G_RC(scan_u64(fl.as<uint64_t>(), pos.as<uint64_t>(), m, &A1, st));
+    if (m > 0)
+        k_compact<<<gsz(m), 256, 0, st>>>(k0.as<uint64_t>(), v0.as<uint32_t>(), fl.as<uint64_t>(),
+                                          pos.as<uint64_t>(), m, k1.as<uint64_t>(),
+                                          v1.as<uint32_t>());
     bool in_tmp = false;
     if (A1 > 0)
         G_RC(radix_sort(k1.as<uint64_t>(), v1.as<uint32_t>(), (int64_t)A1, 2 * b,
