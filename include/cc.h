@@ -84,7 +84,8 @@ typedef struct cc_graph *cc_graph_t;
  *                  from cc_graph_info); entries beyond n' are untouched
  * Self-loops are dropped, parallel arcs merged keeping the smallest length,
  * kept nodes renumbered 0..n'-1 in increasing original id, adjacency lists
- * sorted by neighbour.  Errors: CC_ERR_ARG, CC_ERR_GRAPH, CC_ERR_OOM,
+ * sorted by neighbour.  An undirected graph that suits the search by tiles is
+ * cut into them where memory allows.  Errors: CC_ERR_ARG, CC_ERR_GRAPH, CC_ERR_OOM,
  * CC_ERR_CUDA, CC_ERR_TOO_LARGE (more than 2^31-1 arcs or nodes).
  */
 int cc_graph_from_edges(int64_t n, int64_t m, const uint32_t *src,
@@ -180,7 +181,9 @@ void cc_opts_default(cc_opts *o, int32_t k);
  * hybrid needs per-node thresholds below the largest sampled distance, a
  * second pass with the per-node L(v) masks (section 3, Algorithm 1).
  * Errors: CC_ERR_ARG, CC_ERR_DISCONNECTED, CC_ERR_OOM, CC_ERR_TIMEOUT,
- * CC_ERR_CUDA, CC_ERR_TOO_LARGE (a distance >= 2^32-1).
+ * CC_ERR_CUDA, CC_ERR_TOO_LARGE (a distance to a node, or by any of its arcs
+ * back, >= 2^32-1; with the hybrid and arc lengths or round trips, more than
+ * 2^30 (distance, source) pairs; sums of squared distances beyond 64 bits).
  */
 int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k,
                 const cc_opts *opts, cc_out *out);
@@ -196,9 +199,10 @@ int cc_estimate(cc_graph_t g, const int32_t *sample, int32_t k,
  * opts->device_outputs, any may be NULL: s_hat (sampled nodes: exact S),
  * closeness (n-1)/s_hat, sq_err (0 for sampled nodes), choice (the entry
  * used; -1 for sampled nodes).  opts->eps_* and want_hybrid are ignored;
- * roundtrip must match the graph.  Each entry costs the ε-dependent part of
- * cc_estimate again: thresholds and, where some node needs it, the second
- * traversal pass.  Errors: as cc_estimate; CC_ERR_ARG for n_eps outside
+ * roundtrip must match the graph.  On bit planes one kernel serves every
+ * entry; else each costs the ε-dependent part of cc_estimate again: thresholds
+ * and, where some node needs it, the second traversal pass or the sums over
+ * the rows.  Errors: as cc_estimate; CC_ERR_ARG for n_eps outside
  * 1..64 or an entry with eps_num = 0 or eps_num > eps_den.
  */
 int cc_estimate_adaptive(cc_graph_t g, const int32_t *sample, int32_t k,
@@ -481,8 +485,7 @@ int cc_server_free(cc_server_t s);
 
 /* ---- tuning ---------------------------------------------------------------- */
 /* Direction switch of the breadth-first traversal of one graph (0 restores
- * the default: 6 when the sample fits one 64-bit word and the mean degree
- * is at least 8, else 14): a level
+ * the default, chosen by the sample's words and the mean degree): a level
  * runs top-down while (CSR entries of the frontier) * alpha < (CSR entries
  * of the nodes some source has not reached yet), bottom-up otherwise.
  * A value other than 0 also keeps this search where the graph would be
@@ -501,10 +504,11 @@ int cc_set_tuning(cc_graph_t g, int32_t alpha);
  *                             ones (a byte per node and source) to resolve
  *                             once the distances between sampled nodes are
  *                             known, so no second traversal runs unless a
- *                             band offset exceeds a byte, the error estimate
- *                             is asked for, or the rows do not fit a third
- *                             of the free memory; 0: always the two-pass
- *                             form (no tiles)
+ *                             band offset exceeds a byte or the rows do not
+ *                             fit a third of the free memory; with the error
+ *                             estimate the distances as bit planes, while
+ *                             they stay below 16, in place of these; 0:
+ *                             always the two-pass form (no planes, no tiles)
  *   CC_PARAM_SSSP_DELTA       bucket width of the shortest-path rounds with
  *                             arc lengths (delta-stepping with a near and a
  *                             far queue: labels below the threshold relax
@@ -538,8 +542,9 @@ int cc_set_param(cc_graph_t g, int32_t param, int32_t value);
 
 /* ---- diagnostics --------------------------------------------------------- */
 /* Counters of the last traversal pass run on g: levels, top-down and
- * bottom-up levels, CSR entries examined and frontier words gathered.
- * Any pointer may be NULL. */
+ * bottom-up levels, CSR entries examined and frontier words gathered (a
+ * search by tiles: its rounds, and as words the labels carried on).  Any
+ * pointer may be NULL. */
 int cc_last_pass_stats(cc_graph_t g, int64_t *levels, int64_t *td_levels,
                        int64_t *bu_levels, int64_t *edges_examined,
                        int64_t *words_gathered);
@@ -566,14 +571,16 @@ enum {
 /* Warp time by phase of the last bit-packed traversal pass on g (tracing;
  * the paper has no counterpart): warp_cycles[p] (caller-owned, CC_NUM_PHASES
  * entries) receives the SM clock cycles summed over all warps spent in phase
- * p.  Only the shares are meaningful.  Zero after a weighted pass. */
+ * p.  Only the shares are meaningful.  Zero after a weighted pass or a search by
+ * tiles. */
 int cc_last_pass_phases(cc_graph_t g, int64_t *warp_cycles);
 
 /* Per-level trace of the last traversal pass on g (levels 1 .. D, at most
  * max_levels and at most 64): device time of each level in ns (global timer
  * on the device), whether it ran top-down (1) or bottom-up (0), the frontier
  * size it started from, the CSR entries of that frontier and the frontier
- * words it gathered.  Entry 0 is zero; any pointer may be NULL.  Returns the
+ * words it gathered; zeros after a search by tiles, whose rounds it does not
+ * trace.  Entry 0 is zero; any pointer may be NULL.  Returns the
  * number of entries written (D + 1, capped) or a negative CC_ERR_* code. */
 int cc_last_pass_trace(cc_graph_t g, int32_t max_levels, int64_t *level_ns,
                        int32_t *top_down, int64_t *frontier,

@@ -1147,7 +1147,7 @@ void tiles_free(TileGraph &g)
 //   8.4 / 11.9; from four on (the adaptive hybrid) tiles were ahead
 //   everywhere, 64 / 76 ms at the least;
 // - few tiles run side by side at any k: degree 2.6, 14 K nodes k = 256 5.8 /
-//   10.2, 18 K (2.5 sides) k = 128 5.1 / 5.7, but 7 K (3.3 sides) 7.3 / 5.4;
+//   10.2, 18 K (2.5 sides) k = 128 9.3 / 10.5, but 7 K (3.3 sides) 7.3 / 5.4;
 // - with arc lengths the other search takes 64 sources at a time: degree 4,
 //   60 K nodes k = 64 11.9 / 7.5, k = 200 17 / 26, 16 K 11.0 / 3.1, 12.6 / 11.2.
 // Shortcuts (more tiles than three times the square of the tiles across)

@@ -65,8 +65,9 @@ struct TileJob {
 // of all sources that a level-synchronous estimate would make in its place.
 bool tiles_pay(const TileGraph &g, int64_t k, int passes);
 
-// Words per unit for k sources: as many as leave every CTA of the GPU two
-// units of a fully active round.
+// Words per unit for k sources: as many as leave a fully active round 1,216
+// units, two for every CTA on unit lengths (4 a SM) and about one with arc
+// lengths (6 or 7 a SM).
 int tile_unit_words(const TileGraph &g, int k);
 int launch_tiles(const TileJob &job, cudaStream_t st);
 
