@@ -784,18 +784,18 @@ __device__ void bfs_pass(const BfsJob &J, unsigned team_rank, unsigned team_size
         J.F1[i] = 0;
         J.nxt[i] = 0;
     }
+    // A pass may end before it has reached every node (a graph in parts, a
+    // histogram that turns out too short): the kernels queued behind it index
+    // by the pivot all the same, so it starts at 0.
+    const bool piv = (J.red & RED_PIVOT) != 0;
     for (int64_t v = gtid; v < n; v += gthreads) {
         J.tflag[v] = 0;
         J.fstamp[v] = kInf;
-    }
-    // A pass may end before it has reached every node (a graph in parts, a
-    // histogram that turns out too short): the kernels queued behind it index
-    // by the pivot all the same.
-    if (J.red & RED_PIVOT)
-        for (int64_t v = gtid; v < n; v += gthreads) {
+        if (piv) {
             J.pivot[v] = 0;
             J.delta[v] = 0;
         }
+    }
     for (int i = tid; i < W * 64; i += kBlock) s_hist[i] = 0;
     if (J.red & RED_LC)
         for (int64_t i = gtid; i < 2 * n; i += gthreads) J.lc2[i] = 0;
