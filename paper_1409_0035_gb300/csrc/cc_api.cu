@@ -236,6 +236,7 @@ struct cc_graph {
     // Undirected graphs of short rows, cut into tiles (tiles.cu); their
     // search's rows and queues.  on_tiles: the last first pass ran on them.
     TileGraph tg;
+    TileShape tshape;
     bool has_tiles = false, on_tiles = false;
     // Distances as bit planes (planes.cu).  on_planes: the last first pass
     // left them (on distance rows); deep: the last pass whose depth is known
@@ -640,7 +641,7 @@ int cut_tiles(cc_graph *g)
     if (g->directed || g->n < kTileMinNodes || c.nM + c.nH > 0 || 2 * c.nT < g->n) return CC_OK;
     const int rc = tiles_build(g->n, g->arcs, g->fw.rp.as<int64_t>(), g->fw.col.as<int32_t>(),
                                g->weighted ? g->fw.w.as<uint32_t>() : nullptr, g->tg,
-                               &g->has_tiles, 0);
+                               g->tshape, &g->has_tiles, 0);
     if (rc != CC_OK && rc != CC_ERR_OOM) return rc;
     CK(cudaDeviceSynchronize());  // estimates may run on other streams
     return CC_OK;
@@ -1288,7 +1289,7 @@ bool use_tiles(cc_graph *g, int64_t k, int passes)
     if (g->weighted ? g->sssp_delta != 0
                     : g->band_off || g->alpha != 0 || g->tg.levels < kTileMinLevels)
         return false;
-    if (!tiles_pay(g->tg, k, passes)) return false;
+    if (!tiles_pay(g->tg, g->tshape, k, passes)) return false;
     const double need = (double)k * (double)g->tg.slots * 4.25;
     if ((double)g->t_dist.cap + (double)g->t_dirty0.cap * 2.0 >= need) return true;
     size_t free_b = 0, total_b = 0;
@@ -1978,6 +1979,7 @@ int ccg::graph_borrow_tiles(cc_graph_t dst, cc_graph_t src)
 {
     RC(graph_borrow(dst, src));
     dst->tg = src->tg;
+    dst->tshape = src->tshape;
     dst->has_tiles = dst->tiles_lent = src->has_tiles;
     return CC_OK;
 }
@@ -2141,7 +2143,8 @@ int cc_graph_from_edges(int64_t n, int64_t m, const uint32_t *src, const uint32_
         rc = build_csr_device(n, m, src, dst, w, keep_component != 0, d);
         if (rc == CC_OK) rc = adopt_device_csr(g, d);
         if (rc == CC_OK) rc = cut_tiles(g);
-        if (rc == CC_OK && w && !(g->has_tiles && tiles_pay(g->tg, 1, 1))) rc = build_locality(g);
+        if (rc == CC_OK && w && !(g->has_tiles && tiles_pay(g->tg, g->tshape, 1, 1)))
+            rc = build_locality(g);
         if (d.rp) cudaFree(d.rp);
         if (d.col) cudaFree(d.col);
         if (d.w) cudaFree(d.w);

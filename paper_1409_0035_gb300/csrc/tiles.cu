@@ -985,7 +985,7 @@ __global__ void k_tr_lc(TileReduce R)
 }  // namespace
 
 int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
-                const uint32_t *w, TileGraph &out, bool *ok, cudaStream_t st)
+                const uint32_t *w, TileGraph &out, TileShape &shape, bool *ok, cudaStream_t st)
 {
     *ok = false;
     const int cap = tile_cap(w != nullptr);
@@ -1106,10 +1106,10 @@ int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
     out.tiles = (int32_t)tiles;
     // a tile is about two mean radii across
     out.levels = 2.0 * (double)h[2] / (double)n * (double)h[3];
-    out.depth = (double)h[3];
-    out.neighbours = (double)h[1] / (double)tiles;
-    out.border = (double)ex / (double)std::max(1ull, h[1]) /
-                 std::sqrt((double)n / (double)tiles);
+    shape.depth = (double)h[3];
+    shape.neighbours = (double)h[1] / (double)tiles;
+    shape.border = (double)ex / (double)std::max(1ull, h[1]) /
+                   std::sqrt((double)n / (double)tiles);
     out.perm = perm.take<int32_t>();
     out.iperm = iperm.take<int32_t>();
     out.tb = tb.take<int32_t>();
@@ -1157,17 +1157,17 @@ void tiles_free(TileGraph &g)
 // 0.9 sides, below 64 tiles, most of them at the rim, up to 1.4) gain 1.2 to 16
 // times from k = 1 to 2048; so do strips a tile or two wide (0.6 to 1.03), told
 // by the levels for their tiles (30 x 2000, 11: k = 2048 20 / 62 ms).
-bool tiles_pay(const TileGraph &g, int64_t k, int passes)
+bool tiles_pay(const TileGraph &g, const TileShape &s, int64_t k, int passes)
 {
-    if (g.border > (g.tiles < 64 ? 1.7 : 1.0) && g.levels < 8.0 * (double)g.tiles) {
-        const bool thin = g.neighbours < 2.7 &&
-                          (g.border < 1.6 || (g.tiles < 128 && g.border < 2.5));
+    if (s.border > (g.tiles < 64 ? 1.7 : 1.0) && g.levels < 8.0 * (double)g.tiles) {
+        const bool thin = s.neighbours < 2.7 &&
+                          (s.border < 1.6 || (g.tiles < 128 && s.border < 2.5));
         if (g.iw) return thin || k > 192;
         if (passes >= 4) return true;
         if (thin) return k <= 64 * passes || g.tiles * k <= 24576 * passes;
         return k <= 32 * (passes - 1);
     }
-    if (!g.iw && (double)g.tiles > 3.0 * g.depth * g.depth)
+    if (!g.iw && (double)g.tiles > 3.0 * s.depth * s.depth)
         return (double)g.tiles * (double)k <= 1000.0 * passes * g.levels;
     return true;
 }

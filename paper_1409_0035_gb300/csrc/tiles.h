@@ -23,9 +23,6 @@ struct TileGraph {
     int64_t n = 0, slots = 0;
     int32_t tiles = 0;
     double levels = 0.0;                         // estimated hops across the graph
-    double depth = 0.0;                          // tiles across it, from one of them
-    double neighbours = 0.0;                     // neighbouring tiles of a tile, mean
-    double border = 0.0;                         // arcs to each over the nodes of a side
     int32_t *perm = nullptr, *iperm = nullptr;   // slot -> node, node -> slot
     int32_t *tb = nullptr;                       // tiles + 1: first slot of each
     int32_t *word_tile = nullptr;                // slots / 32: the word's tile
@@ -38,11 +35,19 @@ struct TileGraph {
     uint32_t *iw = nullptr, *ew = nullptr;       // their lengths (null: unit lengths)
 };
 
+// How its tiles lie: for the host.  (The kernels take a TileGraph by value; with
+// these three in it the road network's estimate took 0.5 % longer.)
+struct TileShape {
+    double depth = 0.0;       // tiles across the graph, from one of them
+    double neighbours = 0.0;  // neighbouring tiles of a tile, mean
+    double border = 0.0;      // arcs to each over the nodes of a tile's side
+};
+
 // Cuts an undirected CSR (rows of at most kLightMaxDeg entries; w null: unit
 // lengths) into tiles.  *ok = false, and nothing kept, when the tiles would
 // not be local: see tiles.cu.
 int tiles_build(int64_t n, int64_t arcs, const int64_t *rp, const int32_t *col,
-                const uint32_t *w, TileGraph &out, bool *ok, cudaStream_t st);
+                const uint32_t *w, TileGraph &out, TileShape &shape, bool *ok, cudaStream_t st);
 void tiles_free(TileGraph &g);
 
 struct TileJob {
@@ -63,7 +68,7 @@ struct TileJob {
 
 // Whether a search of k sources by tiles is the faster one; passes: traversals
 // of all sources that a level-synchronous estimate would make in its place.
-bool tiles_pay(const TileGraph &g, int64_t k, int passes);
+bool tiles_pay(const TileGraph &g, const TileShape &s, int64_t k, int passes);
 
 // Words per unit for k sources: as many as leave a fully active round 1,216
 // units, two for every CTA on unit lengths (4 a SM) and about one with arc
