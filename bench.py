@@ -705,7 +705,7 @@ def run_extra(args):
                     unweighted_hybrid_ms=t_u, tau=list(tau),
                     certain=int((beta[C].astype(np.uint64) * tau[1] >= tau[0]).sum()),
                     note="value = k m / weighted-hybrid time; the weighted estimate runs "
-                         "on chunks of distance rows (two sweeps for the hybrid)",
+                         "on the distances as bit planes while they stay below 16",
                     config={"workload": "nodeweighted", "graph": f"R-MAT scale {SCALE}, "
                             f"edge factor {EF}, seed {GSEED}, LCC", "n": nn, "m": m, "k": K,
                             "node_weights": "Pareto(1.2) x 10 + 1, capped at 10^6",
